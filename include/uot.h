@@ -716,6 +716,10 @@ uot_status uot_warmstart_features(const float* p, const float* q, const float* l
  *   (uot_nhwc_transpose of dy) and xT [3][cin_pad][N][H][W]
  *   (uot_nhwc_shift_transpose of x); Cout <= 128, cin_pad 64 or 128; part is
  *   FP32 scratch of splits x 9 x 128 x cin_pad partial sums.
+ * uot_conv_tc_wgrad_nhwc: the same dw together with db[co] = sum_p g[p][co],
+ *   straight from g [P][ldg] and x [P][ldx] (NHWC, ldg and ldx multiples of 8,
+ *   Cout <= min(ldg, 128), Cin <= min(ldx, 128), W = 64); 1 <= splits <= N H
+ *   row ranges of partial sums, part is FP32 scratch of splits x (9 Cin + 1) x 128.
  * uot_nhwc_shift_transpose: xT[d][c][n][y][x] = x[n][y][x + (d-1) dil][c] (0 off the
  *   image), d = 0, 1, 2; x [N][H][W][C], W <= 64.
  * uot_nhwc_transpose: yT[c][p] = y[p][c], y [P][C].
@@ -735,6 +739,9 @@ uot_status uot_conv_tc_forward(const void* x, int ldx, const void* wk, int bn, i
                                int ldy, float* yf, int* err, void* stream);
 uot_status uot_conv_tc_wgrad(const void* dyT, int cout_rows, const void* xT, int cin_pad, int N, int H, int W,
                              int dil, int Cout, int Cin, float* part, int splits, float* dw, int* err, void* stream);
+uot_status uot_conv_tc_wgrad_nhwc(const void* g, int ldg, const void* x, int ldx, int N, int H, int W, int dil,
+                                  int Cout, int Cin, float* part, int splits, float* dw, float* db, int* err,
+                                  void* stream);
 uot_status uot_nhwc_shift_transpose(const void* x, int N, int H, int W, int C, int dil, void* xT, void* stream);
 uot_status uot_nhwc_transpose(const void* y, long long P, int C, void* yT, void* stream);
 uot_status uot_bias_grad_bf16(const void* dy, long long P, int ld, int C, float* db, void* stream);

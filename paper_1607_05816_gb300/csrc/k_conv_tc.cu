@@ -21,11 +21,12 @@
 //                   derivative of the previous layer's leaky ReLU.
 //  backward (weight) dW[co][tap][ci] = sum_p dy[p][co] x[p + s(tap)][ci]: a GEMM
 //                   with M = 128 output channels, N = input channels, K = pixels,
-//                   both operands K-major (pixels contiguous) from transposed
-//                   copies dyT[co][n][y][x] and xT[dx][ci][n][y][x] (x-shifted by
-//                   dx dil on the copy, so that the TMA's innermost coordinate
-//                   stays 0); the y shift is a TMA coordinate.  Split over image
-//                   rows into partial sums, reduced by a second kernel.
+//                   split over image rows into partial sums reduced by a second
+//                   kernel.  wgrad_nhwc (training) reads the NHWC arrays as
+//                   MN-major operands; wgrad_tc takes them K-major (pixels
+//                   contiguous), from transposed copies dyT[co][n][y][x] and
+//                   xT[dx][ci][n][y][x] (x-shifted by dx dil on the copy, so that
+//                   the TMA's innermost coordinate stays 0).
 //
 // The forward / data-gradient kernel is persistent (one CTA per SM walks its
 // share of the 128-pixel tiles) with warp roles: one thread streams the TMA
@@ -616,6 +617,302 @@ __global__ void __launch_bounds__(128, 1)
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN));
 }
 
+// ---------------------------------------------------------------------------
+// Weight and bias gradient straight from the NHWC arrays,
+//   dW[co][dy][dx][ci] = sum_p g[p][co] x[p + (dy, dx) dil][ci],  db[co] = sum_p g[p][co],
+// a GEMM with M = 128 output channels, N = input channels, K = pixels.  Both
+// operands are MN-major: a TMA box of one image row (64 pixels) x 64 channels
+// with 128-byte swizzle is an operand tile as it lands, so neither array is
+// transposed or copied first (the K-major form needed a transposed g and three
+// shifted transposed copies of x: 76 us of a layer's 144 us at 32 images), and
+// the zero padding is the TMA's fill.
+//
+// A CTA has one dx and a range of image rows, and keeps the three dy of that
+// column in tensor memory (3 x 128 columns).  Rows are walked in chains y, y +
+// dil, y + 2 dil, ...: the x rows of a step's three taps are then three
+// consecutive rows of the chain, so each step loads one new x row and one g row
+// (32 KB for three taps).  What bounds it is that traffic from L2 and the
+// operands' reads from shared memory: two neighbouring taps run as one N = 256
+// MMA where their x rows lie side by side in the ring, which halves the reads
+// of g (an N = 128 MMA takes the SM's whole shared-memory bandwidth).
+// Four warps that wait for the accumulators sum g's columns from the staged
+// tiles meanwhile (the CTAs with dx = 0), which gives db without another pass
+// over g (a pass of its own took 165 us a layer).
+//
+// Measured, 128-channel layer, 32 images of 64 x 64: 40 us + 5 us for the sum
+// of the partials, against 68 + 11 us for wgrad_tc, 45 + 31 us for the copies it
+// needs and 165 us for the bias; the MMAs alone would take 20 us at the chip's
+// BF16 rate, the 201 MB from L2 about as long.  A training step: 5.12 -> 2.27 ms.
+// ---------------------------------------------------------------------------
+constexpr int kWgXSlots = 6, kWgGSlots = 4;  // x rows / g rows in flight: 96 + 64 KB at 128 channels
+constexpr int kWgRow = 64 * 128;             // bytes of 64 pixels x 64 channels
+
+// MN-major tile with 128-byte swizzle: 64 channels (128 bytes) x 64 pixels;
+// the next 64 channels kWgRow bytes on, the next 8 pixels 1024 bytes on.
+__device__ __forceinline__ uint64_t desc_mn_sw128(uint32_t saddr) {
+  uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFF);
+  d |= (uint64_t)(kWgRow >> 4) << 16;
+  d |= (uint64_t)(1024 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)2 << 61;
+  return d;
+}
+__host__ __device__ constexpr uint32_t idesc_bf16_mn(int M, int N) {
+  return idesc_bf16(M, N) | (1u << 15) | (1u << 16);
+}
+
+struct WgradNhwcArgs {
+  int N, H, dil, splits;
+  int Cout, Cin;
+  float* part;   // [splits][9][Cin][128]
+  float* bpart;  // [splits][128]
+  int* err;
+};
+
+// The steps (g rows) of a CTA: image n, chain c, position k; y = c + k dil.
+struct WgStep {
+  int H, dil, n, c, k, left;
+  __device__ WgStep(int H_, int dil_, int first, int count) : H(H_), dil(dil_), left(count) {
+    n = first / H;
+    int r = first - n * H;
+    c = 0;
+    for (int len; r >= (len = (H - 1 - c) / dil + 1); ++c) r -= len;
+    k = r;
+  }
+  __device__ int y() const { return c + k * dil; }
+  __device__ bool has_prev() const { return k > 0; }
+  __device__ bool has_next() const { return y() + dil < H; }
+  // the next step continues this chain (its x rows but the last are loaded)
+  __device__ bool continues() const { return left > 1 && has_next(); }
+  __device__ void advance() {
+    if (has_next()) {
+      ++k;
+    } else {
+      k = 0;
+      if (++c >= min(dil, H)) {
+        c = 0;
+        ++n;
+      }
+    }
+    --left;
+  }
+};
+
+template <int BN>
+__global__ void __launch_bounds__(192, 1)
+    wgrad_nhwc(const __grid_constant__ CUtensorMap tmG, const __grid_constant__ CUtensorMap tmX, WgradNhwcArgs a) {
+  constexpr int kXBytes = BN / 64 * kWgRow, kGBytes = 2 * kWgRow;
+  constexpr int kAllocCols = BN == 128 ? 512 : 256;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* sX = align1024(smem_raw);
+  uint8_t* sG = sX + kWgXSlots * kXBytes;
+  __shared__ __align__(8) uint64_t xfull[kWgXSlots], xempty[kWgXSlots], gfull[kWgGSlots], gempty[kWgGSlots], done;
+  __shared__ float bsum[8][128];
+  __shared__ uint32_t tmem_slot;
+  __shared__ int abort_flag;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int dxi = blockIdx.x, split = blockIdx.y;
+  const int total = a.N * a.H;
+  const int first = (int)((int64_t)total * split / a.splits);
+  const int count = (int)((int64_t)total * (split + 1) / a.splits) - first;  // >= 1 (splits <= total)
+  const bool bias = dxi == 1;
+  if (tid == 0) {
+    for (int s = 0; s < kWgXSlots; ++s) {
+      mbar_init(&xfull[s], 1);
+      mbar_init(&xempty[s], 1);
+    }
+    for (int s = 0; s < kWgGSlots; ++s) {
+      mbar_init(&gfull[s], 1);
+      mbar_init(&gempty[s], bias ? 5 : 1);
+    }
+    mbar_init(&done, 1);
+    abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                 "r"(kAllocCols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  const uint32_t tmem = tmem_slot;
+  volatile int* abort = &abort_flag;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int ix = 0, ig = 0;  // x rows and g rows asked for so far
+      bool ok = true;
+      auto load_x = [&](int y, int n) {
+        const int s = ix % kWgXSlots;
+        if (ix >= kWgXSlots && !mbar_wait(&xempty[s], ((ix / kWgXSlots) - 1) & 1, abort)) return false;
+        mbar_expect_tx(&xfull[s], kXBytes);
+#pragma unroll
+        for (int c = 0; c < BN / 64; ++c)
+          tma_load_4d(sX + s * kXBytes + c * kWgRow, &tmX, &xfull[s], c * 64, (dxi - 1) * a.dil, y, n);
+        ++ix;
+        return true;
+      };
+      bool fresh = true;
+      for (WgStep st(a.H, a.dil, first, count); st.left > 0 && ok; st.advance()) {
+        if (fresh && st.has_prev()) ok = load_x(st.y() - a.dil, st.n);
+        if (fresh && ok) ok = load_x(st.y(), st.n);
+        if (ok && st.has_next()) ok = load_x(st.y() + a.dil, st.n);
+        if (!ok) break;
+        const int s = ig % kWgGSlots;
+        if (ig >= kWgGSlots && !(ok = mbar_wait(&gempty[s], ((ig / kWgGSlots) - 1) & 1, abort))) break;
+        mbar_expect_tx(&gfull[s], kGBytes);
+        tma_load_4d(sG + s * kGBytes, &tmG, &gfull[s], 0, 0, st.y(), st.n);
+        tma_load_4d(sG + s * kGBytes + kWgRow, &tmG, &gfull[s], 64, 0, st.y(), st.n);
+        ++ig;
+        fresh = !st.continues();
+      }
+      if (!ok) {
+        // let the copies in flight land before the CTA's shared memory goes away
+        for (int j = max(0, ix - kWgXSlots); j < ix; ++j) mbar_drain(&xfull[j % kWgXSlots], (j / kWgXSlots) & 1);
+        for (int j = max(0, ig - kWgGSlots); j < ig; ++j) mbar_drain(&gfull[j % kWgGSlots], (j / kWgGSlots) & 1);
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      int ix = 0, ig = 0;  // index of this step's first x row / its g row
+      uint32_t inited = 0;
+      bool ok = true;
+      // D[dy0 .. dy0 + nt) += G^T X for nt neighbouring taps whose x rows start at slot xs
+      auto mma = [&](int dy0, int nt, int xs, uint32_t g0) {
+        const uint32_t x0 = smem_u32(sX + xs * kXBytes), acc = tmem + (uint32_t)(dy0 * BN);
+        const uint32_t idesc = nt == 2 ? idesc_bf16_mn(128, 2 * BN) : idesc_bf16_mn(128, BN);
+        const uint32_t have = (inited >> dy0) & 1u;
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+          mma_bf16(acc, desc_mn_sw128(g0 + kk * 2048), desc_mn_sw128(x0 + kk * 2048), idesc, have | (kk != 0));
+        inited |= ((1u << nt) - 1u) << dy0;
+      };
+      bool fresh = true;
+      for (WgStep st(a.H, a.dil, first, count); st.left > 0 && ok; st.advance()) {
+        const int lo = st.has_prev() ? 0 : 1, hi = st.has_next() ? 2 : 1;  // taps dy of this step
+        // x row of tap dy has index ix + dy - lo; rows before the newest are known to be there
+        for (int dy = fresh ? lo : hi; dy <= hi && ok; ++dy) {
+          const int j = ix + dy - lo;
+          ok = mbar_wait(&xfull[j % kWgXSlots], (j / kWgXSlots) & 1, abort);
+        }
+        const int gs = ig % kWgGSlots;
+        if (ok) ok = mbar_wait(&gfull[gs], (ig / kWgGSlots) & 1, abort);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        const uint32_t g0 = smem_u32(sG + gs * kGBytes);
+        for (int dy = lo; dy <= hi;) {
+          const int xs = (ix + dy - lo) % kWgXSlots;
+          const bool pair = dy < hi && xs + 1 < kWgXSlots && ((inited >> dy) & 1u) == ((inited >> (dy + 1)) & 1u);
+          mma(dy, pair ? 2 : 1, xs, g0);
+          dy += pair ? 2 : 1;
+        }
+        mma_commit(&gempty[gs]);
+        ++ig;
+        if (st.continues()) {
+          if (lo == 0) {
+            mma_commit(&xempty[ix % kWgXSlots]);
+            ++ix;
+          }
+          fresh = false;
+        } else {
+          for (int dy = lo; dy <= hi; ++dy, ++ix) mma_commit(&xempty[ix % kWgXSlots]);
+          fresh = true;
+        }
+      }
+      // all MMAs issued complete before tensor memory is read or freed
+      mma_commit(&done);
+      if (!ok) mbar_drain(&done, 0);
+    }
+  } else {
+    const int t = tid - 64;  // 128 threads
+    if (bias) {
+      // column sums of g: thread = 8 channels (chunk) x every eighth pixel
+      const int chunk = t & 15, pr = t >> 4;
+      float acc[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+      for (int i = 0; i < count; ++i) {
+        const int s = i % kWgGSlots;
+        if (!mbar_wait(&gfull[s], (i / kWgGSlots) & 1, abort)) break;
+        const uint8_t* base = sG + s * kGBytes + (chunk >> 3) * kWgRow;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          const int px = pr + 8 * r;  // swizzle: 16-byte chunk index XOR (row mod 8)
+          const uint4 v = *reinterpret_cast<const uint4*>(base + px * 128 + (((chunk & 7) ^ (px & 7)) << 4));
+          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            acc[2 * q] += __uint_as_float(w[q] << 16);
+            acc[2 * q + 1] += __uint_as_float(w[q] & 0xffff0000u);
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&gempty[s]);
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) bsum[pr][chunk * 8 + q] = acc[q];
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      float s = 0.0f;
+#pragma unroll
+      for (int r = 0; r < 8; ++r) s += bsum[r][t];
+      if (!*abort) a.bpart[split * 128 + t] = s;
+    }
+    // accumulators: taps that no step of this CTA touched are zero
+    uint32_t touched = 2u;
+    for (WgStep st(a.H, a.dil, first, count); st.left > 0; st.advance())
+      touched |= (st.has_prev() ? 1u : 0u) | (st.has_next() ? 4u : 0u);
+    bool ok = mbar_wait(&done, 0, abort);
+    ok = __all_sync(0xffffffffu, ok ? 1 : 0) && !*abort;
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const int q = warp & 3, co = q * 32 + lane;
+    if (ok) {
+      for (int dy = 0; dy < 3; ++dy) {
+        float* dst = a.part + ((int64_t)(split * 9 + dy * 3 + dxi) * a.Cin) * 128 + co;
+        for (int cb = 0; cb < a.Cin; cb += 16) {
+          float v[16];
+          if ((touched >> dy) & 1u) {
+            tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(dy * BN + cb), v);
+          } else {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) v[k] = 0.0f;
+          }
+#pragma unroll
+          for (int k = 0; k < 16; ++k)
+            if (cb + k < a.Cin) dst[(int64_t)(cb + k) * 128] = v[k];
+        }
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  if (tid == 0 && *abort && a.err) atomicExch(a.err, 1);
+  if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kAllocCols));
+}
+
+// dW[co][ci][3][3] and db[co] from the partial sums, splits added in order.
+// Lanes run over co (the partials' contiguous index).
+__global__ void __launch_bounds__(128) k_wgrad_nhwc_reduce(const float* __restrict__ part,
+                                                            const float* __restrict__ bpart, int splits, int Cout,
+                                                            int Cin, float* __restrict__ dw, float* __restrict__ db) {
+  const int co = threadIdx.x, row = blockIdx.x;  // row = tap * Cin + ci, the last one the bias
+  if (co >= Cout) return;
+  const bool is_b = row == 9 * Cin;
+  const float* src = is_b ? bpart + co : part + (int64_t)row * 128 + co;
+  const int64_t step = is_b ? 128 : (int64_t)9 * Cin * 128;
+  float s = 0.0f;
+  int k = 0;
+  for (; k + 8 <= splits; k += 8) {
+    float v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = src[(k + u) * step];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s += v[u];
+  }
+  for (; k < splits; ++k) s += src[k * step];
+  if (is_b) db[co] = s;
+  else dw[((int64_t)co * Cin + row % Cin) * 9 + row / Cin] = s;
+}
+
 // ---- layout helpers ----
 
 // xT[d][c][n][y][x] = x[n][y][x + (d - 1) dil][c] (0 outside the image), d = 0, 1, 2.
@@ -856,6 +1153,45 @@ cudaError_t launch_wgrad_tc(const void* dyT, int cout_rows, const void* xT, int 
   return cudaGetLastError();
 }
 
+// g [N][H][64][ldg] (channels beyond ldg read as zero), x [N][H][64][ldx];
+// part: splits * (9 * Cin + 1) * 128 floats.
+cudaError_t launch_wgrad_nhwc(const void* g, int ldg, const void* x, int ldx, int N, int H, int W, int dil, int Cout,
+                              int Cin, float* part, int splits, float* dw, float* db, int* err, cudaStream_t s) {
+  if (W != 64 || ldg % 8 || ldx % 8 || Cout > ldg || Cin > ldx || Cout > 128 || Cin > 128 || splits < 1 ||
+      splits > 65535 || (int64_t)N * H > INT32_MAX || splits > N * H)
+    return cudaErrorInvalidValue;
+  CUtensorMap mg, mx;
+  const uint64_t dg[4] = {(uint64_t)ldg, (uint64_t)W, (uint64_t)H, (uint64_t)N};
+  const uint64_t dx[4] = {(uint64_t)ldx, (uint64_t)W, (uint64_t)H, (uint64_t)N};
+  const uint32_t box[4] = {64, 64, 1, 1};
+  if (!make_map(&mg, g, 4, dg, box) || !make_map(&mx, x, 4, dx, box)) return cudaErrorInvalidValue;
+  WgradNhwcArgs a;
+  a.N = N;
+  a.H = H;
+  a.dil = dil;
+  a.splits = splits;
+  a.Cout = Cout;
+  a.Cin = Cin;
+  a.part = part;
+  a.bpart = part + (size_t)splits * 9 * Cin * 128;
+  a.err = err;
+  const bool wide = Cin > 64;
+  const size_t smem = 1024 + (size_t)kWgXSlots * (wide ? 2 : 1) * kWgRow + (size_t)kWgGSlots * 2 * kWgRow;
+  const dim3 grid(3, splits);
+  cudaError_t e;
+  count_launches(2);
+  if (wide) {
+    if ((e = smem_at_least(wgrad_nhwc<128>, smem))) return e;
+    wgrad_nhwc<128><<<grid, 192, smem, s>>>(mg, mx, a);
+  } else {
+    if ((e = smem_at_least(wgrad_nhwc<64>, smem))) return e;
+    wgrad_nhwc<64><<<grid, 192, smem, s>>>(mg, mx, a);
+  }
+  if ((e = cudaGetLastError())) return e;
+  k_wgrad_nhwc_reduce<<<9 * Cin + 1, 128, 0, s>>>(part, a.bpart, splits, Cout, Cin, dw, db);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_nhwc_to_shifted_cnhw(const void* x, int N, int H, int W, int C, int dil, void* xT,
                                         cudaStream_t s) {
   if (W > 64) return cudaErrorInvalidValue;
@@ -995,6 +1331,15 @@ uot_status uot_conv_tc_wgrad(const void* dyT, int cout_rows, const void* xT, int
   if (!conv_tc_available()) return UOT_EUNSUPPORTED;
   return ck(launch_wgrad_tc(dyT, cout_rows, xT, cin_pad, N, H, W, dil, Cout, Cin, part, splits, dw, err,
                             (cudaStream_t)stream));
+}
+
+uot_status uot_conv_tc_wgrad_nhwc(const void* g, int ldg, const void* x, int ldx, int N, int H, int W, int dil,
+                                  int Cout, int Cin, float* part, int splits, float* dw, float* db, int* err,
+                                  void* stream) {
+  if (!g || !x || !part || !dw || !db || N < 1 || H < 1 || dil < 1 || Cout < 1 || Cin < 1) return UOT_EINVAL;
+  if (!conv_tc_available()) return UOT_EUNSUPPORTED;
+  return ck(launch_wgrad_nhwc(g, ldg, x, ldx, N, H, W, dil, Cout, Cin, part, splits, dw, db, err,
+                              (cudaStream_t)stream));
 }
 
 uot_status uot_nhwc_shift_transpose(const void* x, int N, int H, int W, int C, int dil, void* xT, void* stream) {

@@ -531,6 +531,9 @@ int conv_tc_available();
 cudaError_t launch_conv_tc(const void* x, const void* wk, int bn, const ConvTcLaunch& L, cudaStream_t s);
 cudaError_t launch_wgrad_tc(const void* dyT, int cout_rows, const void* xT, int cin_pad, int N, int H, int W, int dil,
                             int Cout, int Cin, float* part, int splits, float* dw, int* err, cudaStream_t s);
+// weight and bias gradient from the NHWC arrays (no transposed copies)
+cudaError_t launch_wgrad_nhwc(const void* g, int ldg, const void* x, int ldx, int N, int H, int W, int dil, int Cout,
+                              int Cin, float* part, int splits, float* dw, float* db, int* err, cudaStream_t s);
 cudaError_t launch_nhwc_to_shifted_cnhw(const void* x, int N, int H, int W, int C, int dil, void* xT,
                                         cudaStream_t s);
 cudaError_t launch_nhwc_to_cnhw(const void* y, int64_t P, int C, void* yT, cudaStream_t s);

@@ -129,6 +129,9 @@ _SIGS = {
                                       C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p]),
     "uot_conv_tc_wgrad": (C.c_int, [C.c_void_p, C.c_int, C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int,
                                     C.c_int, C.c_int, C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p]),
+    "uot_conv_tc_wgrad_nhwc": (C.c_int, [C.c_void_p, C.c_int, C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int,
+                                         C.c_int, C.c_int, C.c_int, C.c_void_p, C.c_int, C.c_void_p, C.c_void_p,
+                                         C.c_void_p, C.c_void_p]),
     "uot_nhwc_shift_transpose": (C.c_int, [C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_void_p,
                                            C.c_void_p]),
     "uot_nhwc_transpose": (C.c_int, [C.c_void_p, C.c_longlong, C.c_int, C.c_void_p, C.c_void_p]),
@@ -823,6 +826,24 @@ def conv_tc_wgrad(dyT, xT, cin_pad, N, H, W, dil, Cout, Cin, *, splits=64, part=
                                     _ptr(dw, torch.float32, "dw"), _ptr(err, torch.int32, "err"), _stream()),
            "uot_conv_tc_wgrad")
     return dw
+
+
+def conv_tc_wgrad_nhwc(g, x, N, H, W, dil, Cout, Cin, *, splits=50, part=None, dw=None, db=None, err=None):
+    """uot_conv_tc_wgrad_nhwc; g [P, ldg], x [P, ldx] BF16 -> (dw [Cout, Cin, 3, 3], db [Cout]) FP32.  Three
+    CTAs per split: 50 splits fill 150 of the 152 SMs with one CTA each."""
+    f, dev = torch.float32, g.device
+    splits = max(1, min(splits, N * H))
+    dw = torch.empty(Cout, Cin, 3, 3, dtype=f, device=dev) if dw is None else dw
+    db = torch.empty(Cout, dtype=f, device=dev) if db is None else db
+    need = splits * (9 * Cin + 1) * 128
+    part = torch.empty(need, dtype=f, device=dev) if part is None else part
+    if part.numel() < need:
+        raise ValueError(f"part must hold {need} floats")
+    _check(load().uot_conv_tc_wgrad_nhwc(_ptr(g, BF16, "g"), g.shape[-1], _ptr(x, BF16, "x"), x.shape[-1], N, H, W,
+                                         dil, Cout, Cin, _ptr(part, f, "part"), splits, _ptr(dw, f, "dw"),
+                                         _ptr(db, f, "db"), _ptr(err, torch.int32, "err"), _stream()),
+           "uot_conv_tc_wgrad_nhwc")
+    return dw, db
 
 
 def nhwc_shift_transpose(x, N, H, W, dil, out=None):

@@ -258,13 +258,10 @@ class WarmStartNetTC:
             cin, cout, dil, _ = self.layers[li]
             cin_pad, bn, cout_kpad = self._pads(li)
             x = acts[li]
-            xT = uot.nhwc_shift_transpose(x, N, H, W, dil, out=self._buf("xT", (3, x.shape[1], P), torch.bfloat16))
-            gT = uot.nhwc_transpose(g, out=self._buf(("gT", g.shape[1]), (g.shape[1], P), torch.bfloat16))
-            splits = max(1, min(N * H, 64))
-            dw = uot.conv_tc_wgrad(gT, xT, cin_pad, N, H, W, dil, cout, cin, splits=splits,
-                                   part=self._buf(("part", cin_pad), (splits * 9 * 128 * cin_pad,), torch.float32),
-                                   dw=self._buf(("dw", li), (cout, cin, 3, 3), torch.float32), err=self.err)
-            db = uot.bias_grad_bf16(g, cout, out=self._buf(("db", li), (cout,), torch.float32))
+            dw, db = uot.conv_tc_wgrad_nhwc(g, x, N, H, W, dil, cout, cin,
+                                            part=self._buf(("part", cin), (50 * (9 * cin + 1) * 128,), torch.float32),
+                                            dw=self._buf(("dw", li), (cout, cin, 3, 3), torch.float32),
+                                            db=self._buf(("db", li), (cout,), torch.float32), err=self.err)
             grads[li] = (dw, db)
             if li > 0:
                 gin = self._buf(("g", li % 2), (P, cin), torch.bfloat16)
