@@ -9,14 +9,8 @@
 // (point index i*nlines + l), so that d successive passes over the last axis
 // cycle a row-major d-dimensional array back to row-major order.
 //
-// Work per pass: nlines * nout * nin exponentials.  The pass is bound by the
-// SFU (MUFU.EX2) throughput in FP32 and by FP64 arithmetic in FP64.
-//
-// Layout: each warp owns one line and 32*R consecutive outputs (one per lane
-// and register slot).  The warp stages its line in shared memory as
-// {log2-scaled value, coordinate} pairs, shifted by the line's FP64 maximum, so
-// every shared load is a broadcast; each lane then runs a max sweep and a
-// sum-of-exponentials sweep over the line for its R outputs.
+// This file holds the FP32 passes, nlines * nout * nin exponentials each, bound
+// by the FP32 pipe; the FP64 pass is in k_grid_fac.cu.
 #include <string.h>
 
 #include <algorithm>
@@ -29,21 +23,6 @@
 
 namespace uot {
 namespace {
-
-
-__device__ __forceinline__ double warp_max(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-
-__device__ __forceinline__ double load_L(const double* __restrict__ in,
-                                         const double* __restrict__ logw, int in_is_pot,
-                                         int64_t idx, double inv_eps) {
-  const double v = in[idx];
-  if (!in_is_pot) return v;
-  return (v == -kInf) ? -kInf : v * inv_eps + logw[idx];
-}
 
 // FP32 grid pass.  One CTA = one line x (32 * OPL) consecutive outputs; its NW
 // warps split the contraction index j into NW contiguous ranges and combine
@@ -556,120 +535,6 @@ cudaError_t launch_grid_solve_persistent(const PersistLaunch& L, int grid, cudaS
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
-
-namespace {
-
-// FP64 arithmetic throughout.  With zprev holding this pass's results from the
-// previous call at the same eps (use_prev), each output takes that value as
-// its log-sum-exp shift and the pass costs one sweep; an output whose sum
-// leaves [1e-290, 1e290] (a shift too far from the new maximum) is redone with
-// its exact maximum (a max sweep and a sum sweep).  The result does not depend
-// on the shift beyond rounding.
-template <int R, int WARPS>
-__global__ void __launch_bounds__(WARPS * 32)
-    grid_pass_f64(const double* __restrict__ in, const double* __restrict__ logw, int in_is_pot,
-                  int nlines, int nin, const double* __restrict__ yi, int nout,
-                  const double* __restrict__ xo, double eps, Epilogue epi, float* zprev, int use_prev) {
-  extern __shared__ double2 sm_d2[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int l = blockIdx.y * WARPS + warp;
-  const int i0 = blockIdx.x * (32 * R);
-  const int64_t bz = blockIdx.z;
-  in += bz * (int64_t)nlines * nin;
-  const double inv_eps = 1.0 / eps;
-  double num = 0.0, den = 0.0;
-  if (l < nlines) {
-    double2* line = sm_d2 + (size_t)warp * nin;
-    const int64_t base = (int64_t)l * nin;
-    double mx = -kInf;
-    for (int j = lane; j < nin; j += 32) {
-      const double v = load_L(in, logw, in_is_pot, base + j, inv_eps);
-      line[j] = make_double2(v, yi[j]);
-      mx = fmax(mx, v);
-    }
-    mx = warp_max(mx);
-    __syncwarp();
-    if (mx == -kInf) {
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const int i = i0 + lane + 32 * r;
-        if (i < nout) {
-          double a, b;
-          apply_epilogue(epi, bz, (int64_t)i * nlines + l, -kInf, a, b);
-          num += a;
-          den += b;
-        }
-      }
-    } else {
-      float* zp = zprev ? zprev + bz * (int64_t)nout * nlines : nullptr;
-      double xr[R], m[R], s[R];
-      bool spec = use_prev && zp;
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const int i = i0 + lane + 32 * r;
-        xr[r] = xo[i < nout ? i : nout - 1];
-        m[r] = -kInf;
-        s[r] = 0.0;
-        if (spec) {
-          m[r] = (i < nout) ? (double)zp[(int64_t)i * nlines + l] : 0.0;
-          if (!(m[r] > -kInf)) spec = false;  // no usable shift for this lane
-        }
-      }
-      bool exact = !spec;
-      if (spec) {
-        for (int j = 0; j < nin; ++j) {
-          const double2 t = line[j];
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            const double dd = xr[r] - t.y;
-            s[r] += exp((t.x - m[r]) - dd * dd * inv_eps);
-          }
-        }
-#pragma unroll
-        for (int r = 0; r < R; ++r) exact = exact || !(s[r] >= 1e-290 && s[r] <= 1e290);
-      }
-      if (exact) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          m[r] = -kInf;
-          s[r] = 0.0;
-        }
-        for (int j = 0; j < nin; ++j) {
-          const double2 t = line[j];
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            const double dd = xr[r] - t.y;
-            m[r] = fmax(m[r], t.x - dd * dd * inv_eps);
-          }
-        }
-        for (int j = 0; j < nin; ++j) {
-          const double2 t = line[j];
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            const double dd = xr[r] - t.y;
-            s[r] += exp((t.x - m[r]) - dd * dd * inv_eps);
-          }
-        }
-      }
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const int i = i0 + lane + 32 * r;
-        if (i < nout) {
-          const double z = m[r] + log(s[r]);
-          if (zp) zp[(int64_t)i * nlines + l] = (float)z;
-          double a, b;
-          apply_epilogue(epi, bz, (int64_t)i * nlines + l, z, a, b);
-          num += a;
-          den += b;
-        }
-      }
-    }
-  }
-  if (epi.err) block_add2<WARPS * 32>(num, den, epi.err + 2 * bz);
-}
-
-}  // namespace
-
 
 // ---------------------------------------------------------------------------
 // FP32 pass with float-float exponents ("precise pass").  The log-sum-exp
@@ -1573,62 +1438,44 @@ cudaError_t launch_grid_pass_plane(const double* in, const double* logw, int in_
   return cudaGetLastError();
 }
 
-cudaError_t launch_grid_pass(int prec, const double* in, const double* logw, int in_is_pot,
+cudaError_t launch_grid_pass(const double* in, const double* logw, int in_is_pot,
                              int nlines, int nin, const void* yi, int nout, const void* xo,
                              double eps, int nbatch, const Epilogue& epi, cudaStream_t s,
                              float* zprev, int use_prev, double* zero_acc, int tc3_ok, int* tc_err,
                              const BlkAxis* blk, int precise) {
-  if (prec == UOT_F32) {
-    PassArgs a;
-    a.in = reinterpret_cast<const float2*>(in);
-    a.logw = reinterpret_cast<const float2*>(logw);
-    a.in_is_pot = in_is_pot;
-    a.nlines = nlines;
-    a.nin = nin;
-    a.nout = nout;
-    a.yi = (const float*)yi;
-    a.xo = (const float*)xo;
-    a.inv_eps = ff2(ff_make(1.0 / eps));
-    a.k2 = (float)((double)kLog2e / eps);
-    a.zprev = zprev;
-    a.use_prev = use_prev;
-    a.zero_acc = zero_acc;
-    a.tc3_ok = (tc3_ok && nin <= grid_pass_tc3_max_nin()) ? 1 : 0;
-    a.tc_err = tc_err;
-    a.nbatch = nbatch;
-    a.blk = blk ? *blk : BlkAxis{0, 0.0f, 0.0f};
-    if (precise || g_precise_forced.load()) {
-      prof_mark_begin(PROF_GRID_PASS, s);
-      count_launches(1);
-      cudaError_t e = launch_ffp(a, epi, nbatch, s);
-      if (e != cudaSuccess) return e;
-      prof_mark_end(PROF_GRID_PASS, s);
-      return cudaGetLastError();
-    }
-    const int tile = pick_tile(a, nbatch, s);
-    const int fam = (is_blk(tile) && grid_blk_ok(a, tile - kBlkTile0)) ? PROF_GRID_BLK : PROF_GRID_PASS;
-    prof_mark_begin(fam, s);
+  PassArgs a;
+  a.in = reinterpret_cast<const float2*>(in);
+  a.logw = reinterpret_cast<const float2*>(logw);
+  a.in_is_pot = in_is_pot;
+  a.nlines = nlines;
+  a.nin = nin;
+  a.nout = nout;
+  a.yi = (const float*)yi;
+  a.xo = (const float*)xo;
+  a.inv_eps = ff2(ff_make(1.0 / eps));
+  a.k2 = (float)((double)kLog2e / eps);
+  a.zprev = zprev;
+  a.use_prev = use_prev;
+  a.zero_acc = zero_acc;
+  a.tc3_ok = (tc3_ok && nin <= grid_pass_tc3_max_nin()) ? 1 : 0;
+  a.tc_err = tc_err;
+  a.nbatch = nbatch;
+  a.blk = blk ? *blk : BlkAxis{0, 0.0f, 0.0f};
+  if (precise || g_precise_forced.load()) {
+    prof_mark_begin(PROF_GRID_PASS, s);
     count_launches(1);
-    cudaError_t e = launch_f32(tile, a, epi, nbatch, s);
+    cudaError_t e = launch_ffp(a, epi, nbatch, s);
     if (e != cudaSuccess) return e;
-    prof_mark_end(fam, s);
+    prof_mark_end(PROF_GRID_PASS, s);
     return cudaGetLastError();
   }
-  prof_mark_begin(PROF_GRID_PASS, s);
+  const int tile = pick_tile(a, nbatch, s);
+  const int fam = (is_blk(tile) && grid_blk_ok(a, tile - kBlkTile0)) ? PROF_GRID_BLK : PROF_GRID_PASS;
+  prof_mark_begin(fam, s);
   count_launches(1);
-  {
-    constexpr int R = 2, WARPS = 4;
-    dim3 grid((nout + 32 * R - 1) / (32 * R), (nlines + WARPS - 1) / WARPS, nbatch);
-    if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidConfiguration;
-    const size_t smem = (size_t)WARPS * nin * sizeof(double2);
-    if (smem > 48 * 1024) {
-      cudaError_t e = smem_at_least(grid_pass_f64<R, WARPS>, smem);
-      if (e != cudaSuccess) return e;
-    }
-    grid_pass_f64<R, WARPS><<<grid, WARPS * 32, smem, s>>>(
-        in, logw, in_is_pot, nlines, nin, (const double*)yi, nout, (const double*)xo, eps, epi, zprev, use_prev);
-  }
-  prof_mark_end(PROF_GRID_PASS, s);
+  cudaError_t e = launch_f32(tile, a, epi, nbatch, s);
+  if (e != cudaSuccess) return e;
+  prof_mark_end(fam, s);
   return cudaGetLastError();
 }
 

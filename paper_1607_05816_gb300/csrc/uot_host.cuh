@@ -764,6 +764,11 @@ struct Gibbs {
   const void* CT = nullptr;     // dense: C^T in the precision's type
   float* C32[2] = {nullptr, nullptr};  // dense FP64: FP32 copies of C, C^T (row prefilter)
   double* pass[2] = {nullptr, nullptr};  // grid intermediates
+  // FP64 grids: the stored kernel of each (direction, axis) pass and the eps it
+  // was built for (k_grid_fac.cu); NULL: that pass runs plain log-sum-exps
+  double* fac[2][UOT_MAX_DIM] = {};
+  FacTile* fac_tiles[2][UOT_MAX_DIM] = {};
+  double fac_eps[2][UOT_MAX_DIM] = {{-1.0, -1.0, -1.0}, {-1.0, -1.0, -1.0}};
   // FP32 grid passes: result of each (direction, pass) from the previous call,
   // reused as the log-sum-exp shift while eps is unchanged (see k_grid.cu)
   float* zbuf[2][UOT_MAX_DIM] = {{nullptr, nullptr, nullptr}, {nullptr, nullptr, nullptr}};
@@ -808,6 +813,12 @@ struct Gibbs {
       if (speculate)
         for (int k = 0; k < 2 * g.ndim; ++k) sc.reserve<float>((size_t)inter * nbatch);
       if (prec == UOT_MIXED || prec == UOT_F32) sc.reserve<int>(1);
+      for (int dir = 0; dir < 2; ++dir)
+        for (int ax = 0; ax < g.ndim; ++ax)
+          if (fac_wanted(dir, ax)) {
+            sc.reserve<double>(fac64_elems(axis_len(dir, ax, true), axis_len(dir, ax, false)));
+            sc.reserve<FacTile>((axis_len(dir, ax, false) + kFacTile - 1) / kFacTile);
+          }
     } else {
       const int64_t mx = (g.n > g.m ? g.n : g.m);
       sc.reserve<char>(lscratch_bytes(mx));
@@ -819,6 +830,20 @@ struct Gibbs {
         }
       }
     }
+  }
+  int axis_len(int dir, int ax, bool input) const {
+    return (dir == 0) == input ? g.shape_y[ax] : g.shape_x[ax];
+  }
+  int64_t pass_lines(int dir, int ax) const {
+    int64_t nl = 1;
+    for (int t = 0; t < ax; ++t) nl *= axis_len(dir, t, true);
+    for (int t = ax + 1; t < g.ndim; ++t) nl *= axis_len(dir, t, false);
+    return nl;
+  }
+  // A stored kernel costs nin nout exponentials to build, a plain pass nlines
+  // times that: it pays from a few lines on, and in any solve (one build per eps).
+  bool fac_wanted(int dir, int ax) const {
+    return prec == UOT_F64 && host_setup && (speculate || pass_lines(dir, ax) * nbatch >= 8);
   }
   bool points_fast() const {
     return g.kind == UOT_GEOM_POINTS && prec != UOT_F64 && g.d <= 3 && points_chunks_fit(g.n) &&
@@ -881,6 +906,13 @@ struct Gibbs {
       if (speculate)
         for (int d = 0; d < 2; ++d)
           for (int k = 0; k < g.ndim; ++k) zbuf[d][k] = sc.take<float>((size_t)inter * nbatch);
+      for (int dir = 0; dir < 2; ++dir)
+        for (int ax = 0; ax < g.ndim; ++ax)
+          if (fac_wanted(dir, ax)) {
+            fac[dir][ax] = sc.take<double>(fac64_elems(axis_len(dir, ax, true), axis_len(dir, ax, false)));
+            fac_tiles[dir][ax] = sc.take<FacTile>((axis_len(dir, ax, false) + kFacTile - 1) / kFacTile);
+            if (!fac[dir][ax] || !fac_tiles[dir][ax]) return cudaErrorInvalidValue;
+          }
       if (prec == UOT_MIXED || prec == UOT_F32) {
         tc_err = sc.take<int>(1);
         if (!tc_err) return cudaErrorInvalidValue;
@@ -1054,9 +1086,21 @@ struct Gibbs {
         if (prec == UOT_MIXED && !tc_off && tc_ok(dir, ax, eps, in_shape[ax])) {
           err = launch_grid_pass_tc(cur, logw, cur_is_pot, (int)nlines, in_shape[ax], in_axes[ax],
                                     out_shape[ax], out_axes[ax], eps, nbatch, e, s, tc_err, za);
+        } else if (prec == UOT_F64) {
+          const double* yi = (const double*)in_axes[ax];
+          const double* xo = (const double*)out_axes[ax];
+          if (fac[dir][ax] && fac_eps[dir][ax] != eps) {
+            err = launch_fac64_build(xo, out_shape[ax], yi, in_shape[ax], eps, fac[dir][ax], fac_tiles[dir][ax], s);
+            if (err != cudaSuccess) return err;
+            fac_eps[dir][ax] = eps;
+          }
+          prof_mark_begin(PROF_GRID_PASS, s);
+          count_launches(1);
+          err = launch_grid_pass_f64(cur, logw, cur_is_pot, (int)nlines, in_shape[ax], yi, out_shape[ax], xo, eps,
+                                     nbatch, e, fac[dir][ax], fac_tiles[dir][ax], zbuf[dir][k], use_prev, s);
+          prof_mark_end(PROF_GRID_PASS, s);
         } else {
-          err = launch_grid_pass(prec == UOT_F64 ? UOT_F64 : UOT_F32, cur, logw, cur_is_pot,
-                                 (int)nlines, in_shape[ax], in_axes[ax], out_shape[ax],
+          err = launch_grid_pass(cur, logw, cur_is_pot, (int)nlines, in_shape[ax], in_axes[ax], out_shape[ax],
                                  out_axes[ax], eps, nbatch, e, s, zbuf[dir][k], use_prev, za,
                                  tc3_ok(dir, ax, eps, in_shape[ax]), tc_err, &blk[dir][ax], precise ? 1 : 0);
         }
@@ -1193,6 +1237,7 @@ Epilogue prox_epilogue(const DivParams& F, const double* logp, double* pot, cons
   set_eps(e, eps);
   e.Fff = make_div_ff(F, eps);
   e.F = F;
+  e.klz = F.lam / (F.lam + eps);
   e.logp = logp;
   e.pot = pot;
   e.logw = logw;

@@ -223,6 +223,7 @@ struct Epilogue {
   DivFF Fff;
   // EPI_PROX
   DivParams F;
+  double klz;              // lam / (lam + eps) of a KL row (its division, once per launch)
   const double* logp;      // log density of the output side
   double* pot;             // potential written (read first as the old value)
   const double* logw;      // log reference weight of the output side (violation)
@@ -268,7 +269,12 @@ __device__ inline void apply_epilogue(const Epilogue& e, int64_t b, int64_t pt, 
       double S = (z == -kInf) ? -kInf : e.eps * z;
       if (e.zshift) S = (S == -kInf || *e.zshift == -kInf) ? -kInf : S + *e.zshift;
       const double Uold = e.pot[q];
-      const double Unew = prox_update(e.F, e.logp[b * e.bstride_p + pt], S, e.eps);
+      const double lp = e.logp[b * e.bstride_p + pt];
+      double Unew;
+      if (e.F.kind == UOT_DIV_KL)
+        Unew = (S == -kInf || lp == -kInf) ? -kInf : e.klz * (e.eps * lp - S);
+      else
+        Unew = prox_update(e.F, lp, S, e.eps);
       e.pot[q] = Unew;
       if (e.err) violation_terms(Uold, Unew, S, e.logw[pt], e.eps, num, den);
       break;
@@ -499,11 +505,28 @@ cudaError_t launch_grid_pass_plane(const double* in, const double* logw, int in_
                                    int nin2, const void* yi2, int nout2, const void* xo2, float* zprev2,
                                    double eps, int nbatch, int use_prev, double* zero_acc, const Epilogue& epi,
                                    cudaStream_t s);
-cudaError_t launch_grid_pass(int prec, const double* in, const double* logw, int in_is_pot,
+cudaError_t launch_grid_pass(const double* in, const double* logw, int in_is_pot,
                              int nlines, int nin, const void* yi, int nout, const void* xo,
                              double eps, int nbatch, const Epilogue& epi, cudaStream_t s,
                              float* zprev, int use_prev, double* zero_acc = nullptr, int tc3_ok = 0,
                              int* tc_err = nullptr, const BlkAxis* blk = nullptr, int precise = 0);
+// FP64 passes (k_grid_fac.cu).  G [nin][64 x tiles] and tiles [ceil(nout / 64)]
+// hold the stored kernel of one axis at one eps (launch_fac64_build; G NULL:
+// plain log-sum-exps, with zprev / use_prev as above).
+constexpr int kFacTile = 64, kFacMaxSub = 16;
+struct FacTile {
+  int sub;      // blocks of 64 / sub outputs with a centre of their own; 0: plain log-sum-exp
+  double c[kFacMaxSub];
+};
+inline size_t fac64_elems(int nin, int nout) {
+  return (size_t)nin * ((nout + kFacTile - 1) / kFacTile) * kFacTile;
+}
+cudaError_t launch_fac64_build(const double* xo, int nout, const double* yi, int nin, double eps, double* G,
+                               FacTile* tiles, cudaStream_t s);
+cudaError_t launch_grid_pass_f64(const double* in, const double* logw, int in_is_pot, int nlines, int nin,
+                                 const double* yi, int nout, const double* xo, double eps, int nbatch,
+                                 const Epilogue& epi, const double* G, const FacTile* tiles, float* zprev,
+                                 int use_prev, cudaStream_t s);
 // precise = 1 (FP32): the pass with float-float exponents (k_grid.cu,
 // grid_pass_ffp), as every FP32 pass runs while grid_force_precise(1) is set;
 // returns the previous setting

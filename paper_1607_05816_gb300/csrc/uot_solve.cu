@@ -279,7 +279,7 @@ uot_status solve_impl(const uot_geom* g, int batch, const void* p, const void* d
       r.out = G.pass[0];
       r.bstride = (int64_t)H2 * W1;
       const int u = use(0, e);
-      return launch_grid_pass(UOT_F32, V, logdy, 1, H2, W2, ya1, W1, xa1, e, 1, r, st, z[0], u);
+      return launch_grid_pass(V, logdy, 1, H2, W2, ya1, W1, xa1, e, 1, r, st, z[0], u);
     };
     auto fused_args = [&](double e) {
       FusedArgs f;
