@@ -280,21 +280,64 @@ __global__ void __launch_bounds__(kTile * TL * KS) grid_pass_f64(Fac64Args a, Ep
   if (epi.err) block_add2<NT>(num, den, epi.err + 2 * bz);
 }
 
-template <int TL, int KS>
-cudaError_t launch_pass(const Fac64Args& a, const Epilogue& epi, int nbatch, cudaStream_t s) {
-  const dim3 grid((a.nout + kTile - 1) / kTile, (a.nlines + TL - 1) / TL, nbatch);
-  if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidConfiguration;
+// A few outputs without a stored kernel (the operator on one short line): one
+// warp per output, lanes over the inputs, so that the exponentials of a single
+// line spread over the chip; a tile of 64 outputs per CTA leaves them to a few
+// SMs' FP64 pipes (1 x 256 points: 126 us a call against 30).
+__global__ void __launch_bounds__(128) grid_pass_f64_few(Fac64Args a, Epilogue epi) {
+  const int lane = threadIdx.x & 31;
+  const int64_t w = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+  const int64_t per = (int64_t)a.nlines * a.nout;
+  const int64_t bz = blockIdx.y;
+  double num = 0.0, den = 0.0;
+  pdl_wait();
+  pdl_launch_dependents();
+  if (w < per) {
+    const int l = (int)(w % a.nlines), i = (int)(w / a.nlines);
+    const double* in = a.in + (bz * a.nlines + l) * (int64_t)a.nin;
+    const double* lw = a.logw + (int64_t)l * a.nin;
+    const double x = a.xo[i];
+    auto expo = [&](int j) {
+      double v = in[j];
+      if (a.in_is_pot) v = (v == -kInf) ? -kInf : v * a.inv_eps + lw[j];
+      const double d = x - a.yi[j];
+      return v - d * d * a.inv_eps;
+    };
+    double m = -kInf, s = 0.0;
+    for (int j = lane; j < a.nin; j += 32) m = fmax(m, expo(j));
+    m = wmax_d(m);
+    double z = -kInf;
+    if (m != -kInf) {
+      for (int j = lane; j < a.nin; j += 32) s += exp(expo(j) - m);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      z = m + log(s);
+    }
+    if (lane == 0) apply_epilogue(epi, bz, w, z, num, den);
+  }
+  if (epi.err) block_add2<128>(num, den, epi.err + 2 * bz);
+}
+
+template <typename K>
+cudaError_t launch_pdl(K kern, dim3 grid, int threads, const Fac64Args& a, const Epilogue& epi, cudaStream_t s) {
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof(cfg));
   cfg.gridDim = grid;
-  cfg.blockDim = dim3(kTile * TL * KS);
+  cfg.blockDim = dim3(threads);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, grid_pass_f64<TL, KS>, a, epi);
+  return cudaLaunchKernelEx(&cfg, kern, a, epi);
+}
+
+template <int TL, int KS>
+cudaError_t launch_pass(const Fac64Args& a, const Epilogue& epi, int nbatch, cudaStream_t s) {
+  const dim3 grid((a.nout + kTile - 1) / kTile, (a.nlines + TL - 1) / TL, nbatch);
+  if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidConfiguration;
+  return launch_pdl(grid_pass_f64<TL, KS>, grid, kTile * TL * KS, a, epi, s);
 }
 
 }  // namespace
@@ -325,13 +368,13 @@ cudaError_t launch_grid_pass_f64(const double* in, const double* logw, int in_is
   a.tiles = tiles;
   a.zprev = zprev;
   a.use_prev = use_prev;
-  const int64_t items = (int64_t)nlines * nbatch * ((nout + kTile - 1) / kTile);
+  const int64_t outs = (int64_t)nlines * nout;
+  if (!G && outs * nbatch <= 152 * 64 && nbatch <= 65535)
+    return launch_pdl(grid_pass_f64_few, dim3((unsigned)((outs + 3) / 4), nbatch), 128, a, epi, s);
   // Four slices of the inputs per output: 256 x 256, 51 us a pass (one slice 49,
   // eight 66); 300 x 300, 88 (one slice 128: the short last chunk's exponentials
-  // are not hidden); 64 x 64, 7.6 (9.1).  A handful of tiles (1-D grids) takes
-  // eight, for the latency of the plain log-sum-exp.
-  if (items >= 32) return launch_pass<1, 4>(a, epi, nbatch, s);
-  return launch_pass<1, 8>(a, epi, nbatch, s);
+  // are not hidden); 64 x 64, 7.6 (9.1).
+  return launch_pass<1, 4>(a, epi, nbatch, s);
 }
 
 }  // namespace uot
