@@ -435,6 +435,29 @@ cudaError_t noalloc_scratch(char** out) {
 }  // namespace
 }  // namespace uot
 
+namespace uot {
+namespace {
+
+// From raw log-sums z: the plan's marginal (plan.out) and eps z in their place.
+__global__ void k_plan_and_scale(double* __restrict__ z, int64_t n, int ffmode, Epilogue plan, Epilogue scale) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    if (ffmode) {
+      const ff v = ffl(reinterpret_cast<const float2*>(z)[i]);
+      float a, b;
+      apply_epilogue_ff(plan, 0, i, v, a, b);
+      apply_epilogue_ff(scale, 0, i, v, a, b);
+    } else {
+      const double v = z[i];
+      double a, b;
+      apply_epilogue(plan, 0, i, v, a, b);
+      apply_epilogue(scale, 0, i, v, a, b);
+    }
+  }
+}
+
+}  // namespace
+}  // namespace uot
+
 extern "C" {
 
 uot_status uot_gibbs_log_noalloc(const uot_geom* g, const void* W, const void* w, double eps,
@@ -594,22 +617,29 @@ uot_status uot_objective(const uot_geom* g, const void* p, const void* dx, const
   Epilogue e;
   memset(&e, 0, sizeof(e));
   set_eps(e, eps);
-  // r1 = R dy, r2 = R^T dx
+  // one application of K to b gives both r1 = R dy and S = eps log K(b.dy)
+  e.mode = EPI_RAW;
+  e.out = S1;
+  UOT_CK(G.apply(0, Vd, logdy, eps, e, s));
+  Epilogue plan = e, scale = e;
+  plan.mode = EPI_PLAN;
+  plan.ncols = 1;
+  plan.out = r1;
+  plan.pot_shift = Ud;
+  scale.mode = EPI_SCALE;
+  count_launches(1);
+  k_plan_and_scale<<<nblocks(n), kNT, 0, s>>>(S1, n, precision != UOT_F64, plan, scale);
+  UOT_CK(cudaGetLastError());
+  // r2 = R^T dx
   e.mode = EPI_PLAN;
   e.ncols = 1;
-  e.out = r1;
-  e.pot_shift = Ud;
-  UOT_CK(G.apply(0, Vd, logdy, eps, e, s));
   e.out = r2;
   e.pot_shift = Vd;
   UOT_CK(G.apply(1, Ud, logdx, eps, e, s));
-  // z_i = log sum_j K_ij dy_j  (for sum dx dy K) and S = eps log K(b.dy)
+  // z_i = log sum_j K_ij dy_j  (for sum dx dy K)
   e.mode = EPI_RAW;
   e.out = zK1;
   UOT_CK(G.apply(0, zero, logdy, eps, e, s));
-  e.mode = EPI_SCALE;
-  e.out = S1;
-  UOT_CK(G.apply(0, Vd, logdy, eps, e, s));
   const DivParams D1 = make_div(*F1), D2 = make_div(*F2);
   if (precision != UOT_F64) {
     double* arrs_n[] = {Ud, logp, logdx, r1, zK1, S1};

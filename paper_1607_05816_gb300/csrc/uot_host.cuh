@@ -712,6 +712,17 @@ class Scratch {
       : s_(s), fixed_(fixed_base), capacity_(capacity) {}
   ~Scratch() {
     if (base_ && !fixed_) cudaFreeAsync(base_, s_);
+    if (extra_) cudaFreeAsync(extra_, s_);
+  }
+  // One more block that the caller can do without: NULL (and no error) when it
+  // does not fit the device's free memory.
+  void* try_extra(size_t bytes) {
+    if (fixed_ || extra_) return nullptr;
+    if (cudaMallocAsync(&extra_, bytes, s_) != cudaSuccess) {
+      (void)cudaGetLastError();
+      extra_ = nullptr;
+    }
+    return extra_;
   }
   template <typename T>
   void reserve(size_t count) { need_ += round(count * sizeof(T)); }
@@ -745,6 +756,7 @@ class Scratch {
   char* fixed_ = nullptr;
   size_t capacity_ = 0;
   char* base_ = nullptr;
+  void* extra_ = nullptr;
   size_t need_ = 0, off_ = 0;
   bool overflow_ = false;
 };
@@ -789,6 +801,9 @@ struct Gibbs {
   // in float-float (grid_pass_ffp, points_ffp), below the FP32 passes'
   // rounding floor
   bool precise = false;
+  // FP64 point clouds (k_points64.cu), and the eps their stored kernel is of
+  Points64 p64 = {};
+  double p64_eps = -1.0;
   void* Lscratch = nullptr;     // rows: shifted input line
   void* part = nullptr;         // FP32 point clouds: per-chunk partial sums
   float* zrow[2] = {nullptr, nullptr};  // FP32 point clouds: previous results per direction
@@ -822,6 +837,18 @@ struct Gibbs {
     } else {
       const int64_t mx = (g.n > g.m ? g.n : g.m);
       sc.reserve<char>(lscratch_bytes(mx));
+      if (points64() && host_setup) {
+        sc.reserve<float>((size_t)g.n * g.d);
+        sc.reserve<float>((size_t)g.m * g.d);
+        sc.reserve<float>((size_t)mx);
+        if (p64_stored()) {
+          sc.reserve<double>((size_t)g.n);
+          sc.reserve<double>((size_t)g.m);
+          sc.reserve<double>((size_t)g.m);
+          sc.reserve<double>(points64_part_elems(g.n, g.m));
+          sc.reserve<int>(1);
+        }
+      }
       if (points_fast()) {
         sc.reserve<float2>(part_elems());
         if (speculate) {
@@ -844,6 +871,13 @@ struct Gibbs {
   // times that: it pays from a few lines on, and in any solve (one build per eps).
   bool fac_wanted(int dir, int ax) const {
     return prec == UOT_F64 && host_setup && (speculate || pass_lines(dir, ax) * nbatch >= 8);
+  }
+  bool points64() const { return g.kind == UOT_GEOM_POINTS && prec == UOT_F64; }
+  // A solver's passes at one eps share a stored kernel of up to 4 GiB (23000 x
+  // 23000 points), where the device has that much free.
+  bool p64_stored() const {
+    return points64() && host_setup && speculate && nbatch == 1 &&
+           (size_t)g.n * points64_ld(g.m) * sizeof(double) <= ((size_t)4 << 30);
   }
   bool points_fast() const {
     return g.kind == UOT_GEOM_POINTS && prec != UOT_F64 && g.d <= 3 && points_chunks_fit(g.n) &&
@@ -976,6 +1010,36 @@ struct Gibbs {
       const int64_t mx = (g.n > g.m ? g.n : g.m);
       Lscratch = sc.take<char>(lscratch_bytes(mx));
       if (!Lscratch) return cudaErrorInvalidValue;
+      if (points64()) {
+        p64.x = (const double*)g.x;
+        p64.y = (const double*)g.y;
+        p64.n = g.n;
+        p64.m = g.m;
+        p64.d = g.d;
+        p64.Ls = (double*)Lscratch;
+        if (host_setup) {
+          float* x32 = sc.take<float>((size_t)g.n * g.d);
+          float* y32 = sc.take<float>((size_t)g.m * g.d);
+          p64.L32 = sc.take<float>((size_t)mx);
+          if (!x32 || !y32 || !p64.L32) return cudaErrorInvalidValue;
+          count_launches(2);
+          k_from_f64<float><<<nblocks((int64_t)g.n * g.d), kNT, 0, s>>>(p64.x, (int64_t)g.n * g.d, x32);
+          k_from_f64<float><<<nblocks((int64_t)g.m * g.d), kNT, 0, s>>>(p64.y, (int64_t)g.m * g.d, y32);
+          p64.x32 = x32;
+          p64.y32 = y32;
+          if (p64_stored()) {
+            p64.M = sc.take<double>((size_t)g.n);
+            p64.beta = sc.take<double>((size_t)g.m);
+            p64.w = sc.take<double>((size_t)g.m);
+            p64.part = sc.take<double>(points64_part_elems(g.n, g.m));
+            p64.drift = sc.take<int>(1);
+            if (!p64.drift) return cudaErrorInvalidValue;
+            cudaError_t e0 = cudaMemsetAsync(p64.drift, 0, sizeof(int), s);
+            if (e0 != cudaSuccess) return e0;
+            p64.K = (double*)sc.try_extra((size_t)g.n * points64_ld(g.m) * sizeof(double));
+          }
+        }
+      }
       if (g.kind == UOT_GEOM_DENSE && prec == UOT_F64) {
         // the prefilter's block counter (first bytes of the scratch)
         cudaError_t e0 = cudaMemsetAsync(Lscratch, 0, 256, s);
@@ -1133,6 +1197,13 @@ struct Gibbs {
         if (e.logp) e.logp += b * e.bstride_p;
         if (e.pot_shift) e.pot_shift += b * e.bstride;
         if (e.err) e.err += 2 * b;
+      }
+      if (points64()) {
+        const bool first = p64_eps != eps;
+        cudaError_t err = launch_points64(p64, dir, W + (int64_t)b * nin, logw, eps, first, e, s);
+        if (err != cudaSuccess) return err;
+        if (dir == 0 && p64.K) p64_eps = eps;
+        continue;
       }
       const int use_prev = (nbatch == 1 && zrow[dir] != nullptr && zeps[dir] == eps) ? 1 : 0;
       cudaError_t err = launch_rows(prec == UOT_F64 ? UOT_F64 : UOT_F32, rg, nrows, nin,

@@ -689,6 +689,30 @@ cudaError_t launch_points_ffp(const float* x, const float* y, int d, int nout, i
 // Scratch of launch_rows for FP64 dense rows with the FP32 prefilter; its
 // first 4 bytes hold a counter that must be zero before the first launch.
 size_t rows_pf_scratch_bytes(int64_t nin);
+// FP64 point clouds (k_points64.cu).  K NULL: on the fly in both directions.
+struct Points64 {
+  const double* x;     // [n][d]
+  const double* y;     // [m][d]
+  const float* x32;    // FP32 copies (NULL: the shifts are found in FP64)
+  const float* y32;
+  int n, m, d;
+  double* Ls;          // [max(n, m)]
+  float* L32;          // [max(n, m)], with the FP32 copies
+  // stored kernel of one eps: [n][points64_ld(m)], shifts [n], the line it was
+  // stored with [m], weights [m], column partials, and a flag (zero at first)
+  double* K;
+  double* M;
+  double* beta;
+  double* w;
+  double* part;        // points64_part_elems(n, m)
+  int* drift;
+};
+int64_t points64_ld(int m);
+size_t points64_part_elems(int n, int m);
+// dir 0: W on the Y side, result on the X side; first: no pass of this eps has
+// stored its kernel yet (a dir 0 pass then does).
+cudaError_t launch_points64(const Points64& p, int dir, const double* W, const double* logw, double eps, bool first,
+                            const Epilogue& epi, cudaStream_t s);
 int points_nchunks(int nin, int nout);
 bool points_chunks_fit(int nin);
 cudaError_t launch_points(const float* x, const float* y, int d, int nout, int nin,
