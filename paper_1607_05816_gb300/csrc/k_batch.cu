@@ -210,12 +210,12 @@ struct Half {
 // violation terms.
 __device__ __forceinline__ void output_epilogue(const Half& h, int i, float Mo, float So, float mx, float& num,
                                                 float& den) {
-  const ff ln2 = ln2_ff();
   ff z = ff_ninf();
-  if (Mo != -INFINITY && So > 0.0f) z = ff_add_f(ff_add_f(ff_mul_f(ln2, Mo), mx), kLn2 * lg2_approx(So));
+  if (Mo != -INFINITY && So > 0.0f) z = pass_result(mx, Mo, So);
   h.zprev[i] = z.hi;
   const ff eps = ffl(h.eps_ff);
-  const ff S = (z.hi == -INFINITY) ? ff_ninf() : ff_mul(z, eps);
+  ff S = ffn_mul(z, eps);
+  if (z.hi == -INFINITY) S = ff_ninf();
   const ff Un = prox_update_ff(h.F, ffl(h.lpout[i]), S, eps);
   if (h.check) {
     float va, vb;
@@ -235,9 +235,7 @@ __device__ void half_step(const Half& h, float4* st0, typename Stage1<D>::T* st1
   // ---- input line L_j = W_j/eps + log w_j (float-float), staged relative to its maximum ----
   float mx = -INFINITY;
   for (int j = tid; j < nin; j += NT) {
-    const ff w = ffl(h.Win[j]);
-    ff L = ff_ninf();
-    if (w.hi != -INFINITY) L = ff_add(ff_mul(w, ffl(h.inv_eps_ff)), ffl(h.lwin[j]));
+    const ff L = line_value_ff(ffl(h.Win[j]), ffl(h.inv_eps_ff), ffl(h.lwin[j]));
     st0[j] = make_float4(L.hi, L.lo, 0.0f, 0.0f);  // rewritten below by the same thread
     mx = fmaxf(mx, L.hi);
   }

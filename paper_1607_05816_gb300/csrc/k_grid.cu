@@ -268,9 +268,7 @@ __device__ __forceinline__ void grid_item_f32(const PassArgs& a, const Epilogue&
       if (!owns[r]) continue;
       ff z = ff_ninf();
       if (So[r] > 0.0f) {
-        // z = mx + ln2 Mo + ln2 log2(So), the first product kept exact in float-float
-        const ff ln2 = ln2_ff();
-        z = ff_add_f(ff_add_f(ff_mul_f(ln2, Mo[r]), mx), kLn2 * lg2_approx(So[r]));
+        z = pass_result(mx, Mo[r], So[r]);
       }
       if (zprev) zprev[my_pt[r]] = z.hi;
       float n1, d1;
@@ -734,9 +732,7 @@ __device__ __forceinline__ void short_line_lse(ff v0, ff v1, float y0, float y1,
 #pragma unroll
   for (int q = 0; q < OPL; ++q) {
     if (S[q] > 0.0f) {
-      // z = mx + ln2 m + ln2 log2(S), the first product kept exact in float-float
-      const ff ln2 = ln2_ff();
-      z[q] = ff_add_f(ff_add_f(ff_mul_f(ln2, m[q]), mx), kLn2 * lg2_approx(S[q]));
+      z[q] = pass_result(mx, m[q], S[q]);
     }
   }
 }
@@ -849,9 +845,7 @@ __global__ void __launch_bounds__(kShortWarps * 32) grid_pass_f32_short(PassArgs
         if (!owns[q]) continue;
         ff z = ff_ninf();
         if (S[q] > 0.0f) {
-          // z = mx + ln2 m + ln2 log2(S), the first product kept exact in float-float
-          const ff ln2 = ln2_ff();
-          z = ff_add_f(ff_add_f(ff_mul_f(ln2, m[q]), mx), kLn2 * lg2_approx(S[q]));
+          z = pass_result(mx, m[q], S[q]);
         }
         if (zprev) zprev[my_pt[q]] = z.hi;
         float n1, d1;

@@ -29,8 +29,7 @@ struct PassArgs {
 __device__ __forceinline__ ff load_L_ff(const PassArgs& a, const float2* in, int64_t idx) {
   const ff v = ffl(in[idx]);
   if (!a.in_is_pot) return v;
-  if (v.hi == -INFINITY) return ff_ninf();
-  return ff_add(ff_mul(v, ffl(a.inv_eps)), ffl(a.logw[idx]));
+  return line_value_ff(v, ffl(a.inv_eps), ffl(a.logw[idx]));
 }
 
 
@@ -57,7 +56,8 @@ __device__ __forceinline__ void epilogue_apply(const Epilogue& e, int64_t b, int
   }
   num = den = 0.0f;
   const ff eps = ffl(e.eps_ff);
-  ff S = (z.hi == -INFINITY) ? ff_ninf() : ff_mul(z, eps);
+  ff S = ffn_mul(z, eps);
+  if (z.hi == -INFINITY) S = ff_ninf();
   if (e.zshift) S = ff_zshift(S, e.zshift);
   const ff Unew = prox_update_ff(e.Fff, ffl(o.lp), S, eps);
   reinterpret_cast<float2*>(e.pot)[b * e.bstride + pt] = ff2(Unew);

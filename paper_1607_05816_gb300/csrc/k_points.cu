@@ -35,9 +35,7 @@ constexpr int kMaxBlk = 1024;          // inputs per block of the max reduction
 // 1e-6 (measured), so it is not used.
 
 __device__ __forceinline__ ff load_L_pt(const float2* W, const float2* lw, int64_t j, float2 inv_eps) {
-  const ff w = ffl(W[j]);
-  if (w.hi == -INFINITY) return ff_ninf();
-  return ff_add(ff_mul(w, ffl(inv_eps)), ffl(lw[j]));
+  return line_value_ff(ffl(W[j]), ffl(inv_eps), ffl(lw[j]));
 }
 
 // Per-block maxima of the high parts of L_j = W_j/eps + log w_j.
@@ -269,10 +267,7 @@ __global__ void __launch_bounds__(256)
     }
     if (lane == 0) {
       ff z = ff_ninf();
-      if (Lmax != -INFINITY && M != -INFINITY && S > 0.0f) {
-        const ff ln2 = ln2_ff();
-        z = ff_add_f(ff_add_f(ff_mul_f(ln2, M), Lmax), kLn2 * lg2_approx(S));
-      }
+      if (Lmax != -INFINITY && M != -INFINITY && S > 0.0f) z = pass_result(Lmax, M, S);
       if (a.zprev) a.zprev[i] = z.hi;
       apply_epilogue_ff(epi, 0, i, z, num, den);
     }

@@ -78,6 +78,41 @@ __device__ __forceinline__ ff ff_mul_f(ff a, float b) {
   const float e = fmaf(a.lo, b, fmaf(a.hi, b, -p));
   return ff_fast_two_sum(p, e);
 }
+// The same sums and products for finite operands, without the branches that
+// carry infinities: on the critical path of a grid pass (line loads, epilogue)
+// those cost more than the arithmetic.  The caller replaces the result where an
+// operand is infinite.
+__device__ __forceinline__ ff ffn_fast_two_sum(float a, float b) {
+  const float s = a + b;
+  return ff{s, b - (s - a)};
+}
+__device__ __forceinline__ ff ffn_two_sum(float a, float b) {
+  const float s = a + b;
+  const float bb = s - a;
+  return ff{s, (a - (s - bb)) + (b - bb)};
+}
+__device__ __forceinline__ ff ffn_add(ff a, ff b) {
+  const ff s = ffn_two_sum(a.hi, b.hi);
+  return ffn_fast_two_sum(s.hi, s.lo + (a.lo + b.lo));
+}
+__device__ __forceinline__ ff ffn_add_f(ff a, float b) {
+  const ff s = ffn_two_sum(a.hi, b);
+  return ffn_fast_two_sum(s.hi, s.lo + a.lo);
+}
+__device__ __forceinline__ ff ffn_mul(ff a, ff b) {
+  const float p = a.hi * b.hi;
+  const float e = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, fmaf(a.hi, b.hi, -p)));
+  return ffn_fast_two_sum(p, e);
+}
+__device__ __forceinline__ ff ffn_mul_f(ff a, float b) {
+  const float p = a.hi * b;
+  return ffn_fast_two_sum(p, fmaf(a.lo, b, fmaf(a.hi, b, -p)));
+}
+// L = W/eps + log w (-inf where either is)
+__device__ __forceinline__ ff line_value_ff(ff W, ff inv_eps, ff logw) {
+  const ff r = ffn_add(ffn_mul(W, inv_eps), logw);
+  return (W.hi == -INFINITY || logw.hi == -INFINITY) ? ff{-INFINITY, 0.0f} : r;
+}
 __device__ __forceinline__ bool ff_lt(ff a, ff b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }
 __device__ __forceinline__ ff ff_min(ff a, ff b) { return ff_lt(b, a) ? b : a; }
 __device__ __forceinline__ ff ff_max(ff a, ff b) { return ff_lt(a, b) ? b : a; }
@@ -100,6 +135,11 @@ __device__ __forceinline__ float lg2_approx(float x) {
   float y;
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
+}
+
+// mx + ln2 (M + log2 S), the first product kept exact in float-float (finite M, S > 0).
+__device__ __forceinline__ ff pass_result(float mx, float M, float S) {
+  return ffn_add_f(ffn_add_f(ffn_mul_f(ln2_ff(), M), mx), kLn2 * lg2_approx(S));
 }
 
 // Packed FP32 pairs: the f32x2 arithmetic of the sm_100 family.
@@ -288,27 +328,26 @@ __device__ inline void apply_epilogue(const Epilogue& e, int64_t b, int64_t pt, 
   }
 }
 
-// Table 1 in log form, float-float version of prox_update.
+// Table 1 in log form, float-float version of prox_update; the KL, EQ and TV
+// rows without branches on the values.
 __device__ inline ff prox_update_ff(const DivFF& F, ff logp, ff S, ff eps) {
-  if (S.hi == -INFINITY) return ff_ninf();
-  const ff ubar = (logp.hi == -INFINITY) ? ff_ninf() : ff_sub(ff_mul(eps, logp), S);
-  switch (F.kind) {
-    case UOT_DIV_EQ:
-      return ubar;
-    case UOT_DIV_KL:
-      return (ubar.hi == -INFINITY) ? ubar : ff_mul(ffl(F.zf), ubar);
-    case UOT_DIV_TV: {
-      const ff lam = ffl(F.lam);
-      return ff_min(lam, ff_max(ff_neg(lam), ubar));
-    }
-    default: {
-      const ff lo = (F.elog_a.x == -INFINITY || ubar.hi == -INFINITY) ? ff_ninf() : ff_add(ffl(F.elog_a), ubar);
-      const ff inner = ff_max(lo, ff{0.0f, 0.0f});
-      if (F.elog_b.x == INFINITY) return inner;
-      const ff hi = (ubar.hi == -INFINITY) ? ff_ninf() : ff_add(ffl(F.elog_b), ubar);
-      return ff_min(hi, inner);
-    }
+  if (F.kind == UOT_DIV_RG) {
+    if (S.hi == -INFINITY) return ff_ninf();
+    const ff ubar = (logp.hi == -INFINITY) ? ff_ninf() : ff_sub(ff_mul(eps, logp), S);
+    const ff lo = (F.elog_a.x == -INFINITY || ubar.hi == -INFINITY) ? ff_ninf() : ff_add(ffl(F.elog_a), ubar);
+    const ff inner = ff_max(lo, ff{0.0f, 0.0f});
+    if (F.elog_b.x == INFINITY) return inner;
+    const ff hi = (ubar.hi == -INFINITY) ? ff_ninf() : ff_add(ffl(F.elog_b), ubar);
+    return ff_min(hi, inner);
   }
+  ff u = ffn_add(ffn_mul(eps, logp), ff_neg(S));
+  if (F.kind == UOT_DIV_KL) u = ffn_mul(ffl(F.zf), u);
+  if (logp.hi == -INFINITY) u = ff_ninf();
+  if (F.kind == UOT_DIV_TV) {
+    const ff lam = ffl(F.lam);
+    u = ff_min(lam, ff_max(ff_neg(lam), u));
+  }
+  return (S.hi == -INFINITY) ? ff_ninf() : u;
 }
 
 // FP32 violation terms from float-float potentials: r_new = e^{(U_new+S)/eps},
@@ -361,7 +400,8 @@ __device__ inline void apply_epilogue_ff(const Epilogue& e, int64_t b, int64_t p
       break;
     case EPI_PROX: {
       const ff eps = ffl(e.eps_ff);
-      ff S = (z.hi == -INFINITY) ? ff_ninf() : ff_mul(z, eps);
+      ff S = ffn_mul(z, eps);
+      if (z.hi == -INFINITY) S = ff_ninf();
       if (e.zshift) S = ff_zshift(S, e.zshift);
       float2* pot = reinterpret_cast<float2*>(e.pot);
       const ff Uold = ffl(pot[q]);
