@@ -270,7 +270,9 @@ int uot_autotune_table(char* buf, int len);
 
 /*
  * CTA size of uot_solve_batch (a schedule choice; results differ only in FP32
- * summation order).  8 or 16 warps per CTA are compiled; with the tuner on,
+ * summation order).  Few or uneven problems run on clusters of 2 to 8 CTAs of 16
+ * warps (an estimate of the schedule decides), others on one CTA each, as do all
+ * when a size is forced.  8 or 16 warps per CTA are compiled; with the tuner on,
  * the first call for a batch shape (d, largest n, largest m) times both on a
  * sample of the batch (every (nprob/S)-th problem of the size-ordered queue,
  * S = 2 x SM count, six iterations) and keeps the 8-warp CTA unless the other

@@ -9,8 +9,16 @@
 //   T_j = eps log sum_i exp((U_i - |x_i - y_j|^2)/eps) dx_i ;  V_j = prox_F2(T_j)
 //
 // until the marginal violation of the problem is <= tol or the iteration cap.
-// There is no communication between CTAs except the atomic work counter, so
-// no CTA ever waits on another one.
+// There is no communication between work units except the atomic work counter,
+// so no unit ever waits on another one.  A work unit is one CTA, or a cluster of
+// 2, 4 or 8 CTAs that share a problem: CTA r of CL takes output blocks r, r + CL,
+// ..., every CTA stages the whole input side, and a cluster barrier ends each
+// half-step.  One CTA per problem is bounded by the largest problem as soon as
+// its share of the work exceeds the others' (512 clouds of 64 to 2048 points in
+// 2-D, 50 iterations: 28.5 ms, the time of the 2048 x 2048 problem on half an
+// SM; clusters of 2: 20.9 ms, and 19.3 ms with the sweeps unrolled by 8 instead of
+// 2; clusters of 4: 21.3, of 8: 27.9); the cluster size comes from a
+// list-scheduling estimate of the batch (batch_cluster).
 //
 // Per half-step the CTA stages the input side {t_j, y_j} in shared memory
 // (the only per-problem data kept there, so several CTAs share an SM) and
@@ -26,11 +34,15 @@
 // Two CTA sizes (8 or 16 warps) are compiled for each dimension; the first
 // call with a given (d, largest n, largest m) times both on a sample of the
 // batch and keeps the faster one.
+#include <cooperative_groups.h>
 #include <string.h>
 
 #include <algorithm>
+#include <cmath>
+#include <functional>
 #include <map>
 #include <mutex>
+#include <queue>
 #include <string>
 #include <vector>
 
@@ -157,7 +169,7 @@ __device__ __forceinline__ void sweep(const float4* st0, const typename Stage1<D
   const f2p zero2 = pk(0.0f, 0.0f);
   if (exact) {
     float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll 2
+#pragma unroll 8
     for (int j = j0; j < j1; ++j) {
       f2p EA, EB;
       term_exponents<D>(st0, st1, j, X, nk2, zero2, zero2, EA, EB);
@@ -173,7 +185,7 @@ __device__ __forceinline__ void sweep(const float4* st0, const typename Stage1<D
   const f2p MA = pk(mq[0] == -INFINITY ? 0.0f : mq[0], mq[1] == -INFINITY ? 0.0f : mq[1]);
   const f2p MB = pk(mq[2] == -INFINITY ? 0.0f : mq[2], mq[3] == -INFINITY ? 0.0f : mq[3]);
   f2p SA = zero2, SB = zero2;
-#pragma unroll 2
+#pragma unroll 8
   for (int j = j0; j < j1; ++j) {
     f2p EA, EB;
     term_exponents<D>(st0, st1, j, X, nk2, MA, MB, EA, EB);
@@ -226,9 +238,11 @@ __device__ __forceinline__ void output_epilogue(const Half& h, int i, float Mo, 
   h.Wout[i] = ff2(Un);
 }
 
+// CTA `rank` of the CL that share the problem computes output blocks rank,
+// rank + CL, ...; its local block b is the problem's block rank + CL b.
 template <int D, int NW>
-__device__ void half_step(const Half& h, float4* st0, typename Stage1<D>::T* st1, float2* part, float* red,
-                          float& num, float& den) {
+__device__ void half_step(const Half& h, int rank, int CL, float4* st0, typename Stage1<D>::T* st1, float2* part,
+                          float* red, float& num, float& den) {
   constexpr int NT = NW * 32;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nin = h.nin, nout = h.nout;
@@ -242,7 +256,8 @@ __device__ void half_step(const Half& h, float4* st0, typename Stage1<D>::T* st1
   mx = block_max<NT>(mx, red);
   if (mx == -INFINITY) {
     // b = 0 everywhere: every sum is empty
-    for (int i = tid; i < nout; i += NT) output_epilogue(h, i, -INFINITY, 0.0f, 0.0f, num, den);
+    for (int i = tid; i < nout; i += NT)
+      if (CL == 1 || (i / kOB) % CL == rank) output_epilogue(h, i, -INFINITY, 0.0f, 0.0f, num, den);
     __syncthreads();
     return;
   }
@@ -263,12 +278,16 @@ __device__ void half_step(const Half& h, float4* st0, typename Stage1<D>::T* st1
   __syncthreads();
 
   const f2p nk2 = pk(-h.k2, -h.k2);
-  const int nblk = (nout + kOB - 1) / kOB;
+  const int nblk = ((nout + kOB - 1) / kOB - rank + CL - 1) / CL;  // this CTA's blocks
+  if (nblk < 1) {
+    __syncthreads();
+    return;
+  }
   const int split = nblk >= NW ? 1 : NW / nblk;
   if (split == 1) {
     // one warp per block of 128 outputs, the whole contraction each
     for (int b = warp; b < nblk; b += NW) {
-      const int base = b * kOB;
+      const int base = (rank + CL * b) * kOB;
       XPairs X;
       bool valid[4];
       load_x<D>(h.xo, nout, base, lane, X, valid);
@@ -306,7 +325,7 @@ __device__ void half_step(const Half& h, float4* st0, typename Stage1<D>::T* st1
   const int b = warp % nblk, r = warp / nblk;
   const int J = (nin + split - 1) / split;
   const int j0 = min(nin, r * J), j1 = min(nin, j0 + J);
-  const int base = b * kOB;
+  const int base = (rank + CL * b) * kOB;
   XPairs X;
   bool valid[4];
   load_x<D>(h.xo, nout, base, lane, X, valid);
@@ -336,10 +355,10 @@ __device__ void half_step(const Half& h, float4* st0, typename Stage1<D>::T* st1
 #pragma unroll
     for (int u = 0; u < OWN; ++u) {
       const int o = tid + u * NT;  // output o of the CTA's nblk*128
+      const int bo = o / kOB, oo = o % kOB;
       Mo[u] = -INFINITY;
       So[u] = 0.0f;
-      if (o < nblk * kOB && o < nout) {
-        const int bo = o / kOB, oo = o % kOB;
+      if (bo < nblk && (rank + CL * bo) * kOB + oo < nout) {
         for (int rr = 0; rr < split; ++rr) {
           const float2 pr = part[(rr * nblk + bo) * kOB + oo];
           if (pr.y > 0.0f) Mo[u] = fmaxf(Mo[u], pr.x);
@@ -363,7 +382,8 @@ __device__ void half_step(const Half& h, float4* st0, typename Stage1<D>::T* st1
 #pragma unroll
   for (int u = 0; u < OWN; ++u) {
     const int o = tid + u * NT;
-    if (o < nblk * kOB && o < nout) output_epilogue(h, o, Mo[u], So[u], mx, num, den);
+    const int i = (rank + CL * (o / kOB)) * kOB + o % kOB;
+    if (o < nblk * kOB && i < nout) output_epilogue(h, i, Mo[u], So[u], mx, num, den);
   }
   __syncthreads();
 }
@@ -415,31 +435,39 @@ __device__ double block_side_lse(const float2* W, const float2* lp, const float2
   return M + log(S);
 }
 
+// Barrier of the CTAs that share a problem; orders their global writes too.
+template <bool kCl>
+__device__ __forceinline__ void unit_sync() {
+  if constexpr (kCl) cooperative_groups::this_cluster().sync();
+  else __syncthreads();
+}
+
 // Translation step (uot_opts.translate; not in the paper: the translation-
 // invariant formulation of Sejourne, Vialard, Peyre 2022): U += c, V -= c with
 // c = lam1 lam2 / (lam1 + lam2) (log A - log B), the exact maximum of the dual
 // along that direction for KL penalties; A = sum dx p e^{-U/lam1}, B = sum dy
 // q e^{-V/lam2}.  The plan is unchanged.
-template <int NW>
-__device__ void translate_problem(float2* U, float2* V, const float2* lpU, const float2* lwU, const float2* lpV,
+template <int NW, bool kCl>
+__device__ void translate_problem(int rank, int CL, float2* U, float2* V, const float2* lpU, const float2* lwU, const float2* lpV,
                                   const float2* lwV, int n, int m, double2 lam, double* red) {
   constexpr int NT = NW * 32;
   const double la = block_side_lse<NW>(U, lpU, lwU, n, 1.0 / lam.x, red);
   const double lb = block_side_lse<NW>(V, lpV, lwV, m, 1.0 / lam.y, red);
   const double c = (la != -kInf && lb != -kInf) ? lam.x * lam.y / (lam.x + lam.y) * (la - lb) : 0.0;
   const ff cp = ff_make(c), cn = ff_make(-c);
-  for (int i = threadIdx.x; i < n; i += NT) {
+  unit_sync<kCl>();  // every CTA of the unit has summed the old U and V
+  for (int i = threadIdx.x + rank * NT; i < n; i += NT * CL) {
     const float2 u = U[i];
     if (!isinf(u.x)) U[i] = ff2(ff_add(ffl(u), cp));
   }
-  for (int j = threadIdx.x; j < m; j += NT) {
+  for (int j = threadIdx.x + rank * NT; j < m; j += NT * CL) {
     const float2 v = V[j];
     if (!isinf(v.x)) V[j] = ff2(ff_add(ffl(v), cn));
   }
-  __syncthreads();
+  unit_sync<kCl>();
 }
 
-template <int D, int NW>
+template <int D, int NW, bool kCl>
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 3 : 2) batch_solve(BatchArgs a) {
   constexpr int NT = NW * 32;
   typedef typename Stage1<D>::T S1;
@@ -448,17 +476,25 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 3 : 2) batch_solve(BatchArg
   __shared__ int s_prob;
   __shared__ int s_stop;
   __shared__ double tr_red[2 * NW];
+  __shared__ float2 csum;  // this CTA's violation sums, read by its cluster
   const int tid = threadIdx.x;
+  int rank = 0, CL = 1;
+  if constexpr (kCl) {
+    rank = (int)cooperative_groups::this_cluster().block_rank();
+    CL = (int)cooperative_groups::this_cluster().num_blocks();
+  }
   const int lmax = a.nmax > a.mmax ? a.nmax : a.mmax;
   float4* st0 = smem4;
   S1* st1 = reinterpret_cast<S1*>(st0 + lmax);
   float2* part = reinterpret_cast<float2*>(reinterpret_cast<char*>(st0 + lmax) + (size_t)lmax * stage1_bytes<D>());
   for (;;) {
-    if (tid == 0) {
+    if (tid == 0 && rank == 0) {
       const int t = atomicAdd(a.next, 1);
       s_prob = (t < a.nprob) ? a.order[t] : -1;
+      if constexpr (kCl)
+        for (int r = 1; r < CL; ++r) *cooperative_groups::this_cluster().map_shared_rank(&s_prob, r) = s_prob;
     }
-    __syncthreads();
+    unit_sync<kCl>();
     const int k = s_prob;
     if (k < 0) break;
     const int n = a.n[k], m = a.m[k];
@@ -467,9 +503,9 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 3 : 2) batch_solve(BatchArg
     const float* yk = a.y + yo * D;
     float2* U = a.Uff + xo;
     float2* V = a.Vff + yo;
-    for (int i = tid; i < n; i += NT) U[i] = make_float2(0.0f, 0.0f);
-    for (int j = tid; j < m; j += NT) V[j] = make_float2(0.0f, 0.0f);
-    __syncthreads();
+    for (int i = tid + rank * NT; i < n; i += NT * CL) U[i] = make_float2(0.0f, 0.0f);
+    for (int j = tid + rank * NT; j < m; j += NT * CL) V[j] = make_float2(0.0f, 0.0f);
+    unit_sync<kCl>();
     int it_final = 0;
     float err = INFINITY;
     Half h1, h2;
@@ -507,15 +543,28 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 3 : 2) batch_solve(BatchArg
         h1.use_prev = h2.use_prev = it > 0;
         h1.check = check;
         float num = 0.0f, den = 0.0f;
-        half_step<D, NW>(h1, st0, st1, part, red, num, den);
+        half_step<D, NW>(h1, rank, CL, st0, st1, part, red, num, den);
+        if (kCl) unit_sync<kCl>();
         float dn = 0.0f, dd = 0.0f;
-        half_step<D, NW>(h2, st0, st1, part, red, dn, dd);
+        half_step<D, NW>(h2, rank, CL, st0, st1, part, red, dn, dd);
+        if (kCl) unit_sync<kCl>();
         if (a.translate && (final_stage ? check : (it + 1) % a.check_every == 0))
-          translate_problem<NW>(U, V, a.logp + xo, a.logdx + xo, a.logq + yo, a.logdy + yo, n, m, a.lam[k],
+          translate_problem<NW, kCl>(rank, CL, U, V, a.logp + xo, a.logdx + xo, a.logq + yo, a.logdy + yo, n, m, a.lam[k],
                                 tr_red);
         if (final_stage) it_final = it + 1;
         if (check) {
-          const float2 tot = block_sum2<NT>(num, den, red);
+          float2 tot = block_sum2<NT>(num, den, red);
+          if constexpr (kCl) {  // the CTAs' sums, added in rank order by every CTA
+            if (tid == 0) csum = tot;
+            unit_sync<kCl>();
+            tot = make_float2(0.0f, 0.0f);
+            for (int r = 0; r < CL; ++r) {
+              const float2 c = *cooperative_groups::this_cluster().map_shared_rank(&csum, r);
+              tot.x += c.x;
+              tot.y += c.y;
+            }
+            unit_sync<kCl>();  // csum may be written again
+          }
           err = (tot.y > 0.0f) ? tot.x / tot.y : 0.0f;
           if (tid == 0) s_stop = (it > 0 && a.tol > 0.0f && err <= a.tol) ? 1 : 0;
           __syncthreads();
@@ -523,25 +572,25 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 3 : 2) batch_solve(BatchArg
         }
       }
     }
-    for (int i = tid; i < n; i += NT) {
+    for (int i = tid + rank * NT; i < n; i += NT * CL) {
       const float2 u = U[i];
       if (a.Uout64)
         a.Uout64[xo + i] = (u.x == -INFINITY) ? -kInf : (double)u.x + (double)u.y;
       else
         a.Uout[xo + i] = (u.x == -INFINITY) ? u.x : u.x + u.y;
     }
-    for (int j = tid; j < m; j += NT) {
+    for (int j = tid + rank * NT; j < m; j += NT * CL) {
       const float2 v = V[j];
       if (a.Vout64)
         a.Vout64[yo + j] = (v.x == -INFINITY) ? -kInf : (double)v.x + (double)v.y;
       else
         a.Vout[yo + j] = (v.x == -INFINITY) ? v.x : v.x + v.y;
     }
-    if (tid == 0) {
+    if (tid == 0 && rank == 0) {
       a.iters_out[k] = it_final;
       a.err_out[k] = err;
     }
-    __syncthreads();
+    unit_sync<kCl>();  // s_prob has been read by every thread
   }
 }
 
@@ -552,9 +601,9 @@ template <int D, int NW>
 cudaError_t launch_variant(const BatchArgs& a, int grid, cudaStream_t s) {
   const int lmax = std::max(a.nmax, a.mmax);
   const size_t smem = smem_bytes<D, NW>(lmax);
-  cudaError_t e = smem_at_least(batch_solve<D, NW>, smem);
+  cudaError_t e = smem_at_least(batch_solve<D, NW, false>, smem);
   if (e != cudaSuccess) return e;
-  batch_solve<D, NW><<<grid, NW * 32, smem, s>>>(a);
+  batch_solve<D, NW, false><<<grid, NW * 32, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -562,12 +611,12 @@ template <int D, int NW>
 int ctas_variant(int nmax, int mmax) {
   const size_t smem = smem_bytes<D, NW>(std::max(nmax, mmax));
   int nb = 0;
-  if (smem_at_least(batch_solve<D, NW>, smem) !=
+  if (smem_at_least(batch_solve<D, NW, false>, smem) !=
       cudaSuccess) {
     (void)cudaGetLastError();
     return 0;
   }
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_solve<D, NW>, NW * 32, smem) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_solve<D, NW, false>, NW * 32, smem) != cudaSuccess) {
     (void)cudaGetLastError();
     return 0;
   }
@@ -624,6 +673,65 @@ struct BEntry {
 std::mutex g_bmu;
 std::map<BKey, BEntry> g_btuned;
 int g_bforced = -1;  // forced variant, -1: tuned
+
+// ---- clusters ----
+
+// Launch configuration of clusters of CL 16-warp CTAs, and how many clusters
+// the device holds at once (0: not available).
+constexpr int kClWarps = 16;
+template <int D>
+int cluster_config(int CL, int lmax, cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, cudaStream_t s) {
+  const size_t smem = smem_bytes<D, kClWarps>(lmax);
+  int n = 0;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(CL);
+  cfg.blockDim = dim3(kClWarps * 32);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = CL;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (smem_at_least(batch_solve<D, kClWarps, true>, smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, batch_solve<D, kClWarps, true>, &cfg) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
+int cluster_count(int d, int CL, int lmax) {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[1];
+  return d == 1 ? cluster_config<1>(CL, lmax, cfg, attr, nullptr)
+         : d == 2 ? cluster_config<2>(CL, lmax, cfg, attr, nullptr)
+                  : cluster_config<3>(CL, lmax, cfg, attr, nullptr);
+}
+
+template <int D>
+cudaError_t launch_cluster(const BatchArgs& a, int CL, cudaStream_t s) {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[1];
+  const int n = cluster_config<D>(CL, std::max(a.nmax, a.mmax), cfg, attr, s);
+  if (n < 1) return cudaErrorInvalidConfiguration;
+  cfg.gridDim = dim3((unsigned)(CL * std::min(n, a.nprob)));
+  return cudaLaunchKernelEx(&cfg, batch_solve<D, kClWarps, true>, a);
+}
+
+// Cycles of one half-step of a CTA that shares its SM with another one: a term
+// takes 2 d + 3 FMA-pipe lanes, a warp 4 (2 d + 3) pipe cycles per input for its
+// 128 outputs, and eight warps share a pipe; the constant stands for the latencies of the staging,
+// the merge and the epilogue (and of the cluster barrier).
+double half_cost(int d, int nout, int nin, int CL) {
+  const int loc = ((nout + kOB - 1) / kOB + CL - 1) / CL;
+  const int split = loc >= kClWarps ? 1 : kClWarps / loc;
+  const int rounds = (loc + kClWarps - 1) / kClWarps;
+  const double busy = (double)std::min(loc * split, kClWarps) / kClWarps;
+  const double sweep = rounds * std::ceil((double)nin / split) * 8.0 * 4.0 * (2 * d + 3) * busy;
+  return sweep + 600.0 * ((nin + 511) / 512) + 3000.0 + (CL > 1 ? 1500.0 : 0.0);
+}
 
 // Times both CTA sizes on a sample of the batch: every (nprob/S)-th problem
 // of the size-ordered queue, six iterations at the first eps, no tolerance
@@ -738,6 +846,55 @@ std::string batch_tune_table() {
     s += buf;
   }
   return s;
+}
+
+// CTAs per problem: the cluster size whose list schedule (problems in queue
+// order, each to the unit that is free first) ends earliest by half_cost, the
+// smaller one within 3%, and none of more CTAs than the largest side has output
+// blocks.  One CTA where no problem is larger than an eighth of a
+// unit's average load: clusters could shorten such a batch by little.
+int batch_cluster(int d, int nmax, int mmax, const int* n, const int* m, const int* order, int nprob) {
+  {
+    std::lock_guard<std::mutex> lk(g_bmu);
+    if (g_bforced >= 0) return 1;
+  }
+  const int per = ctas_any(d, 1, nmax, mmax) * sm_count();
+  if (per < 1) return 1;
+  int best = 1;
+  double best_t = 0.0;
+  for (int CL : {1, 2, 4, 8}) {
+    if (CL > (std::max(nmax, mmax) + kOB - 1) / kOB) break;
+    const int units = CL == 1 ? per : cluster_count(d, CL, std::max(nmax, mmax));
+    if (units < 1) continue;
+    double sum = 0.0, most = 0.0, end = 0.0;
+    std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+    for (int t = 0; t < nprob; ++t) {
+      const int k = order[t];
+      const double c = half_cost(d, n[k], m[k], CL) + half_cost(d, m[k], n[k], CL);
+      sum += c;
+      most = std::max(most, c);
+      double at = c;
+      if ((int)free_at.size() == units) {
+        at += free_at.top();
+        free_at.pop();
+      }
+      free_at.push(at);
+      end = std::max(end, at);
+    }
+    if (CL == 1) {
+      if (most <= sum / units / 8.0) return 1;
+      best_t = end;
+    } else if (end < 0.97 * best_t) {
+      best_t = end;
+      best = CL;
+    }
+  }
+  return best;
+}
+
+cudaError_t launch_batch_cluster(const BatchArgs& a, int CL, cudaStream_t s) {
+  count_launches(1);
+  return a.d == 1 ? launch_cluster<1>(a, CL, s) : a.d == 2 ? launch_cluster<2>(a, CL, s) : launch_cluster<3>(a, CL, s);
 }
 
 int batch_ctas_per_sm(int d, int variant, int nmax, int mmax) { return ctas_any(d, variant, nmax, mmax); }

@@ -802,6 +802,10 @@ int batch_pick_variant(const BatchArgs& a, const int* h_order, cudaStream_t s);
 int batch_force_warps(int warps);  // 8 or 16 forces a CTA size, 0 returns to the tuned one; -1 if invalid
 std::string batch_tune_table();
 cudaError_t launch_batch(const BatchArgs& a, int variant, int grid, cudaStream_t s);
+// CTAs per problem (1, 2, 4 or 8) for problems of n[k] x m[k] points in queue order;
+// above 1 launch_batch_cluster runs the batch (16-warp CTAs in clusters)
+int batch_cluster(int d, int nmax, int mmax, const int* n, const int* m, const int* order, int nprob);
+cudaError_t launch_batch_cluster(const BatchArgs& a, int CL, cudaStream_t s);
 
 // Translation step for lam1 KL / lam2 KL penalties (uot_opts.translate; not
 // in the paper): per problem b, c_b = lam1 lam2 / (lam1 + lam2) (log A_b -

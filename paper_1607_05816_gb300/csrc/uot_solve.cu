@@ -912,15 +912,20 @@ uot_status uot_solve_batch(int nprob, const uot_batch_problem* probs, int d, con
   a.zV = d_zV;
   a.translate = o->translate;
   a.lam = d_lam;
-  const int variant = batch_pick_variant(a, order.data(), s);
-  const int per_sm = batch_ctas_per_sm(d, variant, nmax, mmax);
-  if (per_sm < 1) {
-    g_last_error = "uot_solve_batch: problem sizes do not fit in shared memory";
-    return UOT_EUNSUPPORTED;
+  const int CL = batch_cluster(d, nmax, mmax, hn.data(), hm.data(), order.data(), nprob);
+  if (CL > 1) {
+    UOT_CK(launch_batch_cluster(a, CL, s));
+  } else {
+    const int variant = batch_pick_variant(a, order.data(), s);
+    const int per_sm = batch_ctas_per_sm(d, variant, nmax, mmax);
+    if (per_sm < 1) {
+      g_last_error = "uot_solve_batch: problem sizes do not fit in shared memory";
+      return UOT_EUNSUPPORTED;
+    }
+    UOT_CK(cudaMemsetAsync(d_next, 0, sizeof(int), s));
+    const int grid = (int)std::min<int64_t>(nprob, (int64_t)sms * per_sm);
+    UOT_CK(launch_batch(a, variant, grid, s));
   }
-  UOT_CK(cudaMemsetAsync(d_next, 0, sizeof(int), s));
-  const int grid = (int)std::min<int64_t>(nprob, (int64_t)sms * per_sm);
-  UOT_CK(launch_batch(a, variant, grid, s));
   UOT_CK(cudaEventRecord(ev1, s));
   std::vector<int> it_h(nprob);
   std::vector<float> er_h(nprob);
