@@ -32,39 +32,14 @@
 
 #include <algorithm>
 
+#include "exp_table.cuh"
 #include "uot_internal.cuh"
 
 namespace uot {
 namespace {
 
-constexpr int kUnits = 256;                       // units per bit of the scaled exponents
-constexpr double kToUnits = 369.32993046757465;   // 256 / ln 2
-constexpr double kFromUnits = 0.0027076061740622863;  // ln 2 / 256
-constexpr double kMagic = 6755399441055744.0;     // 1.5 2^52: adding it rounds to an integer
-constexpr int kMaxUp = 900;                       // a term may be 2^900 times e^shift
 constexpr double kDrift = 300.0;                  // largest log weight before a new kernel
 constexpr double kLeastSum = 1e-150;
-
-// e^a; tab[k] = 2^(k/256)
-__device__ __forceinline__ double exp_tab(double a, const double* tab) {
-  const double t = fma(a, kToUnits, kMagic);  // kMagic + rint(a 256/ln 2)
-  const double r = fma(a, kToUnits, -(t - kMagic));  // |r| <= 1/2
-  const int hi = __double2hiint(t);
-  if ((hi >> 20) != 0x433) {               // 2^51 units or more, or not a number
-    if (t != t || hi > 0x43300000) return __longlong_as_double(0x7ff8000000000000ll);
-    return 0.0;
-  }
-  const long long n64 = __double_as_longlong(t) - __double_as_longlong(kMagic);
-  if (n64 < -1022 * kUnits) return 0.0;    // below the normal range
-  if (n64 > kMaxUp * kUnits) return __longlong_as_double(0x7ff8000000000000ll);  // the shift was no good
-  const int n = (int)n64;
-  constexpr double z = kFromUnits;
-  constexpr double z2 = z * z / 2, z3 = z * z * z / 6, z4 = z * z * z * z / 24;
-  const double p = r * fma(r, fma(r, fma(r, z4, z3), z2), z);  // 2^(r/256) - 1 to 4e-17
-  const double T = tab[n & (kUnits - 1)];
-  const double v = fma(T, p, T);
-  return __hiloint2double(__double2hiint(v) + ((n >> 8) << 20), __double2loint(v));
-}
 
 // The line L and its FP32 copy; with a stored kernel the weights e^{L - beta},
 // and *drift raised where one is too large or a point that had no mass when the
@@ -188,15 +163,10 @@ constexpr int kRowWarps = 8;
 
 // Row pass: a warp per row, then the CTA's epilogues (log, Table 1 row) side by
 // side in the lanes of one warp.
-__device__ __forceinline__ void fill_table(double* tab) {  // 256 threads
-  tab[threadIdx.x] = exp2((double)threadIdx.x / kUnits);
-  __syncthreads();
-}
-
 template <int D>
 __global__ void __launch_bounds__(kRowWarps * 32) points64_rows(Rows64 a, Epilogue epi) {
-  static_assert(kRowWarps * 32 == kUnits, "one table entry a thread");
-  __shared__ double tab[kUnits];
+  static_assert(kRowWarps * 32 == kExpUnits, "one table entry a thread");
+  __shared__ double tab[kExpUnits];
   __shared__ double sS[kRowWarps], sM[kRowWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * kRowWarps + warp;
@@ -228,7 +198,8 @@ __global__ void __launch_bounds__(kRowWarps * 32) points64_rows(Rows64 a, Epilog
     done = S >= kLeastSum && M != -kInf;  // (a NaN is recomputed and stays one)
   }
   if (__syncthreads_or(!done)) {  // block-uniform
-    fill_table(tab);
+    exp_table_load(tab);
+    __syncthreads();
     if (!done) {
       if (build) row64<D, true>(a, i, tab, S, M);
       else row64<D, false>(a, i, tab, S, M);
@@ -317,7 +288,7 @@ __global__ void __launch_bounds__(256) points64_cols_end(Rows64 a, const double*
                                                          const double* __restrict__ beta, int* __restrict__ drift,
                                                          Epilogue epi) {
   constexpr int kMaxF = 256;
-  __shared__ double tab[kUnits];
+  __shared__ double tab[kExpUnits];
   __shared__ double f[kMaxF], red[8][32], zc[32], smx[8];
   __shared__ unsigned bad_mask;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -366,7 +337,8 @@ __global__ void __launch_bounds__(256) points64_cols_end(Rows64 a, const double*
   }
   __syncthreads();
   if (bad_mask) {  // block-uniform
-    fill_table(tab);
+    exp_table_load(tab);
+    __syncthreads();
     for (int q = warp; q < 32; q += 8) {
       if (!((bad_mask >> q) & 1u)) continue;
       double S, M;

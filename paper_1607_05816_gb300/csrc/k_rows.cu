@@ -16,6 +16,7 @@
 
 #include <algorithm>
 
+#include "exp_table.cuh"
 #include "uot_internal.cuh"
 
 namespace uot {
@@ -36,13 +37,12 @@ __device__ __forceinline__ T wsum(T v) {
 }
 
 // L_j = W_j/eps + log w_j in FP64; then Lt_j = (L_j - max L) in T, scaled by
-// log2(e) for the FP32 variant.  Single block; *Lmax receives max L.  Lt32,
-// if given, receives an FP32 copy of the FP64 Lt (the prefilter's input).
+// log2(e) for the FP32 variant.  Single block; *Lmax receives max L.
 template <typename T, int NT>
 __global__ void __launch_bounds__(NT) prepare_L(const double* __restrict__ W,
                                                 const double* __restrict__ logw, int nin,
                                                 double eps, T* __restrict__ Lt,
-                                                double* __restrict__ Lmax, float* __restrict__ Lt32 = nullptr) {
+                                                double* __restrict__ Lmax) {
   __shared__ double red[NT / 32];
   const double inv_eps = 1.0 / eps;
   double mx = -kInf;
@@ -74,7 +74,6 @@ __global__ void __launch_bounds__(NT) prepare_L(const double* __restrict__ W,
     double v = (mx == -kInf) ? -kInf : L - mx;
     if (sizeof(T) == 4) v *= (double)kLog2e;
     Lt[j] = (T)v;
-    if (Lt32) Lt32[j] = (float)v;
   }
   if (threadIdx.x == 0) *Lmax = mx;
 }
@@ -148,283 +147,309 @@ __global__ void __launch_bounds__(WARPS * 32)
   if (epi.err) block_add2<WARPS * 32>(num, den, epi.err);
 }
 
-__device__ __forceinline__ void pdl_wait_prev() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_release_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// ---------------------------------------------------------------------------
+// FP64 rows of a dense cost by chunks of 32 columns.  GB300's FP64 pipe issues
+// 2 operations per clock per SM against 128 for FP32, and at small eps few
+// terms of a row matter.  Terms below e^-(50 + log nin) of the row's largest add
+// less than e^-50 = 2^-72 of the sum together and are left out, by conservative
+// FP32 tests: first per chunk, from the chunk's least cost (chunkmin32, built
+// once with the FP32 copy of C) and the largest input (prepare_L_chunks), then
+// per column on the FP32 copies.  What is left is evaluated in FP64, 32 terms at
+// a time with every lane active.
+//
+// A pass reads the row's least costs (1/32 of the FP32 cost) and the chunks that
+// matter, where the kernel before it read the whole FP32 cost (36 MB at
+// 3000 x 3000) into shared memory and kept every term above e^-746.  WF flow of
+// 3000 samples, eps = 1e-8: 28 -> 16 us a half-step (two kernels and the growth
+// step's share).  20 iterations, 3000 random points in 2-D: eps = 1e-1 16.4 -> 13.3
+// ms (FP64 terms: all of them count), 1e-2 16.4 -> 12.2, 1e-3 16.3 -> 4.4, 1e-4
+// 5.5 -> 2.4.
+// ---------------------------------------------------------------------------
 
-// Launch with programmatic dependent launch: the kernel may start while its
-// predecessor drains and waits for it (griddepcontrol.wait) before reading
-// anything the predecessor writes.
-template <typename Kern, typename... Args>
-cudaError_t launch_pdl(Kern kern, dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
-constexpr int kPfStageMax = 12288;  // inputs staged in shared memory (48 KB)
-constexpr int kPfPrepBlocks = 32;   // blocks of the prefilter's line preparation
-
-// Line preparation of the FP64 prefilter, spread over up to kPfPrepBlocks
-// blocks: L_j = W_j/eps + log w_j in FP64 (L64, for the surviving terms) and
-// as a float-float pair (Lff), and per-block maxima.  The last block to
-// finish (an atomic counter, no waiting) merges the maxima into *Lmax and
-// writes the shifted FP32 line Lt32_j = L_j - max L from the pairs with FP32
-// operations only (the FP64 pipe of one SM would take longer).  With merge =
-// 0 only L64 and Lff are written (any number of blocks): the consumer stages
-// the line and finds its maximum itself.
-__global__ void __launch_bounds__(256) prepare_L_pf(const double* __restrict__ W, const double* __restrict__ logw,
-                                                   int nin, double inv_eps, double* __restrict__ L64,
-                                                   float2* __restrict__ Lff, double* __restrict__ Lmax,
-                                                   float* __restrict__ Lt32, float* __restrict__ lerr,
-                                                   double* __restrict__ part, unsigned* __restrict__ count,
-                                                   int merge) {
-  __shared__ double red[8];
-  __shared__ bool last;
-  pdl_wait_prev();  // W is the preceding kernel's output
-  pdl_release_next();
-  double mx = -kInf;
-  for (int j = blockIdx.x * 256 + threadIdx.x; j < nin; j += gridDim.x * 256) {
-    const double w = W[j];
-    const double L = (w == -kInf) ? -kInf : fma(w, inv_eps, logw[j]);
-    L64[j] = L;
+// L_j = W_j/eps + log w_j in FP64 (L64) and as a float-float pair (Lff); the
+// largest L of each chunk of 32 columns as a pair (Lch).
+__global__ void __launch_bounds__(256) prepare_L_chunks(const double* __restrict__ W, const double* __restrict__ logw,
+                                                        int nin, double inv_eps, double* __restrict__ L64,
+                                                        float2* __restrict__ Lff, float2* __restrict__ Lch) {
+  pdl_wait();  // W is the preceding kernel's output
+  pdl_launch_dependents();
+  const int j = blockIdx.x * 256 + threadIdx.x;
+  auto pair = [](double L) {
     const float hi = (float)L;
-    Lff[j] = make_float2(hi, (L == -kInf) ? 0.0f : (float)(L - (double)hi));
-    mx = fmax(mx, L);
+    return make_float2(hi, (L == -kInf) ? 0.0f : (float)(L - (double)hi));
+  };
+  double L = -kInf;
+  if (j < nin) {
+    const double w = W[j];
+    L = (w == -kInf) ? -kInf : fma(w, inv_eps, logw[j]);
+    L64[j] = L;
+    Lff[j] = pair(L);
   }
-  if (!merge) return;
-  mx = wmax(mx);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int k = 1; k < 8; ++k) mx = fmax(mx, red[k]);
-    part[blockIdx.x] = mx;
-    __threadfence();
-    last = atomicAdd(count, 1u) == gridDim.x - 1;
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  if (threadIdx.x < 32) {  // gridDim.x <= 32 partials, one per lane
-    mx = (threadIdx.x < gridDim.x) ? __ldcg(&part[threadIdx.x]) : -kInf;
-    mx = wmax(mx);
-    if (threadIdx.x == 0) red[0] = mx;
-  }
-  __syncthreads();
-  mx = red[0];
-  const float mhi = (float)mx;
-  const float mlo = (mx == -kInf) ? 0.0f : (float)(mx - (double)mhi);
-#pragma unroll 4
-  for (int j = threadIdx.x; j < nin; j += 256) {
-    const float2 l = __ldcg(&Lff[j]);
-    Lt32[j] = (mx == -kInf || l.x == -INFINITY) ? -INFINITY : (l.x - mhi) + (l.y - mlo);
-  }
-  if (threadIdx.x == 0) {
-    *Lmax = mx;
-    // the pairs carry |L| 2^-47 of representation error besides the FP32 rounding
-    *lerr = (mx == -kInf) ? 4.0f : fmaf(fabsf(mhi), 0x1p-44f, 4.0f);
-    *count = 0u;
+  const double mx = wmax(L);
+  if ((threadIdx.x & 31) == 0 && j < nin) Lch[j >> 5] = pair(mx);
+}
+
+// C32 = C rounded to FP32 and the least C32 of each chunk; one warp per (row, chunk).
+__global__ void __launch_bounds__(256) chunkmin32(const double* __restrict__ C, int64_t nrows, int nin, int nchunk,
+                                                  float* __restrict__ C32, float* __restrict__ Cmin) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t t = blockIdx.x * (int64_t)8 + (threadIdx.x >> 5); t < nrows * nchunk; t += (int64_t)gridDim.x * 8) {
+    const int64_t i = t / nchunk;
+    const int j = (int)(t - i * nchunk) * 32 + lane;
+    float c = INFINITY;
+    if (j < nin) {
+      c = (float)C[i * nin + j];
+      C32[i * nin + j] = c;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) c = fminf(c, __shfl_xor_sync(0xffffffffu, c, o));
+    if (lane == 0) Cmin[t] = c;
   }
 }
 
-// FP64 rows of a dense cost with an FP32 prefilter.  GB300's FP64 pipe
-// issues 2 operations per clock per SM against 128 for FP32, and at small eps
-// most terms of a row underflow (e^a = 0 in FP64 for a < -745.2).  The max
-// sweep and a conservative skip test therefore run on FP32 copies of C and of
-// the shifted input line; the columns that can reach the FP64 range are
-// collected per warp (ballot, shared-memory list) and evaluated in FP64 32 at
-// a time with every lane active, shifted by the FP32 maximum (converted
-// exactly), so the result is the plain FP64 row sum up to FP64 rounding.  The
-// warps' leftover lists (< 32 each) are pooled per CTA and evaluated in full
-// batches too, and every sum is taken in a fixed order.  WPR warps share a row
-// (RPC rows per CTA) so that enough loads are in flight.
-template <int WPR, int RPC, bool kRows>
-__global__ void __launch_bounds__(WPR * RPC * 32)
-    rows_lse_f64_pf(const double* __restrict__ C, const float* __restrict__ C32, int nrows, int nin,
-                    const double* __restrict__ L64, const float* __restrict__ Lt32,
-                    const double* __restrict__ Lmax_p, const float* __restrict__ lerr_p,
-                    const float2* __restrict__ Lff, double k2, Epilogue epi) {
-  constexpr int NT = WPR * RPC * 32, NW = WPR * RPC;
-  // shared memory: the shifted FP32 input line (when it fits) and, with kRows,
-  // the CTA's RPC rows of C32, copied in with cp.async so that every byte is
-  // in flight at once and both sweeps read shared memory
-  extern __shared__ float sL[];
-  __shared__ float sm_m[RPC][WPR];
-  __shared__ double sm_s[RPC][WPR];
-  __shared__ double rsum[RPC];
-  __shared__ int slist[NW][64];
-  __shared__ int pool[NW * 32];     // leftover columns, warp by warp (so row by row)
-  __shared__ double pval[NW * 32];  // their FP64 terms
-  __shared__ int woff[NW + 1];      // exclusive prefix sum of the warps' leftover counts
-  __shared__ float sm_lm[NW];       // the warps' maxima of the line (kRows)
+// One warp per row, NW rows per CTA (rows b, b + G, ... of G CTAs: neighbouring
+// rows with hundreds of terms each, 12 us of one SM's FP64 pipe for ten of them,
+// go to different SMs).  The row's shift m is the largest exponent
+// of the chunk with the largest bound, then of any chunk whose bound lies more
+// than 30 above it, so every exponent stays below 30 plus the FP32 error.
+// Surviving columns are collected per warp (ballot, shared-memory list of
+// kRowList, drained 32 at a time when full); the lists are then evaluated by the
+// whole CTA, so a row with hundreds of terms among rows of five (the edge of a
+// density at small eps) does not wait for one warp's loads, and every sum is taken
+// in a fixed order.
+//
+// At small eps a pass is a chain of latencies and of FP64 instructions of one
+// warp, the CTA's epilogue (some 150 of 16 clocks each); 24 rows per CTA put one
+// epilogue on each SM where 8 put three (3000 rows).
+constexpr int kRowList = 352;
+
+// pval [NW][kRowList + 32], slist likewise, and the chunks' maxima
+template <int NW>
+size_t rows_chunks_smem(int nchunk) {
+  return (size_t)NW * (kRowList + 32) * (sizeof(double) + sizeof(int)) + (size_t)nchunk * sizeof(float);
+}
+
+template <int NW>
+__global__ void __launch_bounds__(NW * 32)
+    rows_lse_f64_chunks(const double* __restrict__ C, const float* __restrict__ C32, const float* __restrict__ Cmin,
+                        int nrows, int nin, int nchunk, const double* __restrict__ L64,
+                        const float2* __restrict__ Lff, const float2* __restrict__ Lch, double k2, float cut,
+                        Epilogue epi) {
+  constexpr int NT = NW * 32;
+  static_assert(NW <= 32 && NT >= kExpUnits, "a table entry a thread, a warp's lanes cover the rows");
+  extern __shared__ double pval[];  // the terms of the lists, row by row
+  int* slist = reinterpret_cast<int*>(pval + NW * (kRowList + 32));  // [NW][kRowList + 32] columns
+  float* sLc = reinterpret_cast<float*>(slist + NW * (kRowList + 32));  // [nchunk] largest input, relative to the line's
+  __shared__ float sm_m[NW];        // the rows' shifts
+  __shared__ double sm_s[NW];
+  __shared__ double sm_lmax;
+  __shared__ int woff[33];          // exclusive prefix sum of the list lengths
+  __shared__ double tab[kExpUnits];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rloc = warp / WPR, part = warp % WPR;
-  const int i = blockIdx.x * RPC + rloc;
-  double num = 0.0, den = 0.0;
-  const bool staged = kRows || nin <= kPfStageMax;
-  double Lmax;
-  float lerr;
-  if (kRows) {
-    // nin % 4 == 0 and 16-byte aligned C32: 16-byte copies of the rows (the cost does
-    // not depend on the preceding kernel, so they are issued before waiting for it)
-    const int q = nin >> 2;
-    const int nr = min(RPC, nrows - (int)blockIdx.x * RPC);
-    for (int t = threadIdx.x; t < q * nr; t += NT) {
-      const int r = t / q, c4 = t - r * q;
-      const float* src = C32 + ((int64_t)(blockIdx.x * RPC + r) * nin + 4 * c4);
-      const unsigned dst = (unsigned)__cvta_generic_to_shared(sL + (size_t)(r + 1) * nin + 4 * c4);
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    pdl_wait_prev();
-    pdl_release_next();
-    // the line from its float-float pairs: every CTA finds the same maximum
-    // (mhi, the FP32 rounding of max L, so Lmax = mhi exactly) and writes the
-    // shifted line Lt32_j = (hi_j - mhi) + lo_j with FP32 operations only
-    float mloc = -INFINITY;
-    for (int j = threadIdx.x; j < nin; j += NT) mloc = fmaxf(mloc, Lff[j].x);
-    mloc = wmax(mloc);
-    if (lane == 0) sm_lm[warp] = mloc;
-    __syncthreads();
-    float mhi = sm_lm[0];
+  const int i = blockIdx.x + warp * gridDim.x;
+  const float* cmin = Cmin + (int64_t)(i < nrows ? i : 0) * nchunk;
+  // before the preceding kernel has ended: the table and the least costs of the first 128 chunks
+  exp_table_load(tab);
+  float q4[4];
 #pragma unroll
-    for (int w = 1; w < NW; ++w) mhi = fmaxf(mhi, sm_lm[w]);
-    for (int j = threadIdx.x; j < nin; j += NT) {
-      const float2 l = Lff[j];
-      sL[j] = (mhi == -INFINITY || l.x == -INFINITY) ? -INFINITY : (l.x - mhi) + l.y;
-    }
-    Lmax = (mhi == -INFINITY) ? -kInf : (double)mhi;
-    // the pairs carry |L| 2^-47 of representation error besides the FP32 rounding
-    lerr = (mhi == -INFINITY) ? 4.0f : fmaf(fabsf(mhi), 0x1p-44f, 4.0f);
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-  } else {
-    pdl_wait_prev();
-    pdl_release_next();
-    if (staged)
-      for (int j = threadIdx.x; j < nin; j += NT) sL[j] = Lt32[j];
-    Lmax = *Lmax_p;
-    lerr = *lerr_p;
-  }
+  for (int u = 0; u < 4; ++u) q4[u] = (lane + 32 * u < nchunk) ? cmin[lane + 32 * u] : INFINITY;
+  pdl_wait();
+  pdl_launch_dependents();
+  // mhi: the FP32 rounding of max L (the shift of the whole line)
+  const float2 l0 = (threadIdx.x < nchunk) ? Lch[threadIdx.x] : make_float2(-INFINITY, 0.0f);
+  float mhi = l0.x;
+  for (int c = threadIdx.x + NT; c < nchunk; c += NT) mhi = fmaxf(mhi, Lch[c].x);
+  mhi = wmax(mhi);
+  if (lane == 0) sm_m[warp] = mhi;
   __syncthreads();
-  const float* L = staged ? sL : Lt32;
-  const bool live = i < nrows && Lmax != -kInf;  // warp-uniform
-  const int64_t rowbase = (int64_t)(live ? i : 0) * nin;
-  const float* crow = kRows ? sL + (size_t)(1 + rloc) * nin : C32 + rowbase;
+#pragma unroll
+  for (int w = 0; w < NW; ++w) mhi = fmaxf(mhi, sm_m[w]);
+  auto shifted = [&](float2 l) { return (mhi == -INFINITY || l.x == -INFINITY) ? -INFINITY : (l.x - mhi) + l.y; };
+  if (threadIdx.x < nchunk) sLc[threadIdx.x] = shifted(l0);
+  for (int c = threadIdx.x + NT; c < nchunk; c += NT) sLc[c] = shifted(Lch[c]);
+  if (threadIdx.x == 0) sm_lmax = (mhi == -INFINITY) ? -kInf : (double)mhi;  // (a conversion takes the FP64 pipe)
+  __syncthreads();
+  // the pairs carry |L| 2^-47 of representation error besides the FP32 rounding
+  const float lerr = (mhi == -INFINITY) ? 4.0f : fmaf(fabsf(mhi), 0x1p-44f, 4.0f);
   const float k2f = (float)k2;
-  float m = -INFINITY;
-  if (live) {
-#pragma unroll 4
-    for (int j = part * 32 + lane; j < nin; j += WPR * 32) m = fmaxf(m, fmaf(-k2f, crow[j], L[j]));
-  }
-  m = wmax(m);
-  if (lane == 0) sm_m[rloc][part] = m;
-  __syncthreads();
-  m = sm_m[rloc][0];
-#pragma unroll
-  for (int w = 1; w < WPR; ++w) m = fmaxf(m, sm_m[rloc][w]);
-  // FP64 term of column j of CTA row r, relative to that row's FP32 maximum
-  auto term = [&](int r, int j) {
-    const int64_t ri = (int64_t)(blockIdx.x * RPC + r);
-    float mr = sm_m[r][0];
-#pragma unroll
-    for (int w = 1; w < WPR; ++w) mr = fmaxf(mr, sm_m[r][w]);
-    const double a64 = fma(-k2, C[ri * nin + j], L64[j] - Lmax) - (double)mr;
-    return a64 > -746.0 ? exp(a64) : 0.0;
+  const bool live = i < nrows && mhi != -INFINITY;  // warp-uniform
+  const float* crow = C32 + (int64_t)(live ? i : 0) * nin;
+  // bound of chunk c = lane mod 32 and its FP32 error (the roundings of k2, c, l and the fma)
+  auto bound = [&](int c, float& tol) {
+    if (c >= nchunk) return -INFINITY;
+    const float l = sLc[c];
+    const float q = c < 64 ? (c < 32 ? q4[0] : q4[1]) : c < 128 ? (c < 96 ? q4[2] : q4[3]) : cmin[c];
+    const float b = fmaf(-k2f, q, l);
+    tol = fmaf(fabsf(b) + fmaf(k2f, fabsf(q), fabsf(l)), 0x1p-22f, lerr);
+    return b;
   };
-  double s = 0.0;
-  int cnt = 0;  // warp-uniform
-  int* lst = slist[warp];
-  if (live && m != -INFINITY) {
-    // warp-uniform sweep (the ballots need every lane)
-    for (int j0 = part * 32; j0 < nin; j0 += WPR * 32) {
-      const int j = j0 + lane;
-      bool keep = false;
-      if (j < nin) {
-        const float c = crow[j], l = L[j];
-        const float t = fmaf(-k2f, c, l);
-        const float a = t - m;
-        // |t - t_FP64| and the error of m are below (k2 c + |l| + |t| + |a|) 2^-22
-        // (the roundings of k2, c, l, the fma and the subtraction) plus lerr
-        const float tol = fmaf(fabsf(t) + fabsf(a) + fmaf(k2f, c, fabsf(l)), 0x1p-22f, lerr);
-        keep = a > -746.0f - tol;
+  // exponents of column j[u] (-inf where j[u] is none); every load is issued before the first
+  // is used (conditional loads wait for one another: 2.6 us for eight)
+  auto exponents = [&](auto& j, auto& t, auto& mag) {
+    constexpr int G = sizeof(j) / sizeof(int);
+    float cv[G];
+    float2 lv[G];
+#pragma unroll
+    for (int u = 0; u < G; ++u) {
+      const int q = (unsigned)j[u] < (unsigned)nin ? j[u] : 0;
+      cv[u] = crow[q];
+      lv[u] = Lff[q];
+    }
+#pragma unroll
+    for (int u = 0; u < G; ++u) {
+      const float l = shifted(lv[u]);
+      t[u] = (unsigned)j[u] < (unsigned)nin ? fmaf(-k2f, cv[u], l) : -INFINITY;
+      mag[u] = fmaf(k2f, fabsf(cv[u]), fabsf(l));
+    }
+  };
+  float m = -INFINITY, best = -INFINITY;
+  if (live) {
+    int jj[8];
+    float tt[8], mg[8];
+    auto largest = [&]() {
+      exponents(jj, tt, mg);
+      float g = tt[0];
+#pragma unroll
+      for (int u = 1; u < 8; ++u) g = fmaxf(g, tt[u]);
+      return wmax(g);
+    };
+    int at = 0;
+    for (int c = lane; c < nchunk; c += 32) {
+      float tol;
+      const float b = bound(c, tol);
+      if (b > best) {
+        best = b;
+        at = c;
       }
-      const unsigned mask = __ballot_sync(0xffffffffu, keep);
-      if (mask) {
-        if (keep) lst[cnt + __popc(mask & ((1u << lane) - 1u))] = j;
-        cnt += __popc(mask);
-        if (cnt >= 32) {  // a full batch: every lane evaluates one term
-          __syncwarp();
-          s += term(rloc, lst[lane]);
-          const int rest = cnt - 32;
-          const int carry = (lane < rest) ? lst[32 + lane] : 0;
-          __syncwarp();
-          if (lane < rest) lst[lane] = carry;
-          __syncwarp();
-          cnt = rest;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float b = __shfl_xor_sync(0xffffffffu, best, o);
+      const int c = __shfl_xor_sync(0xffffffffu, at, o);
+      if (b > best || (b == best && c < at)) {
+        best = b;
+        at = c;
+      }
+    }
+    if (best != -INFINITY) {
+      // that chunk and its neighbours: on a steep line over sorted points all bounds near the
+      // largest are loose, and the row's maximum lies a few chunks away
+#pragma unroll
+      for (int u = 0; u < 8; ++u) jj[u] = 32 * (at + u - 4) + lane;
+      m = largest();
+      for (int c0 = 0; c0 < nchunk; c0 += 32) {
+        float tol = 0.0f;
+        const float b = bound(c0 + lane, tol);
+        unsigned mask = __ballot_sync(0xffffffffu, b - tol > m + 30.0f);
+        while (mask) {  // eight chunks at a time for loads in flight
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            jj[u] = mask ? 32 * (c0 + __ffs(mask) - 1) + lane : nin;
+            mask &= mask - 1;  // 0 stays 0
+          }
+          m = fmaxf(m, largest());
         }
       }
     }
   }
-  if (__any_sync(0xffffffffu, s != 0.0)) s = wsum(s);  // most warps of a row hold no full batch
-  if (lane == 0) sm_s[rloc][part] = s;
-  // pool the leftovers (< 32 per warp) of the whole CTA in a fixed order (warp
-  // by warp, hence row by row), evaluate them 32 at a time, and sum each row's
-  // contiguous segment in a fixed order: the result does not depend on timing
-  if (lane == 0) woff[warp] = cnt;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int o = 0;
-    for (int w = 0; w < NW; ++w) {
-      const int c = woff[w];
-      woff[w] = o;
-      o += c;
+  // FP64 term of column j of CTA row r, relative to that row's shift mr
+  auto term = [&](int r, int j, float mr) {
+    const int64_t ri = (int64_t)(blockIdx.x + r * gridDim.x);
+    return exp_tab(fma(-k2, C[ri * nin + j], L64[j] - sm_lmax) - (double)mr, tab);
+  };
+  double s = 0.0;
+  bool drained = false;
+  int cnt = 0;  // warp-uniform
+  int* lst = slist + warp * (kRowList + 32);
+  if (live && m != -INFINITY) {
+    // warp-uniform sweep over the surviving chunks
+    constexpr int G = 4;
+    for (int c0 = 0; c0 < nchunk; c0 += 32) {
+      float ctol = 0.0f;
+      const float b = bound(c0 + lane, ctol);
+      const float a = b - m;
+      unsigned mask = __ballot_sync(0xffffffffu, a > -cut - fmaf(fabsf(a), 0x1p-22f, ctol));
+      while (mask) {
+        int cj[G];
+        float t[G], mag[G];
+#pragma unroll
+        for (int u = 0; u < G; ++u) {
+          cj[u] = mask ? 32 * (c0 + __ffs(mask) - 1) + lane : nin;
+          mask &= mask - 1;  // 0 stays 0
+        }
+        exponents(cj, t, mag);
+#pragma unroll
+        for (int u = 0; u < G; ++u) {
+          const float d = t[u] - m;
+          // |t - t_FP64| and the error of m are below (k2 c + |l| + |t| + |d|) 2^-22 plus lerr
+          const float tol = fmaf(fabsf(t[u]) + fabsf(d) + mag[u], 0x1p-22f, lerr);
+          const bool keep = cj[u] < nin && d > -cut - tol;
+          const unsigned km = __ballot_sync(0xffffffffu, keep);
+          if (!km) continue;
+          if (keep) lst[cnt + __popc(km & ((1u << lane) - 1u))] = cj[u];
+          cnt += __popc(km);
+          if (cnt > kRowList) {  // a full batch from the list's end: every lane evaluates one term
+            __syncwarp();
+            cnt -= 32;
+            s += term(warp, lst[cnt + lane], m);
+            drained = true;
+            __syncwarp();
+          }
+        }
+      }
     }
-    woff[NW] = o;
+  }
+  if (drained) s = wsum(s);
+  if (lane == 0) {
+    sm_m[warp] = m;  // (the maxima there were read before the last barrier)
+    sm_s[warp] = s;
+    woff[warp] = cnt;
   }
   __syncthreads();
-  __syncwarp();
-  if (lane < cnt) pool[woff[warp] + lane] = lst[lane];
+  if (warp == 0) {
+    const int c = lane < NW ? woff[lane] : 0;
+    int o = c;
+#pragma unroll
+    for (int k = 1; k < 32; k <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, o, k);
+      if (lane >= k) o += v;
+    }
+    woff[lane + 1] = o;  // (lanes from NW on repeat the total)
+    if (lane == 0) woff[0] = 0;
+  }
   __syncthreads();
   const int np = woff[NW];
-  for (int b = warp * 32; b < np; b += NT) {
-    const int k = b + lane;
-    if (k < np) {
-      int r = 0;
-      while (r + 1 < RPC && k >= woff[(r + 1) * WPR]) ++r;
-      pval[k] = term(r, pool[k]);
-    }
+  for (int k = threadIdx.x; k < np; k += NT) {
+    int r = 0;  // the last row that starts at or before k
+#pragma unroll
+    for (int h = 16; h > 0; h >>= 1)
+      if (r + h < NW && woff[r + h] <= k) r += h;
+    pval[k] = term(r, slist[r * (kRowList + 32) + k - woff[r]], sm_m[r]);
   }
   __syncthreads();
-  if (warp < RPC) {
+  // rows of more than kLaneTerms terms are summed by their warps, the others by the
+  // epilogue's lanes (a warp's sum takes five FP64 instructions whatever its length)
+  constexpr int kLaneTerms = 8;
+  if (cnt > kLaneTerms) {
     double t = 0.0;
-    for (int k = woff[warp * WPR] + lane; k < woff[(warp + 1) * WPR]; k += 32) t += pval[k];
+    for (int k = woff[warp] + lane; k < woff[warp + 1]; k += 32) t += pval[k];
     t = wsum(t);
-    if (lane == 0) rsum[warp] = t;
+    if (lane == 0) sm_s[warp] = s + t;
   }
   __syncthreads();
   // the CTA's row epilogues (FP64 log and Table 1 row) side by side in the
-  // lanes of warp 0: one warp instruction stream for RPC rows instead of one
+  // lanes of warp 0: one warp instruction stream for NW rows instead of one
   // per row on the narrow FP64 pipe
-  if (warp == 0 && lane < RPC) {
-    const int r = blockIdx.x * RPC + lane;
+  double num = 0.0, den = 0.0;
+  if (warp == 0 && lane < NW) {
+    const int r = blockIdx.x + lane * gridDim.x;
     if (r < nrows) {
       double z = -kInf;
-      float mr = sm_m[lane][0];
-      double sr = sm_s[lane][0] + rsum[lane];
-#pragma unroll
-      for (int w = 1; w < WPR; ++w) {
-        mr = fmaxf(mr, sm_m[lane][w]);
-        sr += sm_s[lane][w];
-      }
-      if (Lmax != -kInf && mr != -INFINITY) z = Lmax + (double)mr + log(sr);
+      const float mr = sm_m[lane];
+      double t = sm_s[lane];
+      if (woff[lane + 1] - woff[lane] <= kLaneTerms)
+        for (int k = woff[lane]; k < woff[lane + 1]; ++k) t += pval[k];
+      if (mr != -INFINITY) z = sm_lmax + (double)mr + log(t);
       apply_epilogue(epi, 0, r, z, num, den);
     }
   }
@@ -694,8 +719,17 @@ __global__ void __launch_bounds__(kAlg1Warps * 32) alg1_cluster(Alg1ClusterArgs 
 
 }  // namespace
 
-size_t rows_pf_scratch_bytes(int64_t nin) {
-  return 768 + 2 * (((size_t)nin * 8 + 255) & ~(size_t)255) + (((size_t)nin * 4 + 255) & ~(size_t)255);
+// L64 | Lff | Lch of prepare_L_chunks
+size_t rows_chunks_scratch_bytes(int64_t nin) {
+  return 2 * (((size_t)nin * 8 + 255) & ~(size_t)255) + ((size_t)rows_chunks(nin) * 8 + 255);
+}
+
+cudaError_t launch_chunkmin32(const double* C, int64_t nrows, int nin, float* C32, float* Cmin, cudaStream_t s) {
+  const int nchunk = (int)rows_chunks(nin);
+  count_launches(1);
+  chunkmin32<<<(unsigned)std::min<int64_t>((nrows * nchunk + 7) / 8, 152 * 64), 256, 0, s>>>(C, nrows, nin, nchunk, C32,
+                                                                                         Cmin);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_rows(int prec, const RowsGeom& g, int nrows, int nin, const double* W,
@@ -705,8 +739,7 @@ cudaError_t launch_rows(int prec, const RowsGeom& g, int nrows, int nin, const d
     return launch_points_ffp((const float*)g.x, (const float*)g.y, g.d, nrows, nin, W, logw, eps,
                              (float*)scratch_L, zprev, epi, s);
   // scratch_L: nin elements of the precision's type followed by one double
-  // (Lmax); the FP64 dense prefilter adds nin floats, block maxima and a
-  // counter (rows_pf_scratch_bytes).
+  // (Lmax); FP64 dense rows: rows_chunks_scratch_bytes.
   constexpr int WARPS = 8;
   const int grid = (nrows + WARPS - 1) / WARPS;
   if (g.kind == UOT_GEOM_POINTS && (g.d < 1 || g.d > 8)) return cudaErrorInvalidValue;
@@ -736,58 +769,31 @@ cudaError_t launch_rows(int prec, const RowsGeom& g, int nrows, int nin, const d
     double* Lt = (double*)scratch_L;
     double* Lmax = (double*)((char*)scratch_L + (((size_t)nin * 8 + 255) & ~(size_t)255));
     const double* C = (const double*)g.C;
-    // dense rows with an FP32 copy of C: FP32 prefilter (k2 = 1/eps must stay an FP32 number)
-    if (g.kind == UOT_GEOM_DENSE && g.C32 && 1.0 / eps < 1e30) {
-      // scratch: counter (zeroed by the caller) | block maxima [kPfPrepBlocks] | Lmax, lerr |
-      // L64 [nin] | Lff [nin] | Lt32 [nin]; the counter's place does not depend on nin
+    // dense rows with an FP32 copy of C (k2 = 1/eps must stay an FP32 number; the chunks'
+    // bounds, 48 KB for 393,216 columns, must fit in shared memory)
+    if (g.kind == UOT_GEOM_DENSE && g.C32 && 1.0 / eps < 1e30 && rows_chunks(nin) <= 12288) {
       char* base = (char*)scratch_L;
       const size_t r8 = ((size_t)nin * 8 + 255) & ~(size_t)255;
-      double* Lmx = (double*)(base + 512);
-      float* lerr = (float*)(base + 512 + 16);
-      double* L64 = (double*)(base + 768);
-      float2* Lff = (float2*)(base + 768 + r8);
-      float* Lt32 = (float*)(base + 768 + 2 * r8);
-      constexpr int WPR = 4, RPC = 4;
-      const int grid2 = (nrows + RPC - 1) / RPC;
-      // rows and line in shared memory: 16-byte rows (nin % 4 == 0) within 96 KB (opt-in
-      // above 48 KB); the rows kernel then finds the line's maximum itself
-      const size_t rows_bytes = (size_t)(1 + RPC) * nin * 4;
-      const bool rows_smem = (nin % 4 == 0) && rows_bytes <= 96 * 1024 && ((uintptr_t)g.C32 % 16 == 0);
-      const int pblk = rows_smem ? (nin + 255) / 256 : std::max(1, std::min(kPfPrepBlocks, (nin + 255) / 256));
-      cudaError_t e0 = launch_pdl(prepare_L_pf, dim3(pblk), dim3(256), 0, s, W, logw, nin, 1.0 / eps, L64, Lff,
-                                  Lmx, Lt32, lerr, (double*)(base + 256), (unsigned*)base, rows_smem ? 0 : 1);
-      if (e0 != cudaSuccess) return e0;
+      double* L64 = (double*)base;
+      float2* Lff = (float2*)(base + r8);
+      float2* Lch = (float2*)(base + 2 * r8);
+      const int nchunk = (int)rows_chunks(nin);
+      cudaError_t e = launch_pdl(prepare_L_chunks, dim3((nin + 255) / 256), dim3(256), 0, s, W, logw, nin, 1.0 / eps,
+                                 L64, Lff, Lch);
+      if (e != cudaSuccess) return e;
       prof_mark_begin(PROF_ROWS, s);
-      const float2* lff = Lff;
-      if (rows_smem) {
-        {  // opt-in for the current device: rows and line plus the static lists exceed 48 KB from
-           // about 1920 columns on
-          cudaError_t e = smem_at_least(rows_lse_f64_pf<WPR, RPC, true>, 96 * 1024);
-          if (e != cudaSuccess) return e;
-        }
-        const float* c32 = g.C32;
+      auto run = [&](auto kern, int nw) -> cudaError_t {
+        const size_t smem = nw == 8 ? rows_chunks_smem<8>(nchunk) : rows_chunks_smem<24>(nchunk);
+        const cudaError_t e0 = smem_at_least(kern, smem);
+        if (e0 != cudaSuccess) return e0;
         const double* l64 = L64;
-        const float* lt32 = Lt32;
-        const double* lmx = Lmx;
-        const float* le = lerr;
-        cudaError_t e1 = launch_pdl(rows_lse_f64_pf<WPR, RPC, true>, dim3(grid2), dim3(WPR * RPC * 32), rows_bytes, s,
-                                    C, c32, nrows, nin, l64, lt32, lmx, le, lff, 1.0 / eps, epi);
-        if (e1 != cudaSuccess) return e1;
-      } else {
-        const size_t smem = nin <= kPfStageMax ? (size_t)nin * 4 : 0;
-        if (smem > 48 * 1024) return cudaErrorInvalidValue;
-        // the line (up to 48 KB) and the static lists exceed the default 48 KB per block
-        cudaError_t ea = smem_at_least(rows_lse_f64_pf<WPR, RPC, false>, kPfStageMax * 4);
-        if (ea != cudaSuccess) return ea;
-        const float* c32 = g.C32;
-        const double* l64 = L64;
-        const float* lt32 = Lt32;
-        const double* lmx = Lmx;
-        const float* le = lerr;
-        cudaError_t e1 = launch_pdl(rows_lse_f64_pf<WPR, RPC, false>, dim3(grid2), dim3(WPR * RPC * 32), smem, s,
-                                    C, c32, nrows, nin, l64, lt32, lmx, le, lff, 1.0 / eps, epi);
-        if (e1 != cudaSuccess) return e1;
-      }
+        const float2 *lff = Lff, *lch = Lch;
+        return launch_pdl(kern, dim3((nrows + nw - 1) / nw), dim3(nw * 32), smem, s, C, g.C32,
+                          g.Cmin, nrows, nin, nchunk, l64, lff, lch, 1.0 / eps, 50.0f + logf((float)nin), epi);
+      };
+      // rows beyond one 8-row CTA per SM: 24 per CTA (fewer epilogues)
+      e = nrows <= 8 * 152 ? run(&rows_lse_f64_chunks<8>, 8) : run(&rows_lse_f64_chunks<24>, 24);
+      if (e != cudaSuccess) return e;
       prof_mark_end(PROF_ROWS, s);
       return cudaGetLastError();
     }

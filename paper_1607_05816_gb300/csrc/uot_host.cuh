@@ -774,7 +774,8 @@ struct Gibbs {
   int prec;
   size_t esz;
   const void* CT = nullptr;     // dense: C^T in the precision's type
-  float* C32[2] = {nullptr, nullptr};  // dense FP64: FP32 copies of C, C^T (row prefilter)
+  float* C32[2] = {nullptr, nullptr};   // dense FP64: FP32 copies of C, C^T ...
+  float* Cmin[2] = {nullptr, nullptr};  // ... and their least values per row and chunk of 32 columns
   double* pass[2] = {nullptr, nullptr};  // grid intermediates
   // FP64 grids: the stored kernel of each (direction, axis) pass and the eps it
   // was built for (k_grid_fac.cu); NULL: that pass runs plain log-sum-exps
@@ -815,7 +816,10 @@ struct Gibbs {
     esz = (prec == UOT_F64) ? 8 : 4;
     if (g.kind == UOT_GEOM_DENSE) sc.reserve<char>((size_t)g.n * g.m * esz);
     if (g.kind == UOT_GEOM_DENSE && prec == UOT_F64) {
-      for (int k = 0; k < 2; ++k) sc.reserve<float>((size_t)g.n * g.m);
+      for (int k = 0; k < 2; ++k) {
+        sc.reserve<float>((size_t)g.n * g.m);
+        sc.reserve<float>(chunkmin_elems(k));
+      }
       sc.reserve<int>(1);
     }
     if (g.kind == UOT_GEOM_GRID) {
@@ -883,9 +887,13 @@ struct Gibbs {
     return g.kind == UOT_GEOM_POINTS && prec != UOT_F64 && g.d <= 3 && points_chunks_fit(g.n) &&
            points_chunks_fit(g.m);
   }
-  // shifted input line (+ Lmax) and, for FP64 dense rows, its FP32 copy
+  size_t chunkmin_elems(int dir) const {
+    return dir == 0 ? (size_t)(g.n * rows_chunks(g.m)) : (size_t)(g.m * rows_chunks(g.n));
+  }
+  // shifted input line (+ Lmax); FP64 dense rows: the line and its chunks' maxima
   size_t lscratch_bytes(int64_t mx) const {
-    if (g.kind == UOT_GEOM_DENSE && prec == UOT_F64) return std::max((size_t)mx * 8 + 512, rows_pf_scratch_bytes(mx));
+    if (g.kind == UOT_GEOM_DENSE && prec == UOT_F64)
+      return std::max((size_t)mx * 8 + 512, rows_chunks_scratch_bytes(mx));
     return (size_t)mx * 8 + 512;
   }
   size_t part_elems() const {
@@ -904,10 +912,12 @@ struct Gibbs {
       CT = ct;
       if (prec == UOT_F64) {
         const int64_t nm = (int64_t)g.n * g.m;
-        C32[0] = sc.take<float>((size_t)nm);
-        C32[1] = sc.take<float>((size_t)nm);
+        for (int k = 0; k < 2; ++k) {
+          C32[k] = sc.take<float>((size_t)nm);
+          Cmin[k] = sc.take<float>(chunkmin_elems(k));
+        }
         int* dflag = sc.take<int>(1);
-        if (!C32[0] || !C32[1] || !dflag) return cudaErrorInvalidValue;
+        if (!Cmin[0] || !Cmin[1] || !dflag) return cudaErrorInvalidValue;
         // a symmetric cost (X = Y, e.g. the WF flows) serves both directions from
         // one copy: half the working set, which then stays in L2
         bool sym = false;
@@ -921,15 +931,15 @@ struct Gibbs {
           if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
           sym = (h == 0);
         }
-        count_launches(1);
-        k_from_f64<float><<<nblocks(nm), kNT, 0, s>>>((const double*)g.C, nm, C32[0]);
+        cudaError_t ec = launch_chunkmin32((const double*)g.C, g.n, g.m, C32[0], Cmin[0], s);
         if (sym) {
           CT = g.C;
           C32[1] = C32[0];
-        } else {
-          count_launches(1);
-          k_from_f64<float><<<nblocks(nm), kNT, 0, s>>>((const double*)CT, nm, C32[1]);
+          Cmin[1] = Cmin[0];
+        } else if (ec == cudaSuccess) {
+          ec = launch_chunkmin32((const double*)CT, g.m, g.n, C32[1], Cmin[1], s);
         }
+        if (ec != cudaSuccess) return ec;
       }
     }
     if (g.kind == UOT_GEOM_GRID) {
@@ -1039,11 +1049,6 @@ struct Gibbs {
             p64.K = (double*)sc.try_extra((size_t)g.n * points64_ld(g.m) * sizeof(double));
           }
         }
-      }
-      if (g.kind == UOT_GEOM_DENSE && prec == UOT_F64) {
-        // the prefilter's block counter (first bytes of the scratch)
-        cudaError_t e0 = cudaMemsetAsync(Lscratch, 0, 256, s);
-        if (e0 != cudaSuccess) return e0;
       }
       if (points_fast()) {
         part = sc.take<float2>(part_elems());
@@ -1184,6 +1189,7 @@ struct Gibbs {
     rg.d = g.d;
     rg.C = (dir == 0) ? g.C : CT;
     rg.C32 = C32[dir];
+    rg.Cmin = Cmin[dir];
     rg.x = (dir == 0) ? g.x : g.y;
     rg.y = (dir == 0) ? g.y : g.x;
     const int nrows = (dir == 0) ? g.n : g.m;

@@ -505,6 +505,25 @@ template <typename K>
 cudaError_t smem_at_least(K* kernel, size_t bytes) {
   return smem_limit_at_least(reinterpret_cast<const void*>(kernel), bytes);
 }
+
+// Launch with programmatic dependent launch: the kernel may start while its
+// predecessor drains; it waits for it (pdl_wait) before reading anything the
+// predecessor writes.
+template <typename Kern, typename... Args>
+cudaError_t launch_pdl(Kern kern, dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
 void prof_mark_begin(int family, cudaStream_t s);
 void prof_mark_end(int family, cudaStream_t s);
 
@@ -711,7 +730,8 @@ struct RowsGeom {
   const void* x;     // points [nrows*d]
   const void* y;     // points [nin*d]
   int d;
-  const float* C32;  // dense FP64: FP32 copy of C for the row kernel's prefilter (NULL: none)
+  const float* C32;   // dense FP64: FP32 copy of C for the row kernel's tests (NULL: none)
+  const float* Cmin;  // ... and its least value per row and chunk of 32 columns
 };
 // FP32 point clouds with d <= 3 and a `part` buffer use the chunked kernels of
 // k_points.cu (zprev: previous results used as log-sum-exp shifts).
@@ -726,9 +746,12 @@ cudaError_t launch_rows(int prec, const RowsGeom& g, int nrows, int nin, const d
 cudaError_t launch_points_ffp(const float* x, const float* y, int d, int nout, int nin, const double* W,
                               const double* logw, double eps, float* bmax, float* zprev, const Epilogue& epi,
                               cudaStream_t s);
-// Scratch of launch_rows for FP64 dense rows with the FP32 prefilter; its
-// first 4 bytes hold a counter that must be zero before the first launch.
-size_t rows_pf_scratch_bytes(int64_t nin);
+// FP64 dense rows by chunks of 32 columns (k_rows.cu): chunks of a row, scratch
+// of launch_rows, and the set-up of RowsGeom's C32 [nrows][nin] and Cmin
+// [nrows][chunks] from a cost C [nrows][nin].
+inline int64_t rows_chunks(int64_t nin) { return (nin + 31) / 32; }
+size_t rows_chunks_scratch_bytes(int64_t nin);
+cudaError_t launch_chunkmin32(const double* C, int64_t nrows, int nin, float* C32, float* Cmin, cudaStream_t s);
 // FP64 point clouds (k_points64.cu).  K NULL: on the fly in both directions.
 struct Points64 {
   const double* x;     // [n][d]
