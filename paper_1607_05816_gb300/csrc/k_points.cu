@@ -7,15 +7,23 @@
 //    shifted log-values t_j and coordinates are staged in shared memory as
 //    packed pairs; each warp owns 128 outputs (4 per lane, two f32x2 pairs) and
 //    sweeps the chunk.  The log-sum-exp shift of an output is its result from
-//    the previous call at the same eps; a warp whose partial sum overflows
-//    redoes the chunk with the exact chunk maximum.  Writes (shift, sum) per
-//    (chunk, output).
-//  points_combine: one warp per output merges the chunks' pairs; if the
-//    merged sum underflowed (shift far above the result) the warp recomputes
+//    the previous call, scaled by the ratio of the two eps (the potential eps z
+//    moves little from one eps to the next; without it the first pass of every
+//    eps needs a second sweep for the maxima, 22 of the 80 passes of a solve of
+//    10 stages); a warp whose partial sum overflows redoes the chunk with the
+//    exact chunk maximum.  Writes (shift, sum) per (chunk, output).
+//  points_combine: one thread per output merges the chunks' pairs; where the
+//    merged sum underflowed (shift far above the result) a warp recomputes
 //    that output exactly over all inputs; then the epilogue (Table 1 row,
-//    violation terms) runs on the float-float result.
+//    violation terms) runs on the float-float result, 32 outputs a warp.
 //
-// Work: n m exponentials per call, bound by the SFU rate.
+// points_blockmax and points_combine are launched while their predecessors run
+// (programmatic dependent launch).
+// Work: n m terms per call, in three dimensions 9 FP32-pipe operations and one
+// exponential each, bound by the FP32 pipe.  20000 x 20000 points in 3-D: 118 us a
+// sweep (96 us at the pipe's rate), 127 us a pass; a solve of 40 iterations over 11
+// eps 13.4 -> 10.6 ms with the shifts carried from eps to eps, one thread per
+// output in the merge and the overlapped launches.
 #include <string.h>
 
 #include "uot_internal.cuh"
@@ -43,6 +51,8 @@ __global__ void __launch_bounds__(256)
     points_blockmax(const float2* __restrict__ W, const float2* __restrict__ lw, int nin,
                     float2 inv_eps, float* __restrict__ bmax) {
   __shared__ float red[8];
+  pdl_wait();
+  pdl_launch_dependents();
   float m = -INFINITY;
   const int j0 = blockIdx.x * kMaxBlk;
   for (int j = j0 + threadIdx.x; j < min(nin, j0 + kMaxBlk); j += 256) m = fmaxf(m, load_L_pt(W, lw, j, inv_eps).hi);
@@ -73,7 +83,7 @@ struct PtArgs {
   const float* bmax;  // [nbmax] block maxima of L
   float k2;           // log2(e)/eps
   const float* zprev; // [nout] previous result (natural log), or NULL
-  int use_prev;
+  float zscale;       // shift = zprev * zscale; 0: exact maxima
   float2* part;       // [nchunks][nout] (shift, sum) in log2 units relative to Lmax
 };
 
@@ -86,6 +96,8 @@ __global__ void __launch_bounds__(kNW * 32)
   const int j0 = c * a.chunk, j1 = min(a.nin, j0 + a.chunk);
   constexpr int d = D;  // compile-time: no dimension tests in the sweeps
   const float k2 = a.k2;
+  pdl_wait();
+  pdl_launch_dependents();
   const float Lmax = all_max(a.bmax, a.nbmax);
   for (int j = j0 + tid; j < j1; j += kNW * 32) {
     const ff L = load_L_pt(a.W, a.lw, j, a.inv_eps);
@@ -114,12 +126,12 @@ __global__ void __launch_bounds__(kNW * 32)
   const f2p nk2 = pk(-k2, -k2);
   const int nj = j1 - j0;
   float mq[4], sq[4];
-  bool exact = !(a.use_prev && a.zprev);
+  bool exact = !(a.zscale > 0.0f && a.zprev);
   if (!exact) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const float zp = valid[q] ? a.zprev[base + lane + 32 * q] : Lmax;
-      mq[q] = (zp == -INFINITY) ? 0.0f : (zp - Lmax) * kLog2e;
+      const float zp = valid[q] ? a.zprev[base + lane + 32 * q] : -INFINITY;
+      mq[q] = (zp == -INFINITY) ? 0.0f : (zp * a.zscale - Lmax) * kLog2e;
     }
   }
   for (int attempt = 0; attempt < 2; ++attempt) {
@@ -214,65 +226,72 @@ struct CombArgs {
   float* zprev;  // written (NULL: not kept)
 };
 
-// One warp per output: merge chunk partials, exact recomputation if the
-// merged sum underflowed, then the epilogue.
-__global__ void __launch_bounds__(256)
+// One thread per output: merge chunk partials, exact recomputation (by the
+// thread's warp) if the merged sum underflowed, then the epilogue.
+constexpr int kCombThreads = 128;
+
+__global__ void __launch_bounds__(kCombThreads)
     points_combine(CombArgs a, Epilogue epi) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = blockIdx.x * 8 + warp;
+  const int lane = threadIdx.x & 31;
+  const int i = blockIdx.x * kCombThreads + threadIdx.x;
+  const bool owns = i < a.nout;
   float num = 0.0f, den = 0.0f;
+  pdl_wait();
+  pdl_launch_dependents();
   const float Lmax = all_max(a.bmax, a.nbmax);
-  if (i < a.nout) {
-    float M = -INFINITY;
-    for (int c = lane; c < a.nchunks; c += 32) {
+  float M = -INFINITY, S = 0.0f;
+  if (owns) {
+#pragma unroll 4
+    for (int c = 0; c < a.nchunks; ++c) {
       const float2 pr = a.part[(int64_t)c * a.nout + i];
       if (pr.y > 0.0f) M = fmaxf(M, pr.x);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-    float S = 0.0f;
-    if (M != -INFINITY)
-      for (int c = lane; c < a.nchunks; c += 32) {
+    if (M != -INFINITY) {
+#pragma unroll 4
+      for (int c = 0; c < a.nchunks; ++c) {
         const float2 pr = a.part[(int64_t)c * a.nout + i];
         if (pr.y > 0.0f) S += pr.y * ex2_approx(pr.x - M);
       }
+    }
+  }
+  // the shift was far above the result: exact log-sum-exp over all inputs
+  unsigned redo = __ballot_sync(0xffffffffu, owns && !(S >= 0x1p-90f) && Lmax != -INFINITY);
+  for (; redo; redo &= redo - 1) {
+    const int src = __ffs(redo) - 1;
+    const int io = i - lane + src;
+    float xi[3];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) S += __shfl_xor_sync(0xffffffffu, S, o);
-    if (!(S >= 0x1p-90f) && Lmax != -INFINITY) {
-      // the shift was far above the result: exact log-sum-exp over all inputs
-      float xi[3];
+    for (int k = 0; k < 3; ++k) xi[k] = (k < a.d) ? a.x[(int64_t)io * a.d + k] : 0.0f;
+    auto arg = [&](int j) -> float {
+      const ff L = load_L_pt(a.W, a.lw, j, a.inv_eps);
+      if (L.hi == -INFINITY) return -INFINITY;
+      float q = 0.0f;
+      for (int k = 0; k < a.d; ++k) {
+        const float t = xi[k] - a.y[(int64_t)j * a.d + k];
+        q = fmaf(t, t, q);
+      }
+      return fmaf(-a.k2, q, ((L.hi - Lmax) + L.lo) * kLog2e);
+    };
+    float m = -INFINITY;
+    for (int j = lane; j < a.nin; j += 32) m = fmaxf(m, arg(j));
+    m = warp_maxf(m);
+    float s = 0.0f;
+    if (m != -INFINITY)
+      for (int j = lane; j < a.nin; j += 32) s += ex2_approx(arg(j) - m);
 #pragma unroll
-      for (int k = 0; k < 3; ++k) xi[k] = (k < a.d) ? a.x[(int64_t)i * a.d + k] : 0.0f;
-      auto arg = [&](int j) -> float {
-        const ff L = load_L_pt(a.W, a.lw, j, a.inv_eps);
-        if (L.hi == -INFINITY) return -INFINITY;
-        float q = 0.0f;
-        for (int k = 0; k < a.d; ++k) {
-          const float t = xi[k] - a.y[(int64_t)j * a.d + k];
-          q = fmaf(t, t, q);
-        }
-        return fmaf(-a.k2, q, ((L.hi - Lmax) + L.lo) * kLog2e);
-      };
-      float m = -INFINITY;
-      for (int j = lane; j < a.nin; j += 32) m = fmaxf(m, arg(j));
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      float s = 0.0f;
-      if (m != -INFINITY)
-        for (int j = lane; j < a.nin; j += 32) s += ex2_approx(arg(j) - m);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == src) {
       M = m;
       S = s;
     }
-    if (lane == 0) {
-      ff z = ff_ninf();
-      if (Lmax != -INFINITY && M != -INFINITY && S > 0.0f) z = pass_result(Lmax, M, S);
-      if (a.zprev) a.zprev[i] = z.hi;
-      apply_epilogue_ff(epi, 0, i, z, num, den);
-    }
   }
-  if (epi.err) block_add2f<256>(num, den, epi.err);
+  if (owns) {
+    ff z = ff_ninf();
+    if (Lmax != -INFINITY && M != -INFINITY && S > 0.0f) z = pass_result(Lmax, M, S);
+    if (a.zprev) a.zprev[i] = z.hi;
+    apply_epilogue_ff(epi, 0, i, z, num, den);
+  }
+  if (epi.err) block_add2f<kCombThreads>(num, den, epi.err);
 }
 
 // ---------------------------------------------------------------------------
@@ -429,7 +448,7 @@ int points_nchunks(int nin, int nout) {
 
 cudaError_t launch_points(const float* x, const float* y, int d, int nout, int nin,
                           const double* W, const double* logw, double eps, float* bmax,
-                          float* zprev, int use_prev, float2* part, const Epilogue& epi,
+                          float* zprev, float zscale, float2* part, const Epilogue& epi,
                           cudaStream_t s) {
   const int nchunks = points_nchunks(nin, nout);
   const int chunk = (nin + nchunks - 1) / nchunks;
@@ -439,7 +458,8 @@ cudaError_t launch_points(const float* x, const float* y, int d, int nout, int n
   const float2* lwf = reinterpret_cast<const float2*>(logw);
   prof_mark_begin(PROF_ROWS, s);
   count_launches(3);
-  points_blockmax<<<nbmax, 256, 0, s>>>(Wf, lwf, nin, inv_eps, bmax);
+  cudaError_t e = launch_pdl(points_blockmax, dim3(nbmax), dim3(256), 0, s, Wf, lwf, nin, inv_eps, bmax);
+  if (e != cudaSuccess) return e;
   PtArgs a;
   a.x = x;
   a.y = y;
@@ -454,17 +474,20 @@ cudaError_t launch_points(const float* x, const float* y, int d, int nout, int n
   a.bmax = bmax;
   a.k2 = (float)((double)kLog2e / eps);
   a.zprev = zprev;
-  a.use_prev = use_prev;
+  a.zscale = zscale;
   a.part = part;
   const size_t smem = (size_t)2 * chunk * sizeof(float4);
   dim3 grid((nout + kOutBlk - 1) / kOutBlk, nchunks);
   auto run = [&](auto kern) -> cudaError_t {
     cudaError_t e = smem_at_least(kern, smem);
     if (e != cudaSuccess) return e;
+    // launched when the block maxima are done, on an idle GPU: launched early
+    // (programmatically), its CTAs go where blockmax leaves room, four on some SMs instead of
+    // at most three (20000 x 20000 points: 154 us against 118)
     kern<<<grid, kNW * 32, smem, s>>>(a);
     return cudaGetLastError();
   };
-  cudaError_t e = (d == 1) ? run(points_partial<1>) : (d == 2) ? run(points_partial<2>) : run(points_partial<3>);
+  e = (d == 1) ? run(&points_partial<1>) : (d == 2) ? run(&points_partial<2>) : run(&points_partial<3>);
   if (e != cudaSuccess) return e;
   CombArgs b;
   b.x = x;
@@ -481,7 +504,8 @@ cudaError_t launch_points(const float* x, const float* y, int d, int nout, int n
   b.k2 = a.k2;
   b.part = part;
   b.zprev = zprev;
-  points_combine<<<(nout + 7) / 8, 256, 0, s>>>(b, epi);
+  e = launch_pdl(points_combine, dim3((nout + kCombThreads - 1) / kCombThreads), dim3(kCombThreads), 0, s, b, epi);
+  if (e != cudaSuccess) return e;
   prof_mark_end(PROF_ROWS, s);
   return cudaGetLastError();
 }

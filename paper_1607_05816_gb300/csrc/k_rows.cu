@@ -734,7 +734,7 @@ cudaError_t launch_chunkmin32(const double* C, int64_t nrows, int nin, float* C3
 
 cudaError_t launch_rows(int prec, const RowsGeom& g, int nrows, int nin, const double* W,
                         const double* logw, double eps, void* scratch_L, const Epilogue& epi,
-                        cudaStream_t s, float* zprev, int use_prev, void* part, int precise) {
+                        cudaStream_t s, float* zprev, float zscale, void* part, int precise) {
   if ((precise || precise_forced()) && prec == UOT_F32 && g.kind == UOT_GEOM_POINTS && g.d <= 3)
     return launch_points_ffp((const float*)g.x, (const float*)g.y, g.d, nrows, nin, W, logw, eps,
                              (float*)scratch_L, zprev, epi, s);
@@ -748,7 +748,7 @@ cudaError_t launch_rows(int prec, const RowsGeom& g, int nrows, int nin, const d
     // chunked point-cloud kernels; scratch_L holds the block maxima
     count_launches(-2);
     return launch_points((const float*)g.x, (const float*)g.y, g.d, nrows, nin, W, logw, eps,
-                         (float*)scratch_L, zprev, use_prev, reinterpret_cast<float2*>(part), epi, s);
+                         (float*)scratch_L, zprev, zscale, reinterpret_cast<float2*>(part), epi, s);
   }
   if (prec == UOT_F32) {
     float* Lt = (float*)scratch_L;

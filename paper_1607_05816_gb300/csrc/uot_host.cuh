@@ -1211,10 +1211,13 @@ struct Gibbs {
         if (dir == 0 && p64.K) p64_eps = eps;
         continue;
       }
-      const int use_prev = (nbatch == 1 && zrow[dir] != nullptr && zeps[dir] == eps) ? 1 : 0;
+      // shifts from this direction's previous result, also across one step of an
+      // eps schedule (ratios of 1.2 to 2; beyond 4 the potentials move too far)
+      const double ratio = zeps[dir] / eps;
+      const float zscale = (nbatch == 1 && zrow[dir] && ratio >= 1.0 && ratio <= 4.0) ? (float)ratio : 0.0f;
       cudaError_t err = launch_rows(prec == UOT_F64 ? UOT_F64 : UOT_F32, rg, nrows, nin,
                                     W + (int64_t)b * nin, logw, eps, Lscratch, e, s,
-                                    nbatch == 1 ? zrow[dir] : nullptr, use_prev, part, precise ? 1 : 0);
+                                    nbatch == 1 ? zrow[dir] : nullptr, zscale, part, precise ? 1 : 0);
       if (err != cudaSuccess) return err;
     }
     if (zrow[dir] && nbatch == 1) zeps[dir] = eps;

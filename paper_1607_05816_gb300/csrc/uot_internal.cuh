@@ -734,12 +734,13 @@ struct RowsGeom {
   const float* Cmin;  // ... and its least value per row and chunk of 32 columns
 };
 // FP32 point clouds with d <= 3 and a `part` buffer use the chunked kernels of
-// k_points.cu (zprev: previous results used as log-sum-exp shifts).
+// k_points.cu (zprev: previous results, times zscale the log-sum-exp shifts;
+// zscale 0: no use of them).
 // precise = 1 (FP32 point clouds, d <= 3): the pass with float-float
 // exponents (launch_points_ffp) instead of the chunked kernels.
 cudaError_t launch_rows(int prec, const RowsGeom& g, int nrows, int nin, const double* W,
                         const double* logw, double eps, void* scratch_L, const Epilogue& epi,
-                        cudaStream_t s, float* zprev = nullptr, int use_prev = 0,
+                        cudaStream_t s, float* zprev = nullptr, float zscale = 0.0f,
                         void* part = nullptr, int precise = 0);
 // FP32 point clouds (d <= 3), exponents in float-float (k_points.cu); bmax
 // holds ceil(nin / 1024) floats.
@@ -780,7 +781,7 @@ int points_nchunks(int nin, int nout);
 bool points_chunks_fit(int nin);
 cudaError_t launch_points(const float* x, const float* y, int d, int nout, int nin,
                           const double* W, const double* logw, double eps, float* bmax,
-                          float* zprev, int use_prev, float2* part, const Epilogue& epi,
+                          float* zprev, float zscale, float2* part, const Epilogue& epi,
                           cudaStream_t s);
 
 // Persistent batched solver for many point-cloud problems (k_batch.cu).
