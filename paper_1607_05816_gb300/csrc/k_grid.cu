@@ -293,6 +293,256 @@ __global__ void __launch_bounds__(NW * 32, NW == 1 ? 16 : 32 / NW)
   if (epi.err) block_add2f<NW * 32>(num, den, epi.err + 2 * (int64_t)blockIdx.z);
 }
 
+// Four lines per CTA: 4 consecutive lines x (32 * OPL) outputs, the contraction
+// index split over the NW warps as above.  Two things bound the one-line CTA where
+// there are many lines.  The result is stored transposed (point i*nlines + l), so
+// its epilogue uses 8 bytes of every 32-byte sector that it touches (old and new
+// potential, log density, shifts); here the epilogue's threads run over the lines
+// first and use whole sectors.  And of the 5 FP32-pipe operations of a term two,
+// the squared distance, do not depend on the line: a warp computes them once for
+// its 4 lines (3.5 operations a term; the exponential, 32 a clock and SM, becomes
+// the bound).  Arithmetic and summation order are grid_pass_f32's.
+constexpr int kMlLines = 4;
+
+template <int NW, int OPL>
+struct MlTile {
+  static constexpr int kOut = 32 * OPL;
+  static constexpr int kThreads = 32 * NW;
+  static constexpr int kOwn = (kMlLines * kOut + kThreads - 1) / kThreads;
+  static_assert(NW % kMlLines == 0, "whole warps per line in the loading phase");
+  static constexpr int kWarpsPerLine = NW / kMlLines;
+  static constexpr int kLineRegs = 4;
+  // partial sums of a line; 4 float2 of padding put the lines 8 banks apart
+  static constexpr int kPartStride = NW * kOut + 4;
+  static size_t smem(int nin) {
+    return (size_t)nin * (sizeof(float4) + sizeof(float2)) +
+           (size_t)kMlLines * (kPartStride * sizeof(float2) + kOut * sizeof(float));
+  }
+};
+
+template <int NW, int OPL>
+__global__ void __launch_bounds__(MlTile<NW, OPL>::kThreads, (OPL == 4 ? 24 : 32) / NW)
+    grid_pass_f32_ml(PassArgs a, Epilogue epi) {
+  typedef MlTile<NW, OPL> T;
+  constexpr int NL = kMlLines, OUT = T::kOut, NT = T::kThreads, WPL = T::kWarpsPerLine, OWN = T::kOwn,
+                LR = T::kLineRegs, P = OPL / 2;
+  extern __shared__ float4 sml[];  // [nin] the lines' values at j
+  __shared__ float sred[NL][WPL];
+  const int nin = a.nin, nout = a.nout, nlines = a.nlines;
+  float2* sy = reinterpret_cast<float2*>(sml + nin);                             // [nin] {y, y}
+  float2* part = sy + nin;                                                       // [NL][kPartStride]
+  float* sshift = reinterpret_cast<float*>(part + (size_t)NL * T::kPartStride);  // [NL][OUT]
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int i0 = blockIdx.x * OUT, l0 = blockIdx.y * NL;
+  const int64_t bz = blockIdx.z;
+  const float2* in = a.in + bz * (int64_t)nlines * nin;
+  float* zprev = a.zprev ? a.zprev + bz * (int64_t)nout * nlines : nullptr;
+  const bool spec = a.use_prev && zprev;
+  // loading phase: line la, elements jl, jl + JS, ...
+  const int la = warp / WPL, l = l0 + la, jl = (warp % WPL) * 32 + lane;
+  constexpr int JS = 32 * WPL;
+
+  // ---- prologue independent of the preceding kernel ----
+  // output o = tid + r NT of the CTA: line o % NL, output i0 + o / NL
+  const int oline = tid % NL;
+  bool owns[OWN];
+  int64_t my_pt[OWN];
+#pragma unroll
+  for (int r = 0; r < OWN; ++r) {
+    const int oi = (tid + r * NT) / NL;
+    owns[r] = oi < OUT && i0 + oi < nout && l0 + oline < nlines;
+    my_pt[r] = (int64_t)(i0 + oi) * nlines + l0 + oline;
+  }
+  float zp[OWN];
+#pragma unroll
+  for (int r = 0; r < OWN; ++r) zp[r] = (owns[r] && spec) ? zprev[my_pt[r]] : 0.0f;
+  for (int j = tid; j < nin; j += NT) {
+    const float y = a.yi[j];
+    sy[j] = make_float2(y, y);
+  }
+  float xq[OPL];
+#pragma unroll
+  for (int q = 0; q < OPL; ++q) {
+    const int i = i0 + lane + 32 * q;
+    xq[q] = a.xo[i < nout ? i : nout - 1];
+  }
+  pdl_wait();
+  if (a.zero_acc && blockIdx.x == 0 && blockIdx.y == 0 && tid < 2) a.zero_acc[2 * bz + tid] = 0.0;
+  pdl_launch_dependents();
+
+  // ---- line values ----
+  const bool in_regs = nin <= LR * JS;
+  const int64_t base = (int64_t)l * nin;
+  ff lv[LR];
+  float mx = -INFINITY;
+#pragma unroll
+  for (int r = 0; r < LR; ++r) lv[r] = ff_ninf();
+  if (l < nlines) {
+    if (in_regs) {
+#pragma unroll
+      for (int r = 0; r < LR; ++r) {
+        const int j = jl + r * JS;
+        if (j < nin) lv[r] = load_L_ff(a, in, base + j);
+        mx = fmaxf(mx, lv[r].hi);
+      }
+    } else {
+      for (int j = jl; j < nin; j += JS) mx = fmaxf(mx, load_L_ff(a, in, base + j).hi);
+    }
+  }
+  mx = warp_maxf(mx);
+  if (lane == 0) sred[la][warp % WPL] = mx;
+  __syncthreads();
+  float mxo = sred[oline][0];  // of the line whose outputs this thread finishes
+#pragma unroll
+  for (int w = 1; w < WPL; ++w) mxo = fmaxf(mxo, sred[oline][w]);
+#pragma unroll
+  for (int w = 0; w < WPL; ++w) mx = fmaxf(mx, sred[la][w]);
+  auto stage = [&](int j, ff v) {
+    reinterpret_cast<float*>(sml)[4 * j + la] = (v.hi == -INFINITY) ? -INFINITY : ((v.hi - mx) + v.lo) * kLog2e;
+  };
+  if (in_regs) {
+#pragma unroll
+    for (int r = 0; r < LR; ++r) {
+      const int j = jl + r * JS;
+      if (j < nin) stage(j, lv[r]);
+    }
+  } else {
+    for (int j = jl; j < nin; j += JS) stage(j, l < nlines ? load_L_ff(a, in, base + j) : ff_ninf());
+  }
+  // speculative shifts in log2 units relative to the staged line
+#pragma unroll
+  for (int r = 0; r < OWN; ++r) {
+    const int oi = (tid + r * NT) / NL;
+    if (oi < OUT)
+      sshift[oline * OUT + oi] = (!owns[r] || zp[r] == -INFINITY || mxo == -INFINITY) ? 0.0f : (zp[r] - mxo) * kLog2e;
+  }
+  __syncthreads();
+
+  const f2p nk2 = pk(-a.k2, -a.k2);
+  const int J = (nin + NW - 1) / NW;
+  const int j0 = warp * J, j1 = min(nin, j0 + J);
+  f2p X[P];
+#pragma unroll
+  for (int p = 0; p < P; ++p) X[p] = pk(xq[2 * p], xq[2 * p + 1]);
+
+  bool exact = !spec;
+  float num = 0.0f, den = 0.0f;
+  for (int attempt = 0; attempt < 2; ++attempt) {
+    float mq[NL][OPL];
+    if (!exact) {
+#pragma unroll
+      for (int u = 0; u < NL; ++u)
+#pragma unroll
+        for (int q = 0; q < OPL; ++q) mq[u][q] = sshift[u * OUT + lane + 32 * q];
+    } else {
+#pragma unroll
+      for (int u = 0; u < NL; ++u)
+#pragma unroll
+        for (int q = 0; q < OPL; ++q) mq[u][q] = -INFINITY;
+#pragma unroll 2
+      for (int j = j0; j < j1; ++j) {
+        const float4 t4 = sml[j];
+        const float2 y2 = sy[j];
+        const f2p Y = pk(y2.x, y2.y);
+        const float t[NL] = {t4.x, t4.y, t4.z, t4.w};
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+          const f2p D = sub2(X[p], Y);
+          const f2p Q = mul2(D, D);
+#pragma unroll
+          for (int u = 0; u < NL; ++u) {
+            const float2 A = upk(fma2(nk2, Q, pk(t[u], t[u])));
+            mq[u][2 * p] = fmaxf(mq[u][2 * p], A.x);
+            mq[u][2 * p + 1] = fmaxf(mq[u][2 * p + 1], A.y);
+          }
+        }
+      }
+    }
+    f2p MS[NL][P], S[NL][P];
+#pragma unroll
+    for (int u = 0; u < NL; ++u)
+#pragma unroll
+      for (int p = 0; p < P; ++p) {
+        const float m0 = mq[u][2 * p], m1 = mq[u][2 * p + 1];
+        MS[u][p] = pk(m0 == -INFINITY ? 0.0f : m0, m1 == -INFINITY ? 0.0f : m1);
+        S[u][p] = pk(0.0f, 0.0f);
+      }
+#pragma unroll 2
+    for (int j = j0; j < j1; ++j) {
+      const float4 t4 = sml[j];
+      const float2 y2 = sy[j];
+      const f2p Y = pk(y2.x, y2.y);
+      const float t[NL] = {t4.x, t4.y, t4.z, t4.w};
+#pragma unroll
+      for (int p = 0; p < P; ++p) {
+        const f2p D = sub2(X[p], Y);
+        const f2p Q = mul2(D, D);
+#pragma unroll
+        for (int u = 0; u < NL; ++u) {
+          const float2 A = upk(fma2(nk2, Q, sub2(pk(t[u], t[u]), MS[u][p])));
+          S[u][p] = add2(S[u][p], pk(ex2_approx(A.x), ex2_approx(A.y)));
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < NL; ++u)
+#pragma unroll
+      for (int p = 0; p < P; ++p) {
+        const float2 sv = upk(S[u][p]), m = upk(MS[u][p]);
+        // (a maximum of -inf: every staged value of the range is -inf, and so the sum 0)
+        float2* dst = part + (size_t)u * T::kPartStride + warp * OUT + lane + 64 * p;
+        dst[0] = make_float2(m.x, sv.x);
+        dst[32] = make_float2(m.y, sv.y);
+      }
+    __syncthreads();
+
+    // combine the NW ranges of each output
+    const float2* opart = part + (size_t)oline * T::kPartStride;
+    bool bad = false;
+    float Mo[OWN], So[OWN];
+#pragma unroll
+    for (int r = 0; r < OWN; ++r) {
+      const int oi = (tid + r * NT) / NL;
+      Mo[r] = -INFINITY;
+      So[r] = 0.0f;
+      if (oi < OUT) {
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+          const float2 pr = opart[w * OUT + oi];
+          if (pr.y > 0.0f) Mo[r] = fmaxf(Mo[r], pr.x);
+        }
+        if (Mo[r] != -INFINITY) {
+#pragma unroll
+          for (int w = 0; w < NW; ++w) {
+            const float2 pr = opart[w * OUT + oi];
+            if (pr.y > 0.0f) So[r] += pr.y * ex2_approx(pr.x - Mo[r]);
+          }
+        }
+        if (owns[r] && !exact && mxo != -INFINITY) bad = bad || !(So[r] >= 0x1p-90f && So[r] <= 0x1p100f);
+      }
+    }
+    if (!exact && __syncthreads_or(bad ? 1 : 0)) {
+      exact = true;
+      continue;  // block-uniform: redo with exact maxima
+    }
+#pragma unroll
+    for (int r = 0; r < OWN; ++r) {
+      if (!owns[r]) continue;
+      EpiPre pre;
+      epilogue_prefetch(epi, bz, my_pt[r], pre);
+      ff z = ff_ninf();
+      if (So[r] > 0.0f) z = pass_result(mxo, Mo[r], So[r]);
+      if (zprev) zprev[my_pt[r]] = z.hi;
+      float n1, d1;
+      epilogue_apply(epi, bz, my_pt[r], z, pre, n1, d1);
+      num += n1;
+      den += d1;
+    }
+    break;
+  }
+  if (epi.err) block_add2f<NT>(num, den, epi.err + 2 * bz);
+}
+
 // ---------------------------------------------------------------------------
 // Persistent solve: the whole iteration of a single FP32 grid problem in one
 // cooperative launch (all CTAs co-resident).  Each pass is a set of work items
@@ -985,6 +1235,19 @@ constexpr TileShape kTiles[] = {{8, 4}, {4, 4}, {2, 4}, {1, 4}, {8, 2}, {4, 2}, 
 constexpr int kTc3Tile = 7;
 constexpr int kShortTile = 8;
 constexpr int kBlkTile0 = 9;  // + variant 0 .. grid_blk_variants() - 1
+// A tile of 4 or 8 warps takes four lines (grid_pass_f32_ml) where there are lines
+// enough to keep the GPU full of such CTAs.  Measured per pass, best tile of one
+// line against best of four: 32 batches of 128 x 128 lines x inputs 23.3 and 18.8 us,
+// of 64 x 64 6.7 and 5.8; but 224 lines of 56 3.2 and 3.5, 64 of 64 2.9 and 3.5, and in
+// a solve 256 of 256 6.5 and 6.8, and a colour transfer's 2048 lines of 32 and 1024 of
+// 64 8.5 and 8.7 ms: with 65536 inputs a pass is a chain of latencies, longer in the
+// larger CTA.
+constexpr int64_t kMlMinLines = 1024, kMlMinInputs = 131072;
+constexpr size_t kMlSmemMax = 110 * 1024;
+bool ml_ok(const PassArgs& a, int nbatch, int nw) {
+  const int64_t lines = (int64_t)a.nlines * nbatch;
+  return nw >= 4 && lines >= kMlMinLines && lines * a.nin >= kMlMinInputs && MlTile<8, 4>::smem(a.nin) <= kMlSmemMax;
+}
 bool is_blk(int t) { return t >= kBlkTile0 && t < kBlkTile0 + grid_blk_variants(); }
 int blk_mask(const PassArgs& a) {
   int m = 0;
@@ -1036,19 +1299,31 @@ cudaError_t launch_f32_tile(const PassArgs& a, const Epilogue& epi, int nbatch, 
   return cudaLaunchKernelEx(&cfg, grid_pass_f32<NW, OPL>, a, epi);
 }
 
+template <int NW, int OPL>
+cudaError_t launch_f32_ml(const PassArgs& a, const Epilogue& epi, int nbatch, cudaStream_t s) {
+  typedef MlTile<NW, OPL> T;
+  const dim3 grid((a.nout + T::kOut - 1) / T::kOut, (a.nlines + kMlLines - 1) / kMlLines, nbatch);
+  if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidConfiguration;
+  const size_t smem = T::smem(a.nin);
+  const cudaError_t e = smem_at_least(grid_pass_f32_ml<NW, OPL>, smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(grid_pass_f32_ml<NW, OPL>, grid, dim3(T::kThreads), smem, s, a, epi);
+}
+
 cudaError_t launch_f32(int t, const PassArgs& a, const Epilogue& epi, int nbatch, cudaStream_t s) {
   if (t == kTc3Tile && a.tc3_ok)
     return launch_grid_pass_tc3(a.in, a.logw, a.in_is_pot, a.nlines, a.nin, a.yi, a.nout, a.xo, a.inv_eps, a.k2,
                                 nbatch, epi, s, a.tc_err, a.zero_acc);
   if (t == kShortTile && short_ok(a)) return launch_f32_short(a, epi, nbatch, s);
   if (is_blk(t) && grid_blk_ok(a, t - kBlkTile0)) return launch_grid_pass_blk(a, t - kBlkTile0, epi, nbatch, s);
+  const bool ml = ml_ok(a, nbatch, kTiles[t < kNumTiles ? t : 0].nw);
   switch (t) {
-    case 0: return launch_f32_tile<8, 4>(a, epi, nbatch, s);
-    case 1: return launch_f32_tile<4, 4>(a, epi, nbatch, s);
+    case 0: return ml ? launch_f32_ml<8, 4>(a, epi, nbatch, s) : launch_f32_tile<8, 4>(a, epi, nbatch, s);
+    case 1: return ml ? launch_f32_ml<4, 4>(a, epi, nbatch, s) : launch_f32_tile<4, 4>(a, epi, nbatch, s);
     case 2: return launch_f32_tile<2, 4>(a, epi, nbatch, s);
     case 3: return launch_f32_tile<1, 4>(a, epi, nbatch, s);
-    case 4: return launch_f32_tile<8, 2>(a, epi, nbatch, s);
-    case 5: return launch_f32_tile<4, 2>(a, epi, nbatch, s);
+    case 4: return ml ? launch_f32_ml<8, 2>(a, epi, nbatch, s) : launch_f32_tile<8, 2>(a, epi, nbatch, s);
+    case 5: return ml ? launch_f32_ml<4, 2>(a, epi, nbatch, s) : launch_f32_tile<4, 2>(a, epi, nbatch, s);
     case 6: return launch_f32_tile<2, 2>(a, epi, nbatch, s);
     default: return launch_f32_tile<8, 4>(a, epi, nbatch, s);
   }
