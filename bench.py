@@ -53,9 +53,8 @@ MUFU_PEAK_GEXP = SM_COUNT * MUFU_PER_CLK * SM_MAX_MHZ * 1e6 / 1e9
 FP64_PEAK_GFLOPS = 1250.0
 # HBM copy bandwidth measured on this GPU type (MEASURED_PEAKS.json hbm_gbs)
 HBM_PEAK_GBS = 6760.6
-# dram bytes of one rows_lse_f64_pf<4, 4, 1> launch of the wf workload (ncu,
-# profiles/rows_lse_f64_pf_wf3000.md); None once the kernel changes
-WF_ROWS_TRAFFIC_BYTES = 36848640
+# dram bytes of one rows_lse_f64_chunks<24> launch of the wf workload; None: not captured
+WF_ROWS_TRAFFIC_BYTES = None
 # dram bytes of one alg1_cluster launch (2000 iterations of the dense 256 x 256
 # problem; profiles/alg1_cluster_dense256.md); None once the kernel changes
 ALG1_CLUSTER_TRAFFIC_BYTES = 1185792
@@ -493,7 +492,7 @@ def run_single(args, rank, world, local_rank):
                                            iters=500, launch_mode=args.launch_mode)
             info["marg_err"] = float("nan")
             return U_, V_, info
-        work_per_iter, unit_work, kernel = 2.0 * S * n * n, "Gterm/s", "rows_lse_f64_pf<4, 4, 1>"
+        work_per_iter, unit_work, kernel = 2.0 * S * n * n, "Gterm/s", "rows_lse_f64_chunks<24>"
         cfg = {"workload": f"wf-flow-{S}species-3000-eps{eps:g}-tau{tau:g}-alpha1-500it-x4steps",
                "n": n, "species": S, "eps": eps, "tau": tau, "alpha": 1.0, "lambda": 1.0,
                "iters_per_flow_step": 500, "flow_steps_per_bench_step": nflow,
@@ -592,17 +591,17 @@ def run_single(args, rank, world, local_rank):
         if wl in ("bary", "color"):
             line["grid_tiles"] = uot.autotune_table().strip().splitlines()
     elif unit_work == "Gterm/s":
-        # rows_lse_f64_pf: the FP32 prefilter reads the FP32 copy of the cost once
-        # per term (4 B; both sweeps run from shared memory) and evaluates FP64
-        # exponentials only where they do not underflow, so its floor is HBM.
-        gbs = achieved * 4.0
+        # rows_lse_f64_chunks reads the least cost of every chunk of 32 columns (4 B per
+        # 32 terms) and the chunks that can matter; at this eps it is a chain of
+        # latencies, far from any memory rate.
+        gbs = achieved * 4.0 / 32
         line["roofline"] = {"bound": "hbm", "kernel": kernel, "achieved": gbs, "peak": HBM_PEAK_GBS,
                             "unit": "GB/s", "frac": gbs / HBM_PEAK_GBS,
                             "traffic": WF_ROWS_TRAFFIC_BYTES,
                             "traffic_source": ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch "
-                                               "(cold cache; profiles/rows_lse_f64_pf_wf3000.md)")
+                                               "(cold cache)")
                             if WF_ROWS_TRAFFIC_BYTES is not None else None,
-                            "algorithmic_bytes_per_launch": 4.0 * n * n,
+                            "algorithmic_bytes_per_launch": 4.0 * n * ((n + 31) // 32),
                             "terms_per_s": achieved * 1e9,
                             "peak_source": "MEASURED_PEAKS.json hbm_gbs (burst copy), of measured",
                             "timing": timing}
