@@ -487,6 +487,8 @@ __global__ void __launch_bounds__(NW * 32, NW == 8 ? 3 : 2) batch_solve(BatchArg
   float4* st0 = smem4;
   S1* st1 = reinterpret_cast<S1*>(st0 + lmax);
   float2* part = reinterpret_cast<float2*>(reinterpret_cast<char*>(st0 + lmax) + (size_t)lmax * stage1_bytes<D>());
+  // Shared memory of another CTA may be written once that CTA is known to run.
+  if constexpr (kCl) unit_sync<kCl>();
   for (;;) {
     if (tid == 0 && rank == 0) {
       const int t = atomicAdd(a.next, 1);
