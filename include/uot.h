@@ -279,8 +279,13 @@ int uot_autotune_table(char* buf, int len);
  * is more than 3% faster; uot_autotune_table lists the choice.
  * uot_force_batch_warps(w): w = 8 or 16 forces that size, 0 returns to the
  * tuned one; UOT_EINVAL otherwise.
+ * uot_force_batch_cluster(c): c = 1, 2, 4 or 8 CTAs per problem in every batch
+ * (before a forced CTA size: clusters have 16 warps per CTA), 0 returns to the
+ * estimate; UOT_EINVAL otherwise.  A forced size that the device cannot hold
+ * makes uot_solve_batch return UOT_ECUDA.  Process-wide, guarded by a mutex.
  */
 uot_status uot_force_batch_warps(int warps);
+uot_status uot_force_batch_cluster(int ctas);
 
 /*
  * uot_probe_pipes -- throughput probes (instrumentation): out (host) receives

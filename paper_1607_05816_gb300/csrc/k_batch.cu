@@ -675,6 +675,7 @@ struct BEntry {
 std::mutex g_bmu;
 std::map<BKey, BEntry> g_btuned;
 int g_bforced = -1;  // forced variant, -1: tuned
+int g_cforced = 0;   // forced CTAs per problem, 0: estimated
 
 // ---- clusters ----
 
@@ -816,6 +817,13 @@ int batch_force_warps(int warps) {
   return -1;
 }
 
+int batch_force_cluster(int ctas) {
+  if (ctas != 0 && ctas != 1 && ctas != 2 && ctas != 4 && ctas != 8) return -1;
+  std::lock_guard<std::mutex> lk(g_bmu);
+  g_cforced = ctas;
+  return 0;
+}
+
 int batch_pick_variant(const BatchArgs& a, const int* h_order, cudaStream_t s) {
   std::lock_guard<std::mutex> lk(g_bmu);
   if (g_bforced >= 0) return g_bforced;
@@ -858,6 +866,7 @@ std::string batch_tune_table() {
 int batch_cluster(int d, int nmax, int mmax, const int* n, const int* m, const int* order, int nprob) {
   {
     std::lock_guard<std::mutex> lk(g_bmu);
+    if (g_cforced > 0) return g_cforced;
     if (g_bforced >= 0) return 1;
   }
   const int per = ctas_any(d, 1, nmax, mmax) * sm_count();

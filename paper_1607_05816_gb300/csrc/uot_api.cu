@@ -208,6 +208,8 @@ uot_status uot_selftest_bounded_wait(double seconds, void* stream) {
 
 uot_status uot_force_batch_warps(int warps) { return batch_force_warps(warps) == 0 ? UOT_OK : UOT_EINVAL; }
 
+uot_status uot_force_batch_cluster(int ctas) { return batch_force_cluster(ctas) == 0 ? UOT_OK : UOT_EINVAL; }
+
 int uot_autotune_table(char* buf, int len) {
   const std::string t = grid_tile_table() + batch_tune_table();
   if (buf && len > 0) {

@@ -824,6 +824,7 @@ struct BatchArgs {
 int batch_ctas_per_sm(int d, int variant, int nmax, int mmax);
 int batch_pick_variant(const BatchArgs& a, const int* h_order, cudaStream_t s);
 int batch_force_warps(int warps);  // 8 or 16 forces a CTA size, 0 returns to the tuned one; -1 if invalid
+int batch_force_cluster(int ctas);  // 1, 2, 4 or 8 forces CTAs per problem, 0 returns to the estimate; -1 if invalid
 std::string batch_tune_table();
 cudaError_t launch_batch(const BatchArgs& a, int variant, int grid, cudaStream_t s);
 // CTAs per problem (1, 2, 4 or 8) for problems of n[k] x m[k] points in queue order;

@@ -148,6 +148,7 @@ _SIGS = {
     "uot_force_grid_tile": (C.c_int, [C.c_int]),
     "uot_grid_tile_count": (C.c_int, []),
     "uot_force_batch_warps": (C.c_int, [C.c_int]),
+    "uot_force_batch_cluster": (C.c_int, [C.c_int]),
     "uot_selftest_bounded_wait": (C.c_int, [C.c_double, C.c_void_p]),
     "uot_probe_pipes": (C.c_int, [C.POINTER(C.c_double), C.c_void_p]),
     "uot_force_precise_passes": (C.c_int, [C.c_int]),
@@ -231,6 +232,11 @@ def force_grid_tile(idx: int):
 def force_batch_warps(warps: int):
     """CTA size of solve_batch: 8 or 16 warps, 0 = the tuner's choice."""
     _check(load().uot_force_batch_warps(int(warps)), "uot_force_batch_warps")
+
+
+def force_batch_cluster(ctas: int):
+    """CTAs per problem of solve_batch: 1, 2, 4 or 8, 0 = estimated from the batch."""
+    _check(load().uot_force_batch_cluster(int(ctas)), "uot_force_batch_cluster")
 
 
 def selftest_bounded_wait(seconds: float) -> str:
