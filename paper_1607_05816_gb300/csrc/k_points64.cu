@@ -20,11 +20,13 @@
 //   rows     z_i = M_i + log sum_j K_ij e^{L_j - beta_j},
 //   columns  z_j = -beta_j + log sum_i K_ij e^{L_i + M_i},
 // one FP64 multiply-add and 8 bytes a term, in both directions from one copy.
-// A result is used only where underflow cannot have touched it: with all
-// weights below e^300 the terms that K_ij lost are below e^300 2^-1022 nin in
-// sum, so a sum above 1e-150 is exact to rounding; any other row or column is
-// redone on the fly.  A weight above e^300 (the potentials moved by 300 eps)
-// makes the next row pass store the kernel anew.
+// A row is stored with a shift that puts its sum between 1e-30 and 1e30 (the FP32
+// shift where it does, else the FP64 maximum), so K_ij < 1e30.  A result is used
+// only where neither underflow nor overflow can have touched it: with all weights
+// below e^300 the terms that K_ij lost are below e^300 2^-1022 nin in sum, so a sum
+// above 1e-150 is exact to rounding, and no sum comes near 1e300; any other row or
+// column is redone on the fly.  A weight above e^300 (the potentials moved by 300
+// eps) makes the next row pass store the kernel anew.
 //
 // Measured, 3001 x 2477 points in 2-D: 20 iterations and the objective 31.9 ms
 // with two FP64 sweeps and exp() per pass (705 us), 2.76 ms here.
@@ -39,7 +41,7 @@ namespace uot {
 namespace {
 
 constexpr double kDrift = 300.0;                  // largest log weight before a new kernel
-constexpr double kLeastSum = 1e-150;
+constexpr double kLeastSum = 1e-150, kMostSum = 1e300;  // sums of products that are used
 
 // The line L and its FP32 copy; with a stored kernel the weights e^{L - beta},
 // and *drift raised where one is too large or a point that had no mass when the
@@ -108,7 +110,10 @@ __device__ __forceinline__ void row64(const Rows64& a, int i, const double* tab,
     return q;
   };
   // the shift: from the FP32 copies, and once more in FP64 where that left the
-  // sum empty or out of range (exponents beyond FP32's reach, or no mass at all)
+  // sum empty or out of range (exponents beyond FP32's reach, or no mass at all).
+  // Stored terms meet weights up to e^300, so their range is narrower: coordinates
+  // with an offset large against their spread move the FP32 shift by hundreds.
+  constexpr double least = STORE ? 1e-30 : 1e-270, most = STORE ? 1e30 : 1e290;
   for (int attempt = a.x32 ? 0 : 1; attempt < 2; ++attempt) {
     double m;
     if (attempt == 0) {
@@ -155,7 +160,7 @@ __device__ __forceinline__ void row64(const Rows64& a, int i, const double* tab,
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     S = s;
-    if (s >= 1e-270 && s <= 1e290) return;
+    if (s >= least && s <= most) return;
   }
 }
 
@@ -195,7 +200,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) points64_rows(Rows64 a, Epilog
     for (int o = 16; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
     S = s0;
     M = a.M[i];
-    done = S >= kLeastSum && M != -kInf;  // (a NaN is recomputed and stays one)
+    done = S >= kLeastSum && S <= kMostSum && M != -kInf;  // (a NaN is recomputed and stays one)
   }
   if (__syncthreads_or(!done)) {  // block-uniform
     exp_table_load(tab);
@@ -330,7 +335,7 @@ __global__ void __launch_bounds__(256) points64_cols_end(Rows64 a, const double*
 #pragma unroll
     for (int w = 0; w < 8; ++w) s += red[w][lane];
     const double b = (c < a.nrows) ? beta[c] : 0.0;
-    const bool bad = c < a.nrows && (!(s >= kLeastSum) || b == -kInf);
+    const bool bad = c < a.nrows && (!(s >= kLeastSum && s <= kMostSum) || b == -kInf);
     zc[lane] = smax - b + log(s);
     const unsigned m = __ballot_sync(0xffffffffu, bad);
     if (lane == 0) bad_mask = m;
