@@ -227,7 +227,8 @@ __global__ void __launch_bounds__(kRowWarps * 32) points64_rows(Rows64 a, Epilog
   if (epi.err) block_add2<kRowWarps * 32>(num, den, epi.err);
 }
 
-// Column pass over the stored kernel: CTA = 256 columns x kColRows rows.  The
+// Column pass over the stored kernel: CTA = 256 columns x kColRows rows, all in the
+// launch grid's first dimension (the others end at 65535: 4.2 million rows).  The
 // rows' weights e^{L_i + M_i - s} are formed here, s their largest log in this
 // chunk of rows (16 KB of exponentials per chunk, repeated per column tile).
 constexpr int kColRows = 64, kColTile = 256;
@@ -239,7 +240,9 @@ __global__ void __launch_bounds__(kColTile / 2) points64_cols(const double* __re
                                                               double* __restrict__ shift) {
   __shared__ double v[kColRows];
   __shared__ double sh;
-  const int r0 = blockIdx.y * kColRows, nr = min(kColRows, nrows - r0);
+  const int ntiles = (ncols + kColTile - 1) / kColTile;
+  const int chunk = blockIdx.x / ntiles, tile = blockIdx.x - chunk * ntiles;
+  const int r0 = chunk * kColRows, nr = min(kColRows, nrows - r0);
   pdl_wait();
   pdl_launch_dependents();
   if (threadIdx.x < 32) {
@@ -263,11 +266,11 @@ __global__ void __launch_bounds__(kColTile / 2) points64_cols(const double* __re
     for (int u = 0; u < 2; ++u) v[threadIdx.x + 32 * u] = (l[u] == -kInf) ? 0.0 : exp(l[u] - mx);
     if (threadIdx.x == 0) {
       sh = mx;
-      if (blockIdx.x == 0) shift[blockIdx.y] = mx;
+      if (tile == 0) shift[chunk] = mx;
     }
   }
   __syncthreads();
-  const int c = blockIdx.x * kColTile + 2 * threadIdx.x;
+  const int c = tile * kColTile + 2 * threadIdx.x;
   if (c >= ncols) return;
   double s0 = 0.0, s1 = 0.0;
   if (sh != -kInf) {
@@ -279,7 +282,7 @@ __global__ void __launch_bounds__(kColTile / 2) points64_cols(const double* __re
       s1 = fma(kv.y, v[r], s1);
     }
   }
-  double* p = part + (int64_t)blockIdx.y * ld + c;
+  double* p = part + (int64_t)chunk * ld + c;
   *reinterpret_cast<double2*>(p) = make_double2(s0, s1);
 }
 
@@ -408,7 +411,8 @@ cudaError_t launch_points64(const Points64& p, int dir, const double* W, const d
     double* shift = p.part + (int64_t)nchunks * ld;
     a.ld = ld;
     count_launches(2);
-    e = launch_pdl(points64_cols, dim3((p.m + kColTile - 1) / kColTile, nchunks), dim3(kColTile / 2), s,
+    // (a stored kernel has at most 2^29 entries: the product fits)
+    e = launch_pdl(points64_cols, dim3((p.m + kColTile - 1) / kColTile * nchunks), dim3(kColTile / 2), s,
                    (const double*)p.K, ld, p.n, p.m, W, logw, a.inv_eps, (const double*)p.M, p.part, shift);
     if (e != cudaSuccess) return e;
     auto end = [&](auto kern) {
