@@ -288,6 +288,15 @@ uot_status uot_force_batch_warps(int warps);
 uot_status uot_force_batch_cluster(int ctas);
 
 /*
+ * uot_fail_captures(k) -- failure injection for tests, on the host: inside every
+ * CUDA-graph capture of a solver the first k applications of the Gibbs operator
+ * are recorded and the next one returns an error, so the capture fails part way
+ * and the solver goes on launch by launch.  k < 0 (the default) injects nothing.
+ * Returns the previous setting.  Process-wide.
+ */
+int uot_fail_captures(int applications);
+
+/*
  * uot_probe_pipes -- throughput probes (instrumentation): out (host) receives
  * the sustained rates of the pipes the kernels are bound by, in operations per
  * clock per SM measured with in-kernel clock64() over dependent-chain loops

@@ -19,6 +19,18 @@ thread_local std::string g_last_error;
 std::atomic<long long> g_launches{0};
 Prof g_prof;
 
+// Failure injection: applications left in this thread's capture (-1: not capturing).
+static std::atomic<int> g_capture_fault{-1};
+static thread_local int t_capture_left = -1;
+void capture_fault_begin() { t_capture_left = g_capture_fault.load(); }
+void capture_fault_end() { t_capture_left = -1; }
+bool capture_fault() {
+  if (t_capture_left < 0) return false;
+  if (t_capture_left == 0) return true;
+  --t_capture_left;
+  return false;
+}
+
 namespace {
 
 // ---------------------------------------------------------------------------
@@ -207,6 +219,8 @@ uot_status uot_selftest_bounded_wait(double seconds, void* stream) {
 }
 
 uot_status uot_force_batch_warps(int warps) { return batch_force_warps(warps) == 0 ? UOT_OK : UOT_EINVAL; }
+
+int uot_fail_captures(int applications) { return g_capture_fault.exchange(applications < 0 ? -1 : applications); }
 
 uot_status uot_force_batch_cluster(int ctas) { return batch_force_cluster(ctas) == 0 ? UOT_OK : UOT_EINVAL; }
 

@@ -1079,10 +1079,29 @@ struct Gibbs {
     return (reach <= 90.0 && nin <= grid_pass_tc3_max_nin()) ? 1 : 0;
   }
 
+  // The host's records of what the device buffers hold.  A capture changes them
+  // although nothing has run; where it fails they are put back.
+  struct Records {
+    double fac_eps[2][UOT_MAX_DIM], zeps[2], p64_eps;
+  };
+  Records records() const {
+    Records r;
+    memcpy(r.fac_eps, fac_eps, sizeof(fac_eps));
+    memcpy(r.zeps, zeps, sizeof(zeps));
+    r.p64_eps = p64_eps;
+    return r;
+  }
+  void restore(const Records& r) {
+    memcpy(fac_eps, r.fac_eps, sizeof(fac_eps));
+    memcpy(zeps, r.zeps, sizeof(zeps));
+    p64_eps = r.p64_eps;
+  }
+
   // zero_acc: two doubles cleared before the result is produced (violation
   // accumulators of a checked iteration), inside the first kernel when possible.
   cudaError_t apply(int dir, const double* W, const double* logw, double eps, const Epilogue& epi,
                     cudaStream_t s, double* zero_acc = nullptr) {
+    if (capture_fault()) return cudaErrorStreamCaptureInvalidated;
     if (g.kind == UOT_GEOM_GRID) {
       const int use_prev = (zbuf[dir][0] != nullptr && zeps[dir] == eps) ? 1 : 0;
       const int d = g.ndim;
@@ -1232,8 +1251,16 @@ struct Gibbs {
 struct BlockGraph {
   cudaGraphExec_t exec = nullptr;
   long long kernels = 0;
+  // G: the operator that the body applies
   template <class F>
-  cudaError_t capture(F&& body) {
+  cudaError_t capture(Gibbs& G, F&& body) {
+    const Gibbs::Records before = G.records();
+    const cudaError_t e = record(body);
+    if (e != cudaSuccess) G.restore(before);
+    return e;
+  }
+  template <class F>
+  cudaError_t record(F&& body) {
     cudaStream_t cs = nullptr;
     cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
     if (e != cudaSuccess) return e;
@@ -1241,7 +1268,9 @@ struct BlockGraph {
     cudaGraph_t graph = nullptr;
     e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
+      capture_fault_begin();
       const cudaError_t eb = body(cs);
+      capture_fault_end();
       const cudaError_t ee = cudaStreamEndCapture(cs, &graph);
       e = (eb != cudaSuccess) ? eb : ee;
     }

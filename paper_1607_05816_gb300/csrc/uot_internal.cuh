@@ -823,6 +823,11 @@ struct BatchArgs {
 // tuner is on (batch_pick_variant: synchronises `s`; a.next is left dirty).
 int batch_ctas_per_sm(int d, int variant, int nmax, int mmax);
 int batch_pick_variant(const BatchArgs& a, const int* h_order, cudaStream_t s);
+// Failure injection on the host (uot_fail_captures): inside a graph capture, the
+// Gibbs-operator applications after the first few return an error.
+bool capture_fault();
+void capture_fault_begin();
+void capture_fault_end();
 int batch_force_warps(int warps);  // 8 or 16 forces a CTA size, 0 returns to the tuned one; -1 if invalid
 int batch_force_cluster(int ctas);  // 1, 2, 4 or 8 forces CTAs per problem, 0 returns to the estimate; -1 if invalid
 std::string batch_tune_table();

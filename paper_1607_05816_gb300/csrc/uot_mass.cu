@@ -589,7 +589,7 @@ uot_status solve_mass_impl(const uot_geom* g, const void* p, const void* dx, con
   while (it < o->max_iter) {
     if (graph_ok && !first && it > 0 && it % check_every == 0 && it + check_every <= o->max_iter) {
       if (!bg.exec) {
-        cudaError_t e = bg.capture([&](cudaStream_t cs) -> cudaError_t {
+        cudaError_t e = bg.capture(G, [&](cudaStream_t cs) -> cudaError_t {
           for (int k = 0; k < check_every; ++k) {
             cudaError_t e2 = iteration(o->eps, k == check_every - 1, cs);
             if (e2 != cudaSuccess) return e2;

@@ -363,7 +363,7 @@ uot_status solve_impl(const uot_geom* g, int batch, const void* p, const void* d
     while (it < o->max_iter) {
       if (graph_ok && it > 0 && it % check_every == 0 && it + check_every <= o->max_iter) {
         if (!bg.exec) {
-          cudaError_t e = bg.capture([&](cudaStream_t cs) -> cudaError_t {
+          cudaError_t e = bg.capture(G, [&](cudaStream_t cs) -> cudaError_t {
             for (int k = 0; k < check_every; ++k) {
               cudaError_t e2 = iteration(k == check_every - 1, cs);
               if (e2 != cudaSuccess) return e2;
@@ -510,7 +510,7 @@ uot_status solve_impl(const uot_geom* g, int batch, const void* p, const void* d
     while (it < o->max_iter) {
       if (graph_ok && it > 0 && it % check_every == 0 && it + check_every <= o->max_iter) {
         if (!bg.exec) {
-          cudaError_t e = bg.capture([&](cudaStream_t cs) -> cudaError_t {
+          cudaError_t e = bg.capture(G, [&](cudaStream_t cs) -> cudaError_t {
             for (int k = 0; k < check_every; ++k) {
               cudaError_t e2 = iteration(o->eps, k == check_every - 1, translate && k == check_every - 1, cs);
               if (e2 != cudaSuccess) return e2;

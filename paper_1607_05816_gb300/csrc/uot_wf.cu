@@ -266,7 +266,7 @@ uot_status wf_flow_impl(const uot_geom* g, int S, const void* P0, const void* dx
   for (int k = 0; k < nsteps; ++k) {
     if (graph_ok && k > 0) {
       if (!bg.exec) {
-        cudaError_t e = bg.capture([&](cudaStream_t cs) { return step(cs); });
+        cudaError_t e = bg.capture(G, [&](cudaStream_t cs) { return step(cs); });
         if (e != cudaSuccess) {
           graph_ok = false;
           (void)cudaGetLastError();

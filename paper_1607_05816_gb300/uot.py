@@ -149,6 +149,7 @@ _SIGS = {
     "uot_grid_tile_count": (C.c_int, []),
     "uot_force_batch_warps": (C.c_int, [C.c_int]),
     "uot_force_batch_cluster": (C.c_int, [C.c_int]),
+    "uot_fail_captures": (C.c_int, [C.c_int]),
     "uot_selftest_bounded_wait": (C.c_int, [C.c_double, C.c_void_p]),
     "uot_probe_pipes": (C.c_int, [C.POINTER(C.c_double), C.c_void_p]),
     "uot_force_precise_passes": (C.c_int, [C.c_int]),
@@ -237,6 +238,12 @@ def force_batch_warps(warps: int):
 def force_batch_cluster(ctas: int):
     """CTAs per problem of solve_batch: 1, 2, 4 or 8, 0 = estimated from the batch."""
     _check(load().uot_force_batch_cluster(int(ctas)), "uot_force_batch_cluster")
+
+
+def fail_captures(applications: int) -> int:
+    """uot_fail_captures: graph captures fail after this many operator applications
+    (-1: never); returns the previous setting."""
+    return load().uot_fail_captures(int(applications))
 
 
 def selftest_bounded_wait(seconds: float) -> str:
