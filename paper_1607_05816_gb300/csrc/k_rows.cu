@@ -211,7 +211,9 @@ __global__ void __launch_bounds__(256) chunkmin32(const double* __restrict__ C, 
 // rows with hundreds of terms each, 12 us of one SM's FP64 pipe for ten of them,
 // go to different SMs).  The row's shift m is the largest exponent
 // of the chunk with the largest bound, then of any chunk whose bound lies more
-// than 30 above it, so every exponent stays below 30 plus the FP32 error.
+// than 30 above it, so every exponent stays below 30 plus the FP32 error.  Where that
+// error is in the hundreds (exponents of 1e9 and more) terms can leave the FP64
+// range; the warp of such a row redoes it with its FP64 maximum.
 // Surviving columns are collected per warp (ballot, shared-memory list of
 // kRowList, drained 32 at a time when full); the lists are then evaluated by the
 // whole CTA, so a row with hundreds of terms among rows of five (the edge of a
@@ -222,6 +224,8 @@ __global__ void __launch_bounds__(256) chunkmin32(const double* __restrict__ C, 
 // warp, the CTA's epilogue (some 150 of 16 clocks each); 24 rows per CTA put one
 // epilogue on each SM where 8 put three (3000 rows).
 constexpr int kRowList = 352;
+constexpr float kRowFarTol = 200.0f;  // an error that keeps every term between e^-200 and e^430
+constexpr unsigned kRowLeastHi = 123u << 20, kRowMostHi = 0x7ff00000u;  // high words of 2^-900 and infinity
 
 // pval [NW][kRowList + 32], slist likewise, and the chunks' maxima
 template <int NW>
@@ -275,10 +279,10 @@ __global__ void __launch_bounds__(NW * 32)
   const bool live = i < nrows && mhi != -INFINITY;  // warp-uniform
   const float* crow = C32 + (int64_t)(live ? i : 0) * nin;
   // bound of chunk c = lane mod 32 and its FP32 error (the roundings of k2, c, l and the fma)
-  auto bound = [&](int c, float& tol) {
+  auto bound = [&](int c, float& tol, float& q) {
     if (c >= nchunk) return -INFINITY;
     const float l = sLc[c];
-    const float q = c < 64 ? (c < 32 ? q4[0] : q4[1]) : c < 128 ? (c < 96 ? q4[2] : q4[3]) : cmin[c];
+    q = c < 64 ? (c < 32 ? q4[0] : q4[1]) : c < 128 ? (c < 96 ? q4[2] : q4[3]) : cmin[c];
     const float b = fmaf(-k2f, q, l);
     tol = fmaf(fabsf(b) + fmaf(k2f, fabsf(q), fabsf(l)), 0x1p-22f, lerr);
     return b;
@@ -303,6 +307,7 @@ __global__ void __launch_bounds__(NW * 32)
     }
   };
   float m = -INFINITY, best = -INFINITY;
+  float mneg = 0.0f;  // costs below zero: the parts of the shift's exponent may cancel
   if (live) {
     int jj[8];
     float tt[8], mg[8];
@@ -314,9 +319,11 @@ __global__ void __launch_bounds__(NW * 32)
       return wmax(g);
     };
     int at = 0;
+    float qmin = 0.0f;
     for (int c = lane; c < nchunk; c += 32) {
-      float tol;
-      const float b = bound(c, tol);
+      float tol, q;
+      const float b = bound(c, tol, q);
+      qmin = fminf(qmin, q);
       if (b > best) {
         best = b;
         at = c;
@@ -331,6 +338,7 @@ __global__ void __launch_bounds__(NW * 32)
         at = c;
       }
     }
+    if (__any_sync(0xffffffffu, qmin < 0.0f)) mneg = 2.0f * k2f * wmax(-qmin) * 0x1p-22f;
     if (best != -INFINITY) {
       // that chunk and its neighbours: on a steep line over sorted points all bounds near the
       // largest are loose, and the row's maximum lies a few chunks away
@@ -338,8 +346,8 @@ __global__ void __launch_bounds__(NW * 32)
       for (int u = 0; u < 8; ++u) jj[u] = 32 * (at + u - 4) + lane;
       m = largest();
       for (int c0 = 0; c0 < nchunk; c0 += 32) {
-        float tol = 0.0f;
-        const float b = bound(c0 + lane, tol);
+        float tol = 0.0f, q;
+        const float b = bound(c0 + lane, tol, q);
         unsigned mask = __ballot_sync(0xffffffffu, b - tol > m + 30.0f);
         while (mask) {  // eight chunks at a time for loads in flight
 #pragma unroll
@@ -358,17 +366,18 @@ __global__ void __launch_bounds__(NW * 32)
     return exp_tab(fma(-k2, C[ri * nin + j], L64[j] - sm_lmax) - (double)mr, tab);
   };
   double s = 0.0;
-  bool drained = false;
+  bool drained = false, far = !(mneg <= kRowFarTol);
+  const float lowest = -cut - mneg;
   int cnt = 0;  // warp-uniform
   int* lst = slist + warp * (kRowList + 32);
   if (live && m != -INFINITY) {
     // warp-uniform sweep over the surviving chunks
     constexpr int G = 4;
     for (int c0 = 0; c0 < nchunk; c0 += 32) {
-      float ctol = 0.0f;
-      const float b = bound(c0 + lane, ctol);
+      float ctol = 0.0f, q;
+      const float b = bound(c0 + lane, ctol, q);
       const float a = b - m;
-      unsigned mask = __ballot_sync(0xffffffffu, a > -cut - fmaf(fabsf(a), 0x1p-22f, ctol));
+      unsigned mask = __ballot_sync(0xffffffffu, a > lowest - fmaf(fabsf(a), 0x1p-22f, ctol));
       while (mask) {
         int cj[G];
         float t[G], mag[G];
@@ -381,9 +390,11 @@ __global__ void __launch_bounds__(NW * 32)
 #pragma unroll
         for (int u = 0; u < G; ++u) {
           const float d = t[u] - m;
-          // |t - t_FP64| and the error of m are below (k2 c + |l| + |t| + |d|) 2^-22 plus lerr
+          // |t - t_FP64| and the error of m are below (k2 |c| + |l| + |t| + |d|) 2^-22 plus lerr
+          // (and mneg): |m| <= |t| + |d|, and the two parts of an exponent have one sign
           const float tol = fmaf(fabsf(t[u]) + fabsf(d) + mag[u], 0x1p-22f, lerr);
-          const bool keep = cj[u] < nin && d > -cut - tol;
+          const bool keep = cj[u] < nin && d > lowest - tol;
+          far = far || (keep && !(tol <= kRowFarTol));
           const unsigned km = __ballot_sync(0xffffffffu, keep);
           if (!km) continue;
           if (keep) lst[cnt + __popc(km & ((1u << lane) - 1u))] = cj[u];
@@ -436,6 +447,25 @@ __global__ void __launch_bounds__(NW * 32)
     t = wsum(t);
     if (lane == 0) sm_s[warp] = s + t;
   }
+  if (__any_sync(0xffffffffu, far)) {
+    // the largest term's high word (terms are not negative; integer instructions only)
+    unsigned hi = drained ? (unsigned)__double2hiint(s) : 0u;
+    for (int k = woff[warp] + lane; k < woff[warp + 1]; k += 32) hi = max(hi, (unsigned)__double2hiint(pval[k]));
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (hi < kRowLeastHi || hi >= kRowMostHi) {
+      const double* c64 = C + (int64_t)i * nin;
+      double mx = -kInf, t = 0.0;
+      for (int j = lane; j < nin; j += 32) mx = fmax(mx, fma(-k2, c64[j], L64[j] - sm_lmax));
+      mx = wmax(mx);
+      if (mx != -kInf)
+        for (int j = lane; j < nin; j += 32) t += exp_tab(fma(-k2, c64[j], L64[j] - sm_lmax) - mx, tab);
+      t = wsum(t);
+      if (lane == 0) {
+        sm_m[warp] = __int_as_float(0x7fc00000);  // sm_s holds the row's result
+        sm_s[warp] = (mx == -kInf) ? -kInf : sm_lmax + mx + log(t);
+      }
+    }
+  }
   __syncthreads();
   // the CTA's row epilogues (FP64 log and Table 1 row) side by side in the
   // lanes of warp 0: one warp instruction stream for NW rows instead of one
@@ -447,9 +477,13 @@ __global__ void __launch_bounds__(NW * 32)
       double z = -kInf;
       const float mr = sm_m[lane];
       double t = sm_s[lane];
-      if (woff[lane + 1] - woff[lane] <= kLaneTerms)
-        for (int k = woff[lane]; k < woff[lane + 1]; ++k) t += pval[k];
-      if (mr != -INFINITY) z = sm_lmax + (double)mr + log(t);
+      if (mr != mr) {
+        z = t;
+      } else if (mr != -INFINITY) {
+        if (woff[lane + 1] - woff[lane] <= kLaneTerms)
+          for (int k = woff[lane]; k < woff[lane + 1]; ++k) t += pval[k];
+        z = sm_lmax + (double)mr + log(t);
+      }
       apply_epilogue(epi, 0, r, z, num, den);
     }
   }
