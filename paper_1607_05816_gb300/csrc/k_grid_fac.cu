@@ -174,7 +174,10 @@ __global__ void __launch_bounds__(kTile * TL * KS) grid_pass_f64(Fac64Args a, Ep
           m = fmax(m, e);
         }
         m = wmax_d(m);
-        for (int j = lane; j < nc; j += 32) A[j] = (m == -kInf) ? 0.0 : exp(A[j] - m);
+        for (int j = lane; j < nc; j += 32) {
+          const double e = A[j];
+          A[j] = (m == -kInf && e == e) ? 0.0 : exp(e - m);  // (a line of NaN alone has no maximum)
+        }
         __syncwarp();
         if (lane == 0) {
           sM[p] = m;
@@ -211,7 +214,7 @@ __global__ void __launch_bounds__(kTile * TL * KS) grid_pass_f64(Fac64Args a, Ep
         for (int q = 1; q < KS; ++q) s += red[tid + q * kTile * TL];
     }
     const double m = sM[pair];
-    if (ks == 0 && m != -kInf) z = m + log(s);
+    if (ks == 0 && (m != -kInf || s != s)) z = m + log(s);
   } else {
     // plain log-sum-exp: shifted by the previous result where there is one (one
     // sweep), redone with running maxima if a sum leaves [1e-290, 1e290]
@@ -237,7 +240,7 @@ __global__ void __launch_bounds__(kTile * TL * KS) grid_pass_f64(Fac64Args a, Ep
             cm = fmax(cm, Lp[j] - d * d * inv_eps);
           }
           if (cm > m) {
-            s = (m == -kInf) ? 0.0 : s * exp(m - cm);
+            s = (m == -kInf && s == s) ? 0.0 : s * exp(m - cm);
             m = cm;
           }
         }
@@ -246,6 +249,11 @@ __global__ void __launch_bounds__(kTile * TL * KS) grid_pass_f64(Fac64Args a, Ep
           for (int j = ja; j < jb; ++j) {
             const double d = x - sy[j];
             s += exp((Lp[j] - m) - d * d * inv_eps);
+          }
+        } else {
+          for (int j = ja; j < jb; ++j) {
+            const double d = x - sy[j], e = Lp[j] - d * d * inv_eps;
+            if (e != e) s = e;  // NaN has no maximum
           }
         }
       }
@@ -262,7 +270,9 @@ __global__ void __launch_bounds__(kTile * TL * KS) grid_pass_f64(Fac64Args a, Ep
           s = 0.0;
           for (int q = 0; q < KS; ++q) {
             const double mq = rm[tid + q * kTile * TL];
-            if (mq != -kInf) s += (mq == m) ? rs[tid + q * kTile * TL] : rs[tid + q * kTile * TL] * exp(mq - m);
+            const double sq = rs[tid + q * kTile * TL];
+            if (mq == -kInf) s += (sq != sq) ? sq : 0.0;
+            else s += (mq == m) ? sq : sq * exp(mq - m);
           }
         }
       }
@@ -270,7 +280,7 @@ __global__ void __launch_bounds__(kTile * TL * KS) grid_pass_f64(Fac64Args a, Ep
         exact = true;
         continue;
       }
-      if (ks == 0 && m != -kInf) z = m + log(s);
+      if (ks == 0 && (m != -kInf || s != s)) z = m + log(s);
       break;
     }
     if (zp && own && ks == 0) *zp = (float)z;
@@ -304,10 +314,17 @@ __global__ void __launch_bounds__(128) grid_pass_f64_few(Fac64Args a, Epilogue e
       return v - d * d * a.inv_eps;
     };
     double m = -kInf, s = 0.0;
-    for (int j = lane; j < a.nin; j += 32) m = fmax(m, expo(j));
+    bool nan = false;
+    for (int j = lane; j < a.nin; j += 32) {
+      const double e = expo(j);
+      nan = nan || e != e;
+      m = fmax(m, e);
+    }
     m = wmax_d(m);
     double z = -kInf;
-    if (m != -kInf) {
+    if (__any_sync(0xffffffffu, nan)) {
+      z = NAN;
+    } else if (m != -kInf) {
       for (int j = lane; j < a.nin; j += 32) s += exp(expo(j) - m);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);

@@ -167,7 +167,8 @@ __global__ void __launch_bounds__(WARPS * 32)
 // ---------------------------------------------------------------------------
 
 // L_j = W_j/eps + log w_j in FP64 (L64) and as a float-float pair (Lff); the
-// largest L of each chunk of 32 columns as a pair (Lch).
+// largest L of each chunk of 32 columns as a pair (Lch), +inf where one is NaN: the
+// maximum of a line then says so without a test of its own.
 __global__ void __launch_bounds__(256) prepare_L_chunks(const double* __restrict__ W, const double* __restrict__ logw,
                                                         int nin, double inv_eps, double* __restrict__ L64,
                                                         float2* __restrict__ Lff, float2* __restrict__ Lch) {
@@ -186,10 +187,12 @@ __global__ void __launch_bounds__(256) prepare_L_chunks(const double* __restrict
     Lff[j] = pair(L);
   }
   const double mx = wmax(L);
-  if ((threadIdx.x & 31) == 0 && j < nin) Lch[j >> 5] = pair(mx);
+  const bool nan = __any_sync(0xffffffffu, L != L);
+  if ((threadIdx.x & 31) == 0 && j < nin) Lch[j >> 5] = nan ? make_float2(INFINITY, 0.0f) : pair(mx);
 }
 
-// C32 = C rounded to FP32 and the least C32 of each chunk; one warp per (row, chunk).
+// C32 = C rounded to FP32 and the least C32 of each chunk (-inf where one is NaN);
+// one warp per (row, chunk).
 __global__ void __launch_bounds__(256) chunkmin32(const double* __restrict__ C, int64_t nrows, int nin, int nchunk,
                                                   float* __restrict__ C32, float* __restrict__ Cmin) {
   const int lane = threadIdx.x & 31;
@@ -200,6 +203,7 @@ __global__ void __launch_bounds__(256) chunkmin32(const double* __restrict__ C, 
     if (j < nin) {
       c = (float)C[i * nin + j];
       C32[i * nin + j] = c;
+      if (c != c) c = -INFINITY;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) c = fminf(c, __shfl_xor_sync(0xffffffffu, c, o));
@@ -276,6 +280,7 @@ __global__ void __launch_bounds__(NW * 32)
   // the pairs carry |L| 2^-47 of representation error besides the FP32 rounding
   const float lerr = (mhi == -INFINITY) ? 4.0f : fmaf(fabsf(mhi), 0x1p-44f, 4.0f);
   const float k2f = (float)k2;
+  // (mhi = +inf, a NaN on the line: no chunk has a finite bound below, and the epilogue says NaN)
   const bool live = i < nrows && mhi != -INFINITY;  // warp-uniform
   const float* crow = C32 + (int64_t)(live ? i : 0) * nin;
   // bound of chunk c = lane mod 32 and its FP32 error (the roundings of k2, c, l and the fma)
@@ -358,6 +363,7 @@ __global__ void __launch_bounds__(NW * 32)
           m = fmaxf(m, largest());
         }
       }
+      if (m == -INFINITY && best == INFINITY) m = 0.0f;  // NaN costs and nothing else
     }
   }
   // FP64 term of column j of CTA row r, relative to that row's shift mr
@@ -377,7 +383,7 @@ __global__ void __launch_bounds__(NW * 32)
       float ctol = 0.0f, q;
       const float b = bound(c0 + lane, ctol, q);
       const float a = b - m;
-      unsigned mask = __ballot_sync(0xffffffffu, a > lowest - fmaf(fabsf(a), 0x1p-22f, ctol));
+      unsigned mask = __ballot_sync(0xffffffffu, !(a <= lowest - fmaf(fabsf(a), 0x1p-22f, ctol)));  // (NaN counts)
       while (mask) {
         int cj[G];
         float t[G], mag[G];
@@ -393,7 +399,7 @@ __global__ void __launch_bounds__(NW * 32)
           // |t - t_FP64| and the error of m are below (k2 |c| + |l| + |t| + |d|) 2^-22 plus lerr
           // (and mneg): |m| <= |t| + |d|, and the two parts of an exponent have one sign
           const float tol = fmaf(fabsf(t[u]) + fabsf(d) + mag[u], 0x1p-22f, lerr);
-          const bool keep = cj[u] < nin && d > lowest - tol;
+          const bool keep = cj[u] < nin && !(d <= lowest - tol);
           far = far || (keep && !(tol <= kRowFarTol));
           const unsigned km = __ballot_sync(0xffffffffu, keep);
           if (!km) continue;
@@ -461,7 +467,7 @@ __global__ void __launch_bounds__(NW * 32)
         for (int j = lane; j < nin; j += 32) t += exp_tab(fma(-k2, c64[j], L64[j] - sm_lmax) - mx, tab);
       t = wsum(t);
       if (lane == 0) {
-        sm_m[warp] = __int_as_float(0x7fc00000);  // sm_s holds the row's result
+        sm_m[warp] = NAN;  // sm_s holds the row's result
         sm_s[warp] = (mx == -kInf) ? -kInf : sm_lmax + mx + log(t);
       }
     }
@@ -477,7 +483,9 @@ __global__ void __launch_bounds__(NW * 32)
       double z = -kInf;
       const float mr = sm_m[lane];
       double t = sm_s[lane];
-      if (mr != mr) {
+      if (sm_lmax == kInf) {
+        z = NAN;
+      } else if (mr != mr) {
         z = t;
       } else if (mr != -INFINITY) {
         if (woff[lane + 1] - woff[lane] <= kLaneTerms)
