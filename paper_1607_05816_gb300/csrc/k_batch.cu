@@ -649,15 +649,6 @@ int ctas_any(int d, int variant, int nmax, int mmax) {
   }
 }
 
-int sm_count() {
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return 0;
-  }
-  return sms;
-}
-
 struct BKey {
   int dev, d, nmax, mmax;
   bool operator<(const BKey& o) const {

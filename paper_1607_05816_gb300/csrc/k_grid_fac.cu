@@ -386,7 +386,7 @@ cudaError_t launch_grid_pass_f64(const double* in, const double* logw, int in_is
   a.zprev = zprev;
   a.use_prev = use_prev;
   const int64_t outs = (int64_t)nlines * nout;
-  if (!G && outs * nbatch <= 152 * 64 && nbatch <= 65535)
+  if (!G && outs * nbatch <= 64 * sm_count() && nbatch <= 65535)
     return launch_pdl(grid_pass_f64_few, dim3((unsigned)((outs + 3) / 4), nbatch), 128, a, epi, s);
   // Four slices of the inputs per output: 256 x 256, 51 us a pass (one slice 49,
   // eight 66); 300 x 300, 88 (one slice 128: the short last chunk's exponentials

@@ -211,9 +211,10 @@ __global__ void __launch_bounds__(256) chunkmin32(const double* __restrict__ C, 
   }
 }
 
-// One warp per row, NW rows per CTA (rows b, b + G, ... of G CTAs: neighbouring
+// WPR warps per row, NW / WPR rows per CTA (rows b, b + G, ... of G CTAs: neighbouring
 // rows with hundreds of terms each, 12 us of one SM's FP64 pipe for ten of them,
-// go to different SMs).  The row's shift m is the largest exponent
+// go to different SMs); chunk c belongs to warp c mod WPR of its row.  The row's
+// shift m is the largest exponent
 // of the chunk with the largest bound, then of any chunk whose bound lies more
 // than 30 above it, so every exponent stays below 30 plus the FP32 error.  Where that
 // error is in the hundreds (exponents of 1e9 and more) terms can leave the FP64
@@ -223,27 +224,30 @@ __global__ void __launch_bounds__(256) chunkmin32(const double* __restrict__ C, 
 // whole CTA, so a row with hundreds of terms among rows of five (the edge of a
 // density at small eps) does not wait for one warp's loads, and every sum is taken
 // in a fixed order.
+// Rows of at most kShortChunks chunks a warp (kShort) need no bounds: all their
+// exponents fit in registers, with the costs loaded before the preceding kernel has
+// ended (WF flow of 400 samples, two species, eps = 1e-8: 4.0 -> 3.5 ms).
 //
 // At small eps a pass is a chain of latencies and of FP64 instructions of one
-// warp, the CTA's epilogue (some 150 of 16 clocks each); 24 rows per CTA put one
-// epilogue on each SM where 8 put three (3000 rows).
+// warp, the CTA's epilogue (some 150 of 16 clocks each), so many rows share a CTA
+// where there are many.
 constexpr int kRowList = 352;
+constexpr int kShortChunks = 8;  // kShort: chunks per warp, their exponents in registers
 constexpr float kRowFarTol = 200.0f;  // an error that keeps every term between e^-200 and e^430
 constexpr unsigned kRowLeastHi = 123u << 20, kRowMostHi = 0x7ff00000u;  // high words of 2^-900 and infinity
 
-// pval [NW][kRowList + 32], slist likewise, and the chunks' maxima
-template <int NW>
-size_t rows_chunks_smem(int nchunk) {
-  return (size_t)NW * (kRowList + 32) * (sizeof(double) + sizeof(int)) + (size_t)nchunk * sizeof(float);
+// pval [nw][kRowList + 32], slist likewise, and the chunks' maxima
+size_t rows_chunks_smem(int nw, int nchunk) {
+  return (size_t)nw * (kRowList + 32) * (sizeof(double) + sizeof(int)) + (size_t)nchunk * sizeof(float);
 }
 
-template <int NW>
+template <int NW, int WPR, bool kShort>
 __global__ void __launch_bounds__(NW * 32)
     rows_lse_f64_chunks(const double* __restrict__ C, const float* __restrict__ C32, const float* __restrict__ Cmin,
                         int nrows, int nin, int nchunk, const double* __restrict__ L64,
                         const float2* __restrict__ Lff, const float2* __restrict__ Lch, double k2, float cut,
                         Epilogue epi) {
-  constexpr int NT = NW * 32;
+  constexpr int NT = NW * 32, RPC = NW / WPR;
   static_assert(NW <= 32 && NT >= kExpUnits, "a table entry a thread, a warp's lanes cover the rows");
   extern __shared__ double pval[];  // the terms of the lists, row by row
   int* slist = reinterpret_cast<int*>(pval + NW * (kRowList + 32));  // [NW][kRowList + 32] columns
@@ -253,16 +257,36 @@ __global__ void __launch_bounds__(NW * 32)
   __shared__ double sm_lmax;
   __shared__ int woff[33];          // exclusive prefix sum of the list lengths
   __shared__ double tab[kExpUnits];
+  __shared__ float sm_best[NW];     // WPR > 1: the warps' parts of what a row needs
+  __shared__ int sm_at[NW];
+  __shared__ float sm_neg[NW], sm_mx[NW];
+  __shared__ unsigned sm_hi[NW];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = blockIdx.x + warp * gridDim.x;
+  const int rloc = warp / WPR, part = warp % WPR;
+  const int i = blockIdx.x + rloc * gridDim.x;
   const float* cmin = Cmin + (int64_t)(i < nrows ? i : 0) * nchunk;
   // before the preceding kernel has ended: the table and the least costs of the first 128 chunks
   exp_table_load(tab);
-  float q4[4];
+  constexpr int kOwn = kShort ? kShortChunks : 1;
+  float q4[4], cs[kOwn];
 #pragma unroll
-  for (int u = 0; u < 4; ++u) q4[u] = (lane + 32 * u < nchunk) ? cmin[lane + 32 * u] : INFINITY;
+  for (int u = 0; u < (kShort ? 0 : 4); ++u) {
+    const int c = part + WPR * (lane + 32 * u);
+    q4[u] = c < nchunk ? cmin[c] : INFINITY;
+  }
+#pragma unroll
+  for (int u = 0; u < (kShort ? kOwn : 0); ++u) {
+    const int j = 32 * (part + WPR * u) + lane;
+    cs[u] = (i < nrows && j < nin) ? C32[(int64_t)i * nin + j] : INFINITY;
+  }
   pdl_wait();
   pdl_launch_dependents();
+  float2 ls[kOwn];
+#pragma unroll
+  for (int u = 0; u < (kShort ? kOwn : 0); ++u) {
+    const int j = 32 * (part + WPR * u) + lane;
+    ls[u] = j < nin ? Lff[j] : make_float2(-INFINITY, 0.0f);
+  }
   // mhi: the FP32 rounding of max L (the shift of the whole line)
   const float2 l0 = (threadIdx.x < nchunk) ? Lch[threadIdx.x] : make_float2(-INFINITY, 0.0f);
   float mhi = l0.x;
@@ -273,9 +297,11 @@ __global__ void __launch_bounds__(NW * 32)
 #pragma unroll
   for (int w = 0; w < NW; ++w) mhi = fmaxf(mhi, sm_m[w]);
   auto shifted = [&](float2 l) { return (mhi == -INFINITY || l.x == -INFINITY) ? -INFINITY : (l.x - mhi) + l.y; };
-  if (threadIdx.x < nchunk) sLc[threadIdx.x] = shifted(l0);
-  for (int c = threadIdx.x + NT; c < nchunk; c += NT) sLc[c] = shifted(Lch[c]);
   if (threadIdx.x == 0) sm_lmax = (mhi == -INFINITY) ? -kInf : (double)mhi;  // (a conversion takes the FP64 pipe)
+  if (!kShort) {
+    if (threadIdx.x < nchunk) sLc[threadIdx.x] = shifted(l0);
+    for (int c = threadIdx.x + NT; c < nchunk; c += NT) sLc[c] = shifted(Lch[c]);
+  }
   __syncthreads();
   // the pairs carry |L| 2^-47 of representation error besides the FP32 rounding
   const float lerr = (mhi == -INFINITY) ? 4.0f : fmaf(fabsf(mhi), 0x1p-44f, 4.0f);
@@ -283,11 +309,13 @@ __global__ void __launch_bounds__(NW * 32)
   // (mhi = +inf, a NaN on the line: no chunk has a finite bound below, and the epilogue says NaN)
   const bool live = i < nrows && mhi != -INFINITY;  // warp-uniform
   const float* crow = C32 + (int64_t)(live ? i : 0) * nin;
-  // bound of chunk c = lane mod 32 and its FP32 error (the roundings of k2, c, l and the fma)
-  auto bound = [&](int c, float& tol, float& q) {
+  // The warp's chunks are part, part + WPR, ...: bound of its e-th one (e = lane mod 32) and
+  // its FP32 error (the roundings of k2, c, l and the fma).
+  auto bound = [&](int e, float& tol, float& q) {
+    const int c = part + WPR * e;
     if (c >= nchunk) return -INFINITY;
     const float l = sLc[c];
-    q = c < 64 ? (c < 32 ? q4[0] : q4[1]) : c < 128 ? (c < 96 ? q4[2] : q4[3]) : cmin[c];
+    q = e < 64 ? (e < 32 ? q4[0] : q4[1]) : e < 128 ? (e < 96 ? q4[2] : q4[3]) : cmin[c];
     const float b = fmaf(-k2f, q, l);
     tol = fmaf(fabsf(b) + fmaf(k2f, fabsf(q), fabsf(l)), 0x1p-22f, lerr);
     return b;
@@ -311,27 +339,47 @@ __global__ void __launch_bounds__(NW * 32)
       mag[u] = fmaf(k2f, fabsf(cv[u]), fabsf(l));
     }
   };
+  double s = 0.0;
+  bool drained = false, far = false;
+  int cnt = 0;  // warp-uniform
+  int* lst = slist + warp * (kRowList + 32);
   float m = -INFINITY, best = -INFINITY;
   float mneg = 0.0f;  // costs below zero: the parts of the shift's exponent may cancel
-  if (live) {
-    int jj[8];
-    float tt[8], mg[8];
-    auto largest = [&]() {
-      exponents(jj, tt, mg);
-      float g = tt[0];
+  int jj[8];
+  float tt[8], mg[8];
+  auto largest = [&]() {
+    exponents(jj, tt, mg);
+    float g = tt[0];
 #pragma unroll
-      for (int u = 1; u < 8; ++u) g = fmaxf(g, tt[u]);
-      return wmax(g);
-    };
-    int at = 0;
+    for (int u = 1; u < 8; ++u) g = fmaxf(g, tt[u]);
+    return wmax(g);
+  };
+  int at = 0;
+  float ts[kOwn];
+  if (kShort) {  // every exponent of the row in registers
     float qmin = 0.0f;
-    for (int c = lane; c < nchunk; c += 32) {
+    bool nan = false;
+#pragma unroll
+    for (int u = 0; u < kOwn; ++u) {
+      const bool in = 32 * (part + WPR * u) + lane < nin;
+      ts[u] = in ? fmaf(-k2f, cs[u], shifted(ls[u])) : -INFINITY;
+      nan = nan || ts[u] != ts[u];
+      m = fmaxf(m, ts[u]);
+      qmin = fminf(qmin, cs[u]);
+    }
+    m = wmax(m);
+    if (__any_sync(0xffffffffu, nan)) m = fmaxf(m, 0.0f);  // (the row is NaN, with any shift)
+    if (__any_sync(0xffffffffu, qmin < 0.0f)) mneg = 2.0f * k2f * wmax(-qmin) * 0x1p-22f;
+    if (WPR > 1 && lane == 0) sm_neg[warp] = mneg;
+  } else if (live) {
+    float qmin = 0.0f;
+    for (int e = lane; part + WPR * e < nchunk; e += 32) {
       float tol, q;
-      const float b = bound(c, tol, q);
+      const float b = bound(e, tol, q);
       qmin = fminf(qmin, q);
       if (b > best) {
         best = b;
-        at = c;
+        at = part + WPR * e;
       }
     }
 #pragma unroll
@@ -344,42 +392,89 @@ __global__ void __launch_bounds__(NW * 32)
       }
     }
     if (__any_sync(0xffffffffu, qmin < 0.0f)) mneg = 2.0f * k2f * wmax(-qmin) * 0x1p-22f;
+  }
+  if (WPR > 1 && !kShort) {
+    if (lane == 0) {
+      sm_best[warp] = best;
+      sm_at[warp] = at;
+      sm_neg[warp] = mneg;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < WPR; ++w) {
+      const float b = sm_best[rloc * WPR + w];
+      const int c = sm_at[rloc * WPR + w];
+      if (b > best || (b == best && c < at)) {
+        best = b;
+        at = c;
+      }
+      mneg = fmaxf(mneg, sm_neg[rloc * WPR + w]);
+    }
+  }
+  if (!kShort && live) {
     if (best != -INFINITY) {
       // that chunk and its neighbours: on a steep line over sorted points all bounds near the
       // largest are loose, and the row's maximum lies a few chunks away
 #pragma unroll
       for (int u = 0; u < 8; ++u) jj[u] = 32 * (at + u - 4) + lane;
       m = largest();
-      for (int c0 = 0; c0 < nchunk; c0 += 32) {
+      for (int c0 = 0; part + WPR * c0 < nchunk; c0 += 32) {
         float tol = 0.0f, q;
         const float b = bound(c0 + lane, tol, q);
         unsigned mask = __ballot_sync(0xffffffffu, b - tol > m + 30.0f);
         while (mask) {  // eight chunks at a time for loads in flight
 #pragma unroll
           for (int u = 0; u < 8; ++u) {
-            jj[u] = mask ? 32 * (c0 + __ffs(mask) - 1) + lane : nin;
+            jj[u] = mask ? 32 * (part + WPR * (c0 + __ffs(mask) - 1)) + lane : nin;
             mask &= mask - 1;  // 0 stays 0
           }
           m = fmaxf(m, largest());
         }
       }
-      if (m == -INFINITY && best == INFINITY) m = 0.0f;  // NaN costs and nothing else
     }
   }
-  // FP64 term of column j of CTA row r, relative to that row's shift mr
+  if (WPR > 1) {
+    if (lane == 0) sm_mx[warp] = m;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < WPR; ++w) {
+      m = fmaxf(m, sm_mx[rloc * WPR + w]);
+      if (kShort) mneg = fmaxf(mneg, sm_neg[rloc * WPR + w]);
+    }
+  }
+  if (m == -INFINITY && best == INFINITY) m = 0.0f;  // NaN costs and nothing else
+  // FP64 term of column j of the row of warp r, relative to that row's shift mr
   auto term = [&](int r, int j, float mr) {
-    const int64_t ri = (int64_t)(blockIdx.x + r * gridDim.x);
+    const int64_t ri = (int64_t)(blockIdx.x + r / WPR * gridDim.x);
     return exp_tab(fma(-k2, C[ri * nin + j], L64[j] - sm_lmax) - (double)mr, tab);
   };
-  double s = 0.0;
-  bool drained = false, far = !(mneg <= kRowFarTol);
+  far = !(mneg <= kRowFarTol);
   const float lowest = -cut - mneg;
-  int cnt = 0;  // warp-uniform
-  int* lst = slist + warp * (kRowList + 32);
-  if (live && m != -INFINITY) {
+  // |t - t_FP64| and the error of m are below (k2 |c| + |l| + |t| + |d|) 2^-22 plus lerr
+  // (and mneg): |m| <= |t| + |d|, and the two parts of an exponent have one sign
+  auto keeps = [&](float t, float mag) {
+    const float d = t - m;
+    const float tol = fmaf(fabsf(t) + fabsf(d) + mag, 0x1p-22f, lerr);
+    const bool keep = !(d <= lowest - tol);
+    far = far || (keep && !(tol <= kRowFarTol));
+    return keep;
+  };
+  auto append = [&](bool keep, int j) {
+    const unsigned km = __ballot_sync(0xffffffffu, keep);
+    if (keep) lst[cnt + __popc(km & ((1u << lane) - 1u))] = j;
+    cnt += __popc(km);
+  };
+  if (kShort && m != -INFINITY) {
+#pragma unroll
+    for (int u = 0; u < kOwn; ++u) {
+      const int j = 32 * (part + WPR * u) + lane;
+      append(j < nin && keeps(ts[u], fmaf(k2f, fabsf(cs[u]), fabsf(shifted(ls[u])))), j);
+    }
+  }
+  if (!kShort && live && m != -INFINITY) {
     // warp-uniform sweep over the surviving chunks
     constexpr int G = 4;
-    for (int c0 = 0; c0 < nchunk; c0 += 32) {
+    for (int c0 = 0; part + WPR * c0 < nchunk; c0 += 32) {
       float ctol = 0.0f, q;
       const float b = bound(c0 + lane, ctol, q);
       const float a = b - m;
@@ -389,22 +484,13 @@ __global__ void __launch_bounds__(NW * 32)
         float t[G], mag[G];
 #pragma unroll
         for (int u = 0; u < G; ++u) {
-          cj[u] = mask ? 32 * (c0 + __ffs(mask) - 1) + lane : nin;
+          cj[u] = mask ? 32 * (part + WPR * (c0 + __ffs(mask) - 1)) + lane : nin;
           mask &= mask - 1;  // 0 stays 0
         }
         exponents(cj, t, mag);
 #pragma unroll
         for (int u = 0; u < G; ++u) {
-          const float d = t[u] - m;
-          // |t - t_FP64| and the error of m are below (k2 |c| + |l| + |t| + |d|) 2^-22 plus lerr
-          // (and mneg): |m| <= |t| + |d|, and the two parts of an exponent have one sign
-          const float tol = fmaf(fabsf(t[u]) + fabsf(d) + mag[u], 0x1p-22f, lerr);
-          const bool keep = cj[u] < nin && !(d <= lowest - tol);
-          far = far || (keep && !(tol <= kRowFarTol));
-          const unsigned km = __ballot_sync(0xffffffffu, keep);
-          if (!km) continue;
-          if (keep) lst[cnt + __popc(km & ((1u << lane) - 1u))] = cj[u];
-          cnt += __popc(km);
+          append(cj[u] < nin && keeps(t[u], mag[u]), cj[u]);
           if (cnt > kRowList) {  // a full batch from the list's end: every lane evaluates one term
             __syncwarp();
             cnt -= 32;
@@ -444,52 +530,77 @@ __global__ void __launch_bounds__(NW * 32)
     pval[k] = term(r, slist[r * (kRowList + 32) + k - woff[r]], sm_m[r]);
   }
   __syncthreads();
-  // rows of more than kLaneTerms terms are summed by their warps, the others by the
-  // epilogue's lanes (a warp's sum takes five FP64 instructions whatever its length)
-  constexpr int kLaneTerms = 8;
+  // Lists of more than kLaneTerms terms are summed by their warps; where a row has one warp, the
+  // others by the epilogue's lanes (a warp's sum takes five FP64 instructions whatever its length).
+  constexpr int kLaneTerms = WPR > 1 ? 0 : 8;
   if (cnt > kLaneTerms) {
     double t = 0.0;
     for (int k = woff[warp] + lane; k < woff[warp + 1]; k += 32) t += pval[k];
     t = wsum(t);
     if (lane == 0) sm_s[warp] = s + t;
   }
-  if (__any_sync(0xffffffffu, far)) {
-    // the largest term's high word (terms are not negative; integer instructions only)
+  auto redo_outside_range = [&](unsigned hi) {  // hi: the high word of the row's largest term
+    if (hi >= kRowLeastHi && hi < kRowMostHi) return;
+    const double* c64 = C + (int64_t)i * nin;
+    double mx = -kInf, t = 0.0;
+    bool nan = false;
+    for (int j = lane; j < nin; j += 32) {
+      const double a = fma(-k2, c64[j], L64[j] - sm_lmax);
+      nan = nan || a != a;
+      mx = fmax(mx, a);
+    }
+    mx = wmax(mx);
+    nan = __any_sync(0xffffffffu, nan);
+    if (mx != -kInf && !nan)
+      for (int j = lane; j < nin; j += 32) t += exp_tab(fma(-k2, c64[j], L64[j] - sm_lmax) - mx, tab);
+    t = wsum(t);
+    if (lane == 0) {
+      sm_m[warp] = NAN;  // sm_s holds the row's result
+      sm_s[warp] = nan ? (double)NAN : mx == -kInf ? -kInf : sm_lmax + mx + log(t);
+    }
+  };
+  auto largest_hi = [&]() {  // of the warp's terms (not negative; integer instructions only)
     unsigned hi = drained ? (unsigned)__double2hiint(s) : 0u;
     for (int k = woff[warp] + lane; k < woff[warp + 1]; k += 32) hi = max(hi, (unsigned)__double2hiint(pval[k]));
-    hi = __reduce_max_sync(0xffffffffu, hi);
-    if (hi < kRowLeastHi || hi >= kRowMostHi) {
-      const double* c64 = C + (int64_t)i * nin;
-      double mx = -kInf, t = 0.0;
-      for (int j = lane; j < nin; j += 32) mx = fmax(mx, fma(-k2, c64[j], L64[j] - sm_lmax));
-      mx = wmax(mx);
-      if (mx != -kInf)
-        for (int j = lane; j < nin; j += 32) t += exp_tab(fma(-k2, c64[j], L64[j] - sm_lmax) - mx, tab);
-      t = wsum(t);
-      if (lane == 0) {
-        sm_m[warp] = NAN;  // sm_s holds the row's result
-        sm_s[warp] = (mx == -kInf) ? -kInf : sm_lmax + mx + log(t);
-      }
+    return __reduce_max_sync(0xffffffffu, hi);
+  };
+  if (WPR == 1) {
+    if (__any_sync(0xffffffffu, far)) redo_outside_range(largest_hi());
+    __syncthreads();
+  } else if (__syncthreads_or(far)) {
+    const unsigned hi = largest_hi();
+    if (lane == 0) sm_hi[warp] = hi;
+    __syncthreads();
+    if (part == 0 && live && m != -INFINITY) {
+      unsigned top = hi;
+#pragma unroll
+      for (int w = 1; w < WPR; ++w) top = max(top, sm_hi[rloc * WPR + w]);
+      redo_outside_range(top);
     }
+    __syncthreads();
   }
-  __syncthreads();
   // the CTA's row epilogues (FP64 log and Table 1 row) side by side in the
-  // lanes of warp 0: one warp instruction stream for NW rows instead of one
+  // lanes of warp 0: one warp instruction stream for RPC rows instead of one
   // per row on the narrow FP64 pipe
   double num = 0.0, den = 0.0;
-  if (warp == 0 && lane < NW) {
+  if (warp == 0 && lane < RPC) {
     const int r = blockIdx.x + lane * gridDim.x;
     if (r < nrows) {
       double z = -kInf;
-      const float mr = sm_m[lane];
-      double t = sm_s[lane];
+      const float mr = sm_m[lane * WPR];
+      double t = sm_s[lane * WPR];
       if (sm_lmax == kInf) {
         z = NAN;
       } else if (mr != mr) {
         z = t;
       } else if (mr != -INFINITY) {
-        if (woff[lane + 1] - woff[lane] <= kLaneTerms)
-          for (int k = woff[lane]; k < woff[lane + 1]; ++k) t += pval[k];
+        if (WPR == 1) {
+          if (woff[lane + 1] - woff[lane] <= kLaneTerms)
+            for (int k = woff[lane]; k < woff[lane + 1]; ++k) t += pval[k];
+        } else {
+#pragma unroll
+          for (int w = 1; w < WPR; ++w) t += sm_s[lane * WPR + w];
+        }
         z = sm_lmax + (double)mr + log(t);
       }
       apply_epilogue(epi, 0, r, z, num, den);
@@ -769,7 +880,7 @@ size_t rows_chunks_scratch_bytes(int64_t nin) {
 cudaError_t launch_chunkmin32(const double* C, int64_t nrows, int nin, float* C32, float* Cmin, cudaStream_t s) {
   const int nchunk = (int)rows_chunks(nin);
   count_launches(1);
-  chunkmin32<<<(unsigned)std::min<int64_t>((nrows * nchunk + 7) / 8, 152 * 64), 256, 0, s>>>(C, nrows, nin, nchunk, C32,
+  chunkmin32<<<(unsigned)std::min<int64_t>((nrows * nchunk + 7) / 8, 64 * sm_count()), 256, 0, s>>>(C, nrows, nin, nchunk, C32,
                                                                                          Cmin);
   return cudaGetLastError();
 }
@@ -824,17 +935,32 @@ cudaError_t launch_rows(int prec, const RowsGeom& g, int nrows, int nin, const d
                                  L64, Lff, Lch);
       if (e != cudaSuccess) return e;
       prof_mark_begin(PROF_ROWS, s);
-      auto run = [&](auto kern, int nw) -> cudaError_t {
-        const size_t smem = nw == 8 ? rows_chunks_smem<8>(nchunk) : rows_chunks_smem<24>(nchunk);
+      auto run = [&](auto kern, int nw, int rpc) -> cudaError_t {
+        const size_t smem = rows_chunks_smem(nw, nchunk);
         const cudaError_t e0 = smem_at_least(kern, smem);
         if (e0 != cudaSuccess) return e0;
         const double* l64 = L64;
         const float2 *lff = Lff, *lch = Lch;
-        return launch_pdl(kern, dim3((nrows + nw - 1) / nw), dim3(nw * 32), smem, s, C, g.C32,
+        return launch_pdl(kern, dim3((nrows + rpc - 1) / rpc), dim3(nw * 32), smem, s, C, g.C32,
                           g.Cmin, nrows, nin, nchunk, l64, lff, lch, 1.0 / eps, 50.0f + logf((float)nin), epi);
       };
-      // rows beyond one 8-row CTA per SM: 24 per CTA (fewer epilogues)
-      e = nrows <= 8 * 152 ? run(&rows_lse_f64_chunks<8>, 8) : run(&rows_lse_f64_chunks<24>, 24);
+      // Warps per row, so that few rows still fill the GPU (one warp a row left 1 x 300000
+      // at 2.3 times the time of the four-warp kernel before, 300 x 300 at 1.17).  Times of
+      // 20 iterations with 1, 2, 4 warps: 300 rows 1.19, 0.90, 0.80 ms; 400 rows (WF, eps
+      // 1e-3) 2.7, 2.2, 2.2; 1216 rows 3.5, 3.0, 2.6 at eps 1e-2 but 2.2, 2.3, 2.6 (WF, 1e-8);
+      // 3000 rows (WF, 1e-8) 3.2, 4.1, 5.0.  152 rows of 30000 columns: 4 warps 1.16 ms, 16 0.69.
+      const int sms = sm_count();
+      auto by_length = [&](auto shrt, auto lng, int nw, int wpr) {
+        return nchunk <= kShortChunks * wpr ? run(shrt, nw, nw / wpr) : run(lng, nw, nw / wpr);
+      };
+      if (nrows <= sms && nchunk >= 128)
+        e = run(&rows_lse_f64_chunks<16, 16, false>, 16, 1);
+      else if (nrows <= 2 * sms)
+        e = by_length(&rows_lse_f64_chunks<8, 4, true>, &rows_lse_f64_chunks<8, 4, false>, 8, 4);
+      else if (nrows <= 8 * sms)
+        e = by_length(&rows_lse_f64_chunks<8, 2, true>, &rows_lse_f64_chunks<8, 2, false>, 8, 2);
+      else
+        e = by_length(&rows_lse_f64_chunks<8, 1, true>, &rows_lse_f64_chunks<8, 1, false>, 8, 1);
       if (e != cudaSuccess) return e;
       prof_mark_end(PROF_ROWS, s);
       return cudaGetLastError();

@@ -506,6 +506,16 @@ cudaError_t smem_at_least(K* kernel, size_t bytes) {
   return smem_limit_at_least(reinterpret_cast<const void*>(kernel), bytes);
 }
 
+// SMs of the current device (0 if it cannot be asked).
+inline int sm_count() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 0;
+  }
+  return sms;
+}
+
 // Launch with programmatic dependent launch: the kernel may start while its
 // predecessor drains; it waits for it (pdl_wait) before reading anything the
 // predecessor writes.
