@@ -236,9 +236,14 @@ constexpr int kShortChunks = 8;  // kShort: chunks per warp, their exponents in 
 constexpr float kRowFarTol = 200.0f;  // an error that keeps every term between e^-200 and e^430
 constexpr unsigned kRowLeastHi = 123u << 20, kRowMostHi = 0x7ff00000u;  // high words of 2^-900 and infinity
 
+// Chunks' maxima kept in shared memory (48 KB, 393,216 columns); those of later chunks
+// are read from L2 where they are used.
+constexpr int kStagedChunks = 12288;
+
 // pval [nw][kRowList + 32], slist likewise, and the chunks' maxima
 size_t rows_chunks_smem(int nw, int nchunk) {
-  return (size_t)nw * (kRowList + 32) * (sizeof(double) + sizeof(int)) + (size_t)nchunk * sizeof(float);
+  return (size_t)nw * (kRowList + 32) * (sizeof(double) + sizeof(int)) +
+         (size_t)std::min(nchunk, kStagedChunks) * sizeof(float);
 }
 
 template <int NW, int WPR, bool kShort>
@@ -251,7 +256,7 @@ __global__ void __launch_bounds__(NW * 32)
   static_assert(NW <= 32 && NT >= kExpUnits, "a table entry a thread, a warp's lanes cover the rows");
   extern __shared__ double pval[];  // the terms of the lists, row by row
   int* slist = reinterpret_cast<int*>(pval + NW * (kRowList + 32));  // [NW][kRowList + 32] columns
-  float* sLc = reinterpret_cast<float*>(slist + NW * (kRowList + 32));  // [nchunk] largest input, relative to the line's
+  float* sLc = reinterpret_cast<float*>(slist + NW * (kRowList + 32));  // largest inputs, relative to the line's
   __shared__ float sm_m[NW];        // the rows' shifts
   __shared__ double sm_s[NW];
   __shared__ double sm_lmax;
@@ -300,7 +305,7 @@ __global__ void __launch_bounds__(NW * 32)
   if (threadIdx.x == 0) sm_lmax = (mhi == -INFINITY) ? -kInf : (double)mhi;  // (a conversion takes the FP64 pipe)
   if (!kShort) {
     if (threadIdx.x < nchunk) sLc[threadIdx.x] = shifted(l0);
-    for (int c = threadIdx.x + NT; c < nchunk; c += NT) sLc[c] = shifted(Lch[c]);
+    for (int c = threadIdx.x + NT; c < min(nchunk, kStagedChunks); c += NT) sLc[c] = shifted(Lch[c]);
   }
   __syncthreads();
   // the pairs carry |L| 2^-47 of representation error besides the FP32 rounding
@@ -314,7 +319,7 @@ __global__ void __launch_bounds__(NW * 32)
   auto bound = [&](int e, float& tol, float& q) {
     const int c = part + WPR * e;
     if (c >= nchunk) return -INFINITY;
-    const float l = sLc[c];
+    const float l = c < kStagedChunks ? sLc[c] : shifted(Lch[c]);
     q = e < 64 ? (e < 32 ? q4[0] : q4[1]) : e < 128 ? (e < 96 ? q4[2] : q4[3]) : cmin[c];
     const float b = fmaf(-k2f, q, l);
     tol = fmaf(fabsf(b) + fmaf(k2f, fabsf(q), fabsf(l)), 0x1p-22f, lerr);
@@ -922,9 +927,8 @@ cudaError_t launch_rows(int prec, const RowsGeom& g, int nrows, int nin, const d
     double* Lt = (double*)scratch_L;
     double* Lmax = (double*)((char*)scratch_L + (((size_t)nin * 8 + 255) & ~(size_t)255));
     const double* C = (const double*)g.C;
-    // dense rows with an FP32 copy of C (k2 = 1/eps must stay an FP32 number; the chunks'
-    // bounds, 48 KB for 393,216 columns, must fit in shared memory)
-    if (g.kind == UOT_GEOM_DENSE && g.C32 && 1.0 / eps < 1e30 && rows_chunks(nin) <= 12288) {
+    // dense rows with an FP32 copy of C (k2 = 1/eps must stay an FP32 number)
+    if (g.kind == UOT_GEOM_DENSE && g.C32 && 1.0 / eps < 1e30) {
       char* base = (char*)scratch_L;
       const size_t r8 = ((size_t)nin * 8 + 255) & ~(size_t)255;
       double* L64 = (double*)base;
