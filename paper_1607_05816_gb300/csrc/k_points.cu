@@ -12,10 +12,10 @@
 //    eps needs a second sweep for the maxima, 22 of the 80 passes of a solve of
 //    10 stages); a warp whose partial sum overflows redoes the chunk with the
 //    exact chunk maximum.  Writes (shift, sum) per (chunk, output).
-//  points_combine: one thread per output merges the chunks' pairs; where the
-//    merged sum underflowed (shift far above the result) a warp recomputes
-//    that output exactly over all inputs; then the epilogue (Table 1 row,
-//    violation terms) runs on the float-float result, 32 outputs a warp.
+//  points_combine: one thread per output (a warp where outputs are few and chunks
+//    many) merges the chunks' pairs; where the merged sum underflowed (shift far
+//    above the result) a warp recomputes that output exactly over all inputs; then
+//    the epilogue (Table 1 row, violation terms) runs on the float-float result.
 //
 // points_blockmax and points_combine are launched while their predecessors run
 // (programmatic dependent launch).
@@ -226,14 +226,17 @@ struct CombArgs {
   float* zprev;  // written (NULL: not kept)
 };
 
-// One thread per output: merge chunk partials, exact recomputation (by the
-// thread's warp) if the merged sum underflowed, then the epilogue.
+// T threads per output (1, or a warp where outputs are few and chunks many): merge chunk
+// partials, exact recomputation (by the thread's warp) if the merged sum underflowed, then
+// the epilogue.
 constexpr int kCombThreads = 128;
 
+template <int T>
 __global__ void __launch_bounds__(kCombThreads)
     points_combine(CombArgs a, Epilogue epi) {
   const int lane = threadIdx.x & 31;
-  const int i = blockIdx.x * kCombThreads + threadIdx.x;
+  const int i = (blockIdx.x * kCombThreads + threadIdx.x) / T;
+  const int c0 = T == 1 ? 0 : lane;
   const bool owns = i < a.nout;
   float num = 0.0f, den = 0.0f;
   pdl_wait();
@@ -242,23 +245,28 @@ __global__ void __launch_bounds__(kCombThreads)
   float M = -INFINITY, S = 0.0f;
   if (owns) {
 #pragma unroll 4
-    for (int c = 0; c < a.nchunks; ++c) {
+    for (int c = c0; c < a.nchunks; c += T) {
       const float2 pr = a.part[(int64_t)c * a.nout + i];
       if (pr.y > 0.0f) M = fmaxf(M, pr.x);
     }
+    if (T > 1) M = warp_maxf(M);
     if (M != -INFINITY) {
 #pragma unroll 4
-      for (int c = 0; c < a.nchunks; ++c) {
+      for (int c = c0; c < a.nchunks; c += T) {
         const float2 pr = a.part[(int64_t)c * a.nout + i];
         if (pr.y > 0.0f) S += pr.y * ex2_approx(pr.x - M);
       }
     }
+    if (T > 1)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) S += __shfl_xor_sync(0xffffffffu, S, o);
   }
   // the shift was far above the result: exact log-sum-exp over all inputs
   unsigned redo = __ballot_sync(0xffffffffu, owns && !(S >= 0x1p-90f) && Lmax != -INFINITY);
+  if (T > 1) redo &= 1u;  // one output
   for (; redo; redo &= redo - 1) {
     const int src = __ffs(redo) - 1;
-    const int io = i - lane + src;
+    const int io = T > 1 ? i : i - lane + src;
     float xi[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) xi[k] = (k < a.d) ? a.x[(int64_t)io * a.d + k] : 0.0f;
@@ -285,7 +293,7 @@ __global__ void __launch_bounds__(kCombThreads)
       S = s;
     }
   }
-  if (owns) {
+  if (owns && (T == 1 || lane == 0)) {
     ff z = ff_ninf();
     if (Lmax != -INFINITY && M != -INFINITY && S > 0.0f) z = pass_result(Lmax, M, S);
     if (a.zprev) a.zprev[i] = z.hi;
@@ -504,7 +512,18 @@ cudaError_t launch_points(const float* x, const float* y, int d, int nout, int n
   b.k2 = a.k2;
   b.part = part;
   b.zprev = zprev;
-  e = launch_pdl(points_combine, dim3((nout + kCombThreads - 1) / kCombThreads), dim3(kCombThreads), 0, s, b, epi);
+  // One thread per output reads its chunks one after the other, a latency each: 100 outputs
+  // and 5,000,000 inputs 2.69 ms a call, 2.01 with a warp per output (100 and 300,000: 364
+  // and 318 us; 4000 and 100,000: 432 and 415).  With outputs enough to fill the GPU the
+  // warps only repeat work: 8000 and 100,000 569 and 581 us, 20000 and 100,000 1018 and 1044;
+  // nor do they help with few chunks (1000 and 20,000: 278 and 285).  The warp form is not
+  // launched early: 100 and 5,000,000 then takes 2.17 ms.
+  if (nout <= 32 * sm_count() && nchunks >= 64) {
+    points_combine<32><<<(nout + kCombThreads / 32 - 1) / (kCombThreads / 32), kCombThreads, 0, s>>>(b, epi);
+    e = cudaGetLastError();
+  } else {
+    e = launch_pdl(points_combine<1>, dim3((nout + kCombThreads - 1) / kCombThreads), dim3(kCombThreads), 0, s, b, epi);
+  }
   if (e != cudaSuccess) return e;
   prof_mark_end(PROF_ROWS, s);
   return cudaGetLastError();
