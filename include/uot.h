@@ -288,6 +288,21 @@ uot_status uot_force_batch_warps(int warps);
 uot_status uot_force_batch_cluster(int ctas);
 
 /*
+ * uot_set_stored_kernel_limit(bytes) -- device memory of the stored FP64 kernels.
+ * uot_solve, uot_solve_mass, uot_wf_flow (one species) and the other single-problem
+ * solvers on FP64 point clouds keep the kernel of the current eps (8 n m bytes)
+ * for the length of the call, besides their scratch, where it takes at most `bytes`
+ * (default 4 GiB) and, above 64 MiB, at most half of the device's free memory;
+ * otherwise every pass evaluates its terms on the fly (about ten times slower, the
+ * same results to rounding).  Solves that run at the same time each keep their own.
+ * 0: never stored.  bytes < 0 changes nothing.  Returns the previous limit.
+ * Process-wide; read when a call plans its memory.
+ * FP64 grids keep 8 nin nout bytes per axis and direction (at most 72 MB each) as
+ * part of their scratch; this limit does not apply to them.
+ */
+long long uot_set_stored_kernel_limit(long long bytes);
+
+/*
  * uot_fail_captures(k) -- failure injection for tests, on the host: inside every
  * CUDA-graph capture of a solver the first k applications of the Gibbs operator
  * are recorded and the next one returns an error, so the capture fails part way

@@ -19,6 +19,9 @@ thread_local std::string g_last_error;
 std::atomic<long long> g_launches{0};
 Prof g_prof;
 
+static std::atomic<long long> g_stored_limit{4ll << 30};
+long long stored_kernel_limit() { return g_stored_limit.load(); }
+
 // Failure injection: applications left in this thread's capture (-1: not capturing).
 static std::atomic<int> g_capture_fault{-1};
 static thread_local int t_capture_left = -1;
@@ -219,6 +222,10 @@ uot_status uot_selftest_bounded_wait(double seconds, void* stream) {
 }
 
 uot_status uot_force_batch_warps(int warps) { return batch_force_warps(warps) == 0 ? UOT_OK : UOT_EINVAL; }
+
+long long uot_set_stored_kernel_limit(long long bytes) {
+  return bytes < 0 ? g_stored_limit.load() : g_stored_limit.exchange(bytes);
+}
 
 int uot_fail_captures(int applications) { return g_capture_fault.exchange(applications < 0 ? -1 : applications); }
 

@@ -715,9 +715,18 @@ class Scratch {
     if (extra_) cudaFreeAsync(extra_, s_);
   }
   // One more block that the caller can do without: NULL (and no error) when it
-  // does not fit the device's free memory.
+  // does not fit, or (above 64 MiB) would take more than half of what the device
+  // has free, so that the process's other users of the device keep room.
   void* try_extra(size_t bytes) {
     if (fixed_ || extra_) return nullptr;
+    size_t free_bytes = 0, total = 0;
+    if (bytes > ((size_t)64 << 20)) {
+      if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return nullptr;
+      }
+      if (bytes > free_bytes / 2) return nullptr;
+    }
     if (cudaMallocAsync(&extra_, bytes, s_) != cudaSuccess) {
       (void)cudaGetLastError();
       extra_ = nullptr;
@@ -805,6 +814,7 @@ struct Gibbs {
   // FP64 point clouds (k_points64.cu), and the eps their stored kernel is of
   Points64 p64 = {};
   double p64_eps = -1.0;
+  bool p64_on = false;          // p64_stored() when the scratch was planned
   void* Lscratch = nullptr;     // rows: shifted input line
   void* part = nullptr;         // FP32 point clouds: per-chunk partial sums
   float* zrow[2] = {nullptr, nullptr};  // FP32 point clouds: previous results per direction
@@ -845,7 +855,8 @@ struct Gibbs {
         sc.reserve<float>((size_t)g.n * g.d);
         sc.reserve<float>((size_t)g.m * g.d);
         sc.reserve<float>((size_t)mx);
-        if (p64_stored()) {
+        p64_on = p64_stored();
+        if (p64_on) {
           sc.reserve<double>((size_t)g.n);
           sc.reserve<double>((size_t)g.m);
           sc.reserve<double>((size_t)g.m);
@@ -877,11 +888,12 @@ struct Gibbs {
     return prec == UOT_F64 && host_setup && (speculate || pass_lines(dir, ax) * nbatch >= 8);
   }
   bool points64() const { return g.kind == UOT_GEOM_POINTS && prec == UOT_F64; }
-  // A solver's passes at one eps share a stored kernel of up to 4 GiB (23000 x
-  // 23000 points), where the device has that much free.
+  // A solver's passes at one eps share a stored kernel of up to
+  // uot_set_stored_kernel_limit bytes (4 GiB: 23000 x 23000 points), where the
+  // device has twice that free.
   bool p64_stored() const {
     return points64() && host_setup && speculate && nbatch == 1 &&
-           (size_t)g.n * points64_ld(g.m) * sizeof(double) <= ((size_t)4 << 30);
+           (long long)((size_t)g.n * points64_ld(g.m) * sizeof(double)) <= stored_kernel_limit();
   }
   bool points_fast() const {
     return g.kind == UOT_GEOM_POINTS && prec != UOT_F64 && g.d <= 3 && points_chunks_fit(g.n) &&
@@ -1037,7 +1049,7 @@ struct Gibbs {
           k_from_f64<float><<<nblocks((int64_t)g.m * g.d), kNT, 0, s>>>(p64.y, (int64_t)g.m * g.d, y32);
           p64.x32 = x32;
           p64.y32 = y32;
-          if (p64_stored()) {
+          if (p64_on) {
             p64.M = sc.take<double>((size_t)g.n);
             p64.beta = sc.take<double>((size_t)g.m);
             p64.w = sc.take<double>((size_t)g.m);

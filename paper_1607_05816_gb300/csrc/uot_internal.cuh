@@ -833,6 +833,7 @@ struct BatchArgs {
 // tuner is on (batch_pick_variant: synchronises `s`; a.next is left dirty).
 int batch_ctas_per_sm(int d, int variant, int nmax, int mmax);
 int batch_pick_variant(const BatchArgs& a, const int* h_order, cudaStream_t s);
+long long stored_kernel_limit();  // bytes (uot_set_stored_kernel_limit)
 // Failure injection on the host (uot_fail_captures): inside a graph capture, the
 // Gibbs-operator applications after the first few return an error.
 bool capture_fault();

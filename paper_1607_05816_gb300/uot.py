@@ -150,6 +150,7 @@ _SIGS = {
     "uot_force_batch_warps": (C.c_int, [C.c_int]),
     "uot_force_batch_cluster": (C.c_int, [C.c_int]),
     "uot_fail_captures": (C.c_int, [C.c_int]),
+    "uot_set_stored_kernel_limit": (C.c_longlong, [C.c_longlong]),
     "uot_selftest_bounded_wait": (C.c_int, [C.c_double, C.c_void_p]),
     "uot_probe_pipes": (C.c_int, [C.POINTER(C.c_double), C.c_void_p]),
     "uot_force_precise_passes": (C.c_int, [C.c_int]),
@@ -238,6 +239,12 @@ def force_batch_warps(warps: int):
 def force_batch_cluster(ctas: int):
     """CTAs per problem of solve_batch: 1, 2, 4 or 8, 0 = estimated from the batch."""
     _check(load().uot_force_batch_cluster(int(ctas)), "uot_force_batch_cluster")
+
+
+def set_stored_kernel_limit(nbytes: int) -> int:
+    """uot_set_stored_kernel_limit: device memory that an FP64 point-cloud solve may take
+    for its stored kernel (0: none); returns the previous limit."""
+    return int(load().uot_set_stored_kernel_limit(int(nbytes)))
 
 
 def fail_captures(applications: int) -> int:
