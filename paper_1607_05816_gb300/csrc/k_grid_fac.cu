@@ -47,7 +47,7 @@ __device__ __forceinline__ double wmax_d(double v) {
 __global__ void __launch_bounds__(256) fac64_build(const double* __restrict__ xo, int nout,
                                                    const double* __restrict__ yi, int nin, double inv_eps,
                                                    double* __restrict__ G, FacTile* __restrict__ tiles) {
-  __shared__ double s_lo[8], s_hi[8];
+  __shared__ double s_lo[8], s_hi[8], s_xl[kFacMaxSub], s_xh[kFacMaxSub];
   __shared__ FacTile s_t;
   const int tile = blockIdx.x, i0 = tile * kTile;
   const int tid = threadIdx.x;
@@ -62,35 +62,56 @@ __global__ void __launch_bounds__(256) fac64_build(const double* __restrict__ xo
     s_lo[tid >> 5] = lo;
     s_hi[tid >> 5] = hi;
   }
+  // the tile's outputs in 16 blocks of 4: least and largest coordinate
+  constexpr int kLeast = kTile / kFacMaxSub;
+  if (tid < kFacMaxSub) {
+    double xl = kInf, xh = -kInf;
+#pragma unroll
+    for (int u = 0; u < kLeast; ++u) {
+      const int i = i0 + tid * kLeast + u;
+      if (i < nout) {
+        xl = fmin(xl, xo[i]);
+        xh = fmax(xh, xo[i]);
+      }
+    }
+    s_xl[tid] = xl;
+    s_xh[tid] = xh;
+  }
   __syncthreads();
-  if (tid == 0) {
-    for (int w = 1; w < 8; ++w) {
+  // Lane p of the first warp tries block s of a cut into sub blocks, p = sub - 1 + s
+  // (31 of them; one thread trying all took 46 us at 64 outputs: an operator call on 64 x 64
+  // at eps 1e-4 0.42 ms, 0.33 here).
+  if (tid < 32) {
+    for (int w = 0; w < 8; ++w) {
       lo = fmin(lo, s_lo[w]);
       hi = fmax(hi, s_hi[w]);
     }
-    FacTile t;
-    t.sub = 0;
-    for (int sub = 1; sub <= kFacMaxSub && !t.sub; sub *= 2) {
-      bool ok = true;
-      for (int s = 0; s < sub; ++s) {
-        const int a = i0 + s * (kTile / sub), b = min(nout, a + kTile / sub);
-        double xl = kInf, xh = -kInf;
-        for (int i = a; i < b; ++i) {
-          xl = fmin(xl, xo[i]);
-          xh = fmax(xh, xo[i]);
-        }
-        const double c = (a < b) ? 0.5 * (xl + xh) : xo[i0];
-        const double d = (a < b) ? fmax(xh - c, c - xl) : 0.0;
-        const double D = fmax(fabs(c - lo), fabs(c - hi));
-        ok = ok && (d * d + 2.0 * d * D) * inv_eps <= kMaxReach;  // false for NaN as well
-        t.c[s] = c;
+    const int sub = 1 << (31 - __clz(tid + 1)), s = tid + 1 - sub, per = kFacMaxSub / sub;
+    bool ok = true;
+    double c = 0.0;
+    if (sub <= kFacMaxSub) {
+      double xl = kInf, xh = -kInf;
+      for (int u = 0; u < per; ++u) {
+        xl = fmin(xl, s_xl[s * per + u]);
+        xh = fmax(xh, s_xh[s * per + u]);
       }
-      if (ok) t.sub = sub;
+      const bool some = i0 + s * (kTile / sub) < nout;
+      c = some ? 0.5 * (xl + xh) : xo[i0];
+      const double d = some ? fmax(xh - c, c - xl) : 0.0;
+      const double D = fmax(fabs(c - lo), fabs(c - hi));
+      ok = (d * d + 2.0 * d * D) * inv_eps <= kMaxReach;  // false for NaN as well
     }
-    s_t = t;
-    if (blockIdx.y == 0) tiles[tile] = t;
+    const unsigned fits = __ballot_sync(0xffffffffu, ok);
+    int best = 0;  // the fewest blocks that all fit
+    for (int k = kFacMaxSub; k; k /= 2) {
+      const unsigned all = ((1u << k) - 1u) << (k - 1);
+      if ((fits & all) == all) best = k;
+    }
+    if (tid == 0) s_t.sub = best;
+    if (sub == best) s_t.c[s] = c;
   }
   __syncthreads();
+  if (blockIdx.y == 0 && tid == 0) tiles[tile] = s_t;
   if (s_t.sub == 0) return;
   const int o = tid & (kTile - 1), i = i0 + o;
   const int64_t ld = (int64_t)gridDim.x * kTile;
