@@ -18,7 +18,7 @@
 // 2-D, 50 iterations: 28.5 ms, the time of the 2048 x 2048 problem on half an
 // SM; clusters of 2: 20.9 ms, and 19.3 ms with the sweeps unrolled by 8 instead of
 // 2; clusters of 4: 21.3, of 8: 27.9); the cluster size comes from a
-// list-scheduling estimate of the batch (batch_cluster).
+// simulated schedule of the batch (batch_cluster).
 //
 // Per half-step the CTA stages the input side {t_j, y_j} in shared memory
 // (the only per-problem data kept there, so several CTAs share an SM) and
@@ -714,17 +714,79 @@ cudaError_t launch_cluster(const BatchArgs& a, int CL, cudaStream_t s) {
   return cudaLaunchKernelEx(&cfg, batch_solve<D, kClWarps, true>, a);
 }
 
-// Cycles of one half-step of a CTA that shares its SM with another one: a term
-// takes 2 d + 3 FMA-pipe lanes, a warp 4 (2 d + 3) pipe cycles per input for its
-// 128 outputs, and eight warps share a pipe; the constant stands for the latencies of the staging,
-// the merge and the epilogue (and of the cluster barrier).
-double half_cost(int d, int nout, int nin, int CL) {
-  const int loc = ((nout + kOB - 1) / kOB + CL - 1) / CL;
-  const int split = loc >= kClWarps ? 1 : kClWarps / loc;
-  const int rounds = (loc + kClWarps - 1) / kClWarps;
-  const double busy = (double)std::min(loc * split, kClWarps) / kClWarps;
-  const double sweep = rounds * std::ceil((double)nin / split) * 8.0 * 4.0 * (2 * d + 3) * busy;
-  return sweep + 600.0 * ((nin + 511) / 512) + 3000.0 + (CL > 1 ? 1500.0 : 0.0);
+// Cycles of the two half-steps of a problem on a cluster of CL CTAs: `pipe`, the sweeps, takes
+// `shared` times as long where a second CTA shares the SM, `wait` (staging, barriers, merge, epilogue)
+// does not.  From the time per half-step of equal 2-D problems, one and two CTAs per SM: 300
+// points 6.7 and 11.8 us on one CTA, 6.2 and 9.6 on two; 1000 points 37.1 and 70.5, 21.1 and
+// 38.5 (1.95 times the sweeps), eight 8.6 and 13.7 (1.75); 512 points 14.0 us, 16.1 in 3-D.
+struct BatchCost {
+  double pipe, wait, shared;
+};
+BatchCost problem_cost(int d, int n, int m, int CL) {
+  BatchCost c{0.0, 0.0, CL > 4 ? 1.75 : 1.95};
+  for (int h = 0; h < 2; ++h) {
+    const int nout = h ? m : n, nin = h ? n : m;
+    const int loc = ((nout + kOB - 1) / kOB + CL - 1) / CL;
+    const int split = loc >= kClWarps ? 1 : kClWarps / loc;
+    const int on_pipe = (loc * split + 3) / 4;  // sweeps on the fullest of the SM's four partitions
+    c.pipe += on_pipe * std::ceil((double)nin / split) * (18.5 + 8.25 * d) + 2000.0;
+    c.wait += 2500.0 + 3.0 * nin + (CL > 1 ? 2000.0 : 0.0);
+  }
+  return c;
+}
+
+// Time at which the last problem ends: queue order, `groups` sets of SMs that hold up to
+// `slots` (1 or 2) problems each, the next problem into the slot that becomes free; two problems
+// of a group take turns on its pipes.  Where the first problems fill more than a slot per
+// group, neighbours in the queue share one (300 clouds of 64 to 2048 points last as long as the
+// largest two together).
+double batch_end(const std::vector<BatchCost>& jobs, int groups, int slots) {
+  struct Group {
+    int job[2] = {-1, -1};
+    double left[2] = {0.0, 0.0};  // fraction of the job
+    double at = 0.0, next = 0.0;
+  };
+  std::vector<Group> g(groups);
+  typedef std::pair<double, int> Event;
+  std::priority_queue<Event, std::vector<Event>, std::greater<Event>> events;
+  const int njobs = (int)jobs.size();
+  int queued = 0;
+  double end = 0.0;
+  auto duration = [&](const Group& q, int u) {
+    const BatchCost& c = jobs[q.job[u]];
+    return (q.job[0] >= 0 && q.job[1] >= 0 ? c.shared : 1.0) * c.pipe + c.wait;
+  };
+  auto plan = [&](int i) {
+    Group& q = g[i];
+    q.next = kInf;
+    for (int u = 0; u < 2; ++u)
+      if (q.job[u] >= 0) q.next = std::min(q.next, q.at + q.left[u] * duration(q, u));
+    if (q.next < kInf) events.push(Event(q.next, i));
+  };
+  const int pairs = std::max(0, std::min(njobs, groups * slots) - groups);
+  for (int i = 0; i < groups; ++i)
+    for (int u = 0; u < (i < pairs ? 2 : 1) && queued < njobs; ++u) {
+      g[i].job[u] = queued++;
+      g[i].left[u] = 1.0;
+    }
+  for (int i = 0; i < groups; ++i) plan(i);
+  while (!events.empty()) {
+    const Event e = events.top();
+    events.pop();
+    Group& q = g[e.second];
+    double took[2];
+    for (int u = 0; u < 2; ++u) took[u] = q.job[u] >= 0 ? (e.first - q.at) / duration(q, u) : 0.0;
+    q.at = end = e.first;
+    for (int u = 0; u < 2; ++u) {
+      if (q.job[u] < 0) continue;
+      q.left[u] -= took[u];
+      if (q.left[u] > 1e-9) continue;
+      q.job[u] = queued < njobs ? queued++ : -1;
+      q.left[u] = 1.0;
+    }
+    plan(e.second);
+  }
+  return end;
 }
 
 // Times both CTA sizes on a sample of the batch: every (nprob/S)-th problem
@@ -849,44 +911,36 @@ std::string batch_tune_table() {
   return s;
 }
 
-// CTAs per problem: the cluster size whose list schedule (problems in queue
-// order, each to the unit that is free first) ends earliest by half_cost, the
-// smaller one within 3%, and none of more CTAs than the largest side has output
-// blocks.  One CTA where no problem is larger than an eighth of a
-// unit's average load: clusters could shorten such a batch by little.
+// CTAs per problem: the cluster size whose schedule ends earliest (batch_end), the smaller one
+// within 3%, and none of more CTAs than the largest side has output blocks.  One CTA where no
+// problem is larger than a fourth of an SM's average load: clusters could shorten such a batch
+// by little.  A first form of the estimate counted every CTA as sharing its SM and took two CTAs
+// for 152 problems of 300 points, 1.60 ms where one CTA takes 1.31.
 int batch_cluster(int d, int nmax, int mmax, const int* n, const int* m, const int* order, int nprob) {
   {
     std::lock_guard<std::mutex> lk(g_bmu);
     if (g_cforced > 0) return g_cforced;
     if (g_bforced >= 0) return 1;
   }
-  const int per = ctas_any(d, 1, nmax, mmax) * sm_count();
-  if (per < 1) return 1;
+  const int sms = sm_count(), slots = std::min(2, ctas_any(d, 1, nmax, mmax));
+  if (slots < 1 || sms < 1) return 1;
+  std::vector<BatchCost> jobs(nprob);
   int best = 1;
   double best_t = 0.0;
   for (int CL : {1, 2, 4, 8}) {
     if (CL > (std::max(nmax, mmax) + kOB - 1) / kOB) break;
-    const int units = CL == 1 ? per : cluster_count(d, CL, std::max(nmax, mmax));
-    if (units < 1) continue;
-    double sum = 0.0, most = 0.0, end = 0.0;
-    std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+    const int groups = CL == 1 ? sms : cluster_count(d, CL, std::max(nmax, mmax)) / slots;
+    if (groups < 1) continue;
+    double sum = 0.0, most = 0.0;
     for (int t = 0; t < nprob; ++t) {
       const int k = order[t];
-      const double c = half_cost(d, n[k], m[k], CL) + half_cost(d, m[k], n[k], CL);
-      sum += c;
-      most = std::max(most, c);
-      double at = c;
-      if ((int)free_at.size() == units) {
-        at += free_at.top();
-        free_at.pop();
-      }
-      free_at.push(at);
-      end = std::max(end, at);
+      jobs[t] = problem_cost(d, n[k], m[k], CL);
+      sum += jobs[t].pipe;
+      most = std::max(most, jobs[t].pipe);
     }
-    if (CL == 1) {
-      if (most <= sum / units / 8.0) return 1;
-      best_t = end;
-    } else if (end < 0.97 * best_t) {
+    if (CL == 1 && most <= sum / sms / 4.0) return 1;
+    const double end = batch_end(jobs, groups, slots);
+    if (CL == 1 || end < 0.97 * best_t) {
       best_t = end;
       best = CL;
     }
