@@ -160,6 +160,24 @@ __device__ __forceinline__ void term_exponents(const float4* st0, const typename
   EB = fma2(nk2, QB, sub2(T, MB));
 }
 
+// body(j) for j0 <= j < j1, eight at a time and the rest in pairs: problems of 64 points leave a
+// warp four inputs, which a loop unrolled by eight alone takes one by one.
+template <typename F>
+__device__ __forceinline__ void for_inputs(int j0, int j1, F&& body) {
+  int j = j0;
+#pragma unroll 1
+  for (; j + 8 <= j1; j += 8) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) body(j + u);
+  }
+#pragma unroll 1
+  for (; j + 2 <= j1; j += 2) {
+    body(j);
+    body(j + 1);
+  }
+  if (j < j1) body(j);
+}
+
 // Log2-sum-exp of a lane's 4 outputs over staged inputs [j0, j1): with
 // `exact` the per-output maxima are computed first (returned in mq), else
 // the shifts in mq are used.  Returns the shifted sums in sq.
@@ -169,8 +187,7 @@ __device__ __forceinline__ void sweep(const float4* st0, const typename Stage1<D
   const f2p zero2 = pk(0.0f, 0.0f);
   if (exact) {
     float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll 8
-    for (int j = j0; j < j1; ++j) {
+    for_inputs(j0, j1, [&](int j) {
       f2p EA, EB;
       term_exponents<D>(st0, st1, j, X, nk2, zero2, zero2, EA, EB);
       const float2 A = upk(EA), B = upk(EB);
@@ -178,21 +195,20 @@ __device__ __forceinline__ void sweep(const float4* st0, const typename Stage1<D
       m4[1] = fmaxf(m4[1], A.y);
       m4[2] = fmaxf(m4[2], B.x);
       m4[3] = fmaxf(m4[3], B.y);
-    }
+    });
 #pragma unroll
     for (int q = 0; q < 4; ++q) mq[q] = m4[q];
   }
   const f2p MA = pk(mq[0] == -INFINITY ? 0.0f : mq[0], mq[1] == -INFINITY ? 0.0f : mq[1]);
   const f2p MB = pk(mq[2] == -INFINITY ? 0.0f : mq[2], mq[3] == -INFINITY ? 0.0f : mq[3]);
   f2p SA = zero2, SB = zero2;
-#pragma unroll 8
-  for (int j = j0; j < j1; ++j) {
+  for_inputs(j0, j1, [&](int j) {
     f2p EA, EB;
     term_exponents<D>(st0, st1, j, X, nk2, MA, MB, EA, EB);
     const float2 A = upk(EA), B = upk(EB);
     SA = add2(SA, pk(ex2_approx(A.x), ex2_approx(A.y)));
     SB = add2(SB, pk(ex2_approx(B.x), ex2_approx(B.y)));
-  }
+  });
   const float2 a = upk(SA), b = upk(SB);
   sq[0] = a.x;
   sq[1] = a.y;
