@@ -1477,10 +1477,17 @@ TuneEntry tune_tiles(const PassArgs& base, int nbatch, cudaStream_t s) {
     for (int t = 0; t < kNumTiles; ++t) {
       if (!okt[t]) continue;
       ent.us[t] = tmin[t];
-      if (!is_blk(t) && tmin[t] < best) {
+      if (!is_blk(t) && t != kShortTile && tmin[t] < best) {
         best = tmin[t];
         ent.tile = t;
       }
+    }
+    // The warp-per-line kernel has to win by 5% too: between passes of other tiles it can
+    // take longer than in this chain of its own launches (20 batches of 93 x 57, 60 iterations:
+    // 5.87 us here against 6.03 for the next best tile, but 2.24 against 1.94 ms in the solve).
+    if (okt[kShortTile] && 1.05f * tmin[kShortTile] < best) {
+      best = tmin[kShortTile];
+      ent.tile = kShortTile;
     }
     // The chain above differs from a solve's (no prox epilogue, no potential
     // inputs), and tiles within a few percent of each other here can rank
