@@ -103,6 +103,18 @@ def mass_div(uot_or_oracle, name):
     return {"eq": m.EQ(), "kl": m.KL(LAM), "tv": m.TV(LAM), "rg": m.RG(0.8, 1.2)}[name]
 
 
+def json_line(line):
+    """One line of JSON; numbers that JSON has no word for (a violation that a workload does not
+    measure) become null."""
+    def clean(v):
+        if isinstance(v, dict):
+            return {k: clean(x) for k, x in v.items()}
+        if isinstance(v, (list, tuple)):
+            return [clean(x) for x in v]
+        return None if isinstance(v, float) and not math.isfinite(v) else v
+    return json.dumps(clean(line), allow_nan=False)
+
+
 def config_dict(extra=None, mass=None):
     c = {"workload": WORKLOAD + (f"-mass-{MASS_DIVS[mass]}-m0{MASS_M0}" if mass else ""), "grid": [H, W], "lambda": LAM, "eps": EPS, "eps_start": EPS_START,
          "eps_stages": STAGES, "iters_per_stage": IPS, "tol": TOL, "check_every": CHECK_EVERY,
@@ -890,7 +902,7 @@ def run_reference(args, rank, world):
                          "sample": f"{per_step} iterations per step at eps=1e-3"},
         "e2e": {"value": value, "unit": "iters/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0},
     }
-    print(json.dumps(line), flush=True)
+    print(json_line(line), flush=True)
 
 
 # ----------------------------------------------------------------------------
@@ -1263,7 +1275,7 @@ def main():
                     line["cpu_baseline_all_cores"] = oracle_baselines("grid2d", host_cores(),
                                                                       one_core=False)["all_cores"]
         if line is not None:
-            print(json.dumps(line), flush=True)
+            print(json_line(line), flush=True)
     finally:
         if world > 1:
             import torch.distributed as dist
