@@ -335,17 +335,14 @@ __global__ void __launch_bounds__(128) grid_pass_f64_few(Fac64Args a, Epilogue e
       return v - d * d * a.inv_eps;
     };
     double m = -kInf, s = 0.0;
-    bool nan = false;
-    for (int j = lane; j < a.nin; j += 32) {
-      const double e = expo(j);
-      nan = nan || e != e;
-      m = fmax(m, e);
-    }
+    for (int j = lane; j < a.nin; j += 32) m = fmax(m, expo(j));
     m = wmax_d(m);
     double z = -kInf;
-    if (__any_sync(0xffffffffu, nan)) {
-      z = NAN;
-    } else if (m != -kInf) {
+    if (m == -kInf) {  // every input is empty, or NaN, which has no maximum
+      bool nan = false;
+      for (int j = lane; j < a.nin; j += 32) nan = nan || expo(j) != expo(j);
+      if (__any_sync(0xffffffffu, nan)) z = NAN;
+    } else {
       for (int j = lane; j < a.nin; j += 32) s += exp(expo(j) - m);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);

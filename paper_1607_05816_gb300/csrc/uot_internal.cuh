@@ -11,6 +11,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 
 #include "../../include/uot.h"
@@ -506,14 +507,20 @@ cudaError_t smem_at_least(K* kernel, size_t bytes) {
   return smem_limit_at_least(reinterpret_cast<const void*>(kernel), bytes);
 }
 
-// SMs of the current device (0 if it cannot be asked).
+// SMs of the current device (0 if it cannot be asked), asked once per device: launch rules
+// read it for every pass.
 inline int sm_count() {
+  static std::atomic<int> known[64];
   int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return 0;
+  if (cudaGetDevice(&dev) == cudaSuccess) {
+    if (dev < 64 && (sms = known[dev].load(std::memory_order_relaxed)) > 0) return sms;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) {
+      if (dev < 64) known[dev].store(sms, std::memory_order_relaxed);
+      return sms;
+    }
   }
-  return sms;
+  (void)cudaGetLastError();
+  return 0;
 }
 
 // Launch with programmatic dependent launch: the kernel may start while its
