@@ -790,13 +790,19 @@ double batch_end(const std::vector<BatchCost>& jobs, int groups, int slots) {
     const Event e = events.top();
     events.pop();
     Group& q = g[e.second];
-    double took[2];
-    for (int u = 0; u < 2; ++u) took[u] = q.job[u] >= 0 ? (e.first - q.at) / duration(q, u) : 0.0;
+    double todo[2], time[2];
+    for (int u = 0; u < 2; ++u) {
+      time[u] = q.job[u] >= 0 ? duration(q, u) : 0.0;
+      todo[u] = q.job[u] >= 0 ? q.left[u] * time[u] : kInf;
+    }
+    const double step = std::min(todo[0], todo[1]);  // (not from the clock: its rounding could end no job)
     q.at = end = e.first;
     for (int u = 0; u < 2; ++u) {
       if (q.job[u] < 0) continue;
-      q.left[u] -= took[u];
-      if (q.left[u] > 1e-9) continue;
+      if (todo[u] > step * (1.0 + 1e-9)) {
+        q.left[u] -= step / time[u];
+        continue;
+      }
       q.job[u] = queued < njobs ? queued++ : -1;
       q.left[u] = 1.0;
     }
