@@ -275,7 +275,7 @@ int uot_autotune_table(char* buf, int len);
  * when a size is forced.  8 or 16 warps per CTA are compiled; with the tuner on,
  * the first call for a batch shape (d, largest n, largest m) times both on a
  * sample of the batch (every (nprob/S)-th problem of the size-ordered queue,
- * S = 2 x SM count, six iterations) and keeps the 8-warp CTA unless the other
+ * S = 8 x SM count, six iterations) and keeps the 8-warp CTA unless the other
  * is more than 3% faster; uot_autotune_table lists the choice.
  * uot_force_batch_warps(w): w = 8 or 16 forces that size, 0 returns to the
  * tuned one; UOT_EINVAL otherwise.
