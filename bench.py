@@ -51,10 +51,6 @@ MUFU_PEAK_GEXP = SM_COUNT * MUFU_PER_CLK * SM_MAX_MHZ * 1e6 / 1e9
 # FP64 pipe (Algorithm 1 matvec): GB300 runs FP64 at 1.25 TFLOP/s nominal,
 # i.e. 2 DFMA per clock per SM.
 FP64_PEAK_GFLOPS = 1250.0
-# HBM copy bandwidth measured on this GPU type (MEASURED_PEAKS.json hbm_gbs)
-HBM_PEAK_GBS = 6760.6
-# dram bytes of one rows_lse_f64_chunks<24> launch of the wf workload; None: not captured
-WF_ROWS_TRAFFIC_BYTES = None
 # dram bytes of one alg1_cluster launch (2000 iterations of the dense 256 x 256
 # problem; profiles/alg1_cluster_dense256.md); None once the kernel changes
 ALG1_CLUSTER_TRAFFIC_BYTES = 1185792
@@ -418,14 +414,13 @@ def run_ours(args, rank, world, local_rank):
         probe["mufu_ex2_per_clk_per_sm"], probe["ffma_per_clk_per_sm"] / FP32_OPS_PER_TERM["grid"])
         * SM_COUNT * SM_MAX_MHZ * 1e6 / 1e9)
     if prec == uot.F64:
-        # the FP64 pass evaluates one FP64 exp() per term: its ceiling is the
-        # measured FP64 exponential rate, not the MUFU (kept as context)
+        # the FP64 pass multiplies with a stored kernel, one FP64 multiply-add per term
         r = line["roofline"]
-        peak64 = probe["dexp_per_clk_per_sm"] * SM_COUNT * SM_MAX_MHZ * 1e6 / 1e9
-        r.update({"binding_pipe": "fp64 (exp)", "peak": peak64, "frac": r["achieved"] / peak64,
-                  "peak_source": "measured: the library's FP64 exp() throughput probe (64 warps per SM, "
+        peak64 = probe["dfma_per_clk_per_sm"] * SM_COUNT * SM_MAX_MHZ * 1e6 / 1e9
+        r.update({"binding_pipe": "fp64 (fma)", "peak": peak64, "frac": r["achieved"] / peak64, "unit": "Gterm/s",
+                  "peak_source": "measured: the library's FP64 FMA throughput probe (64 warps per SM, "
                                  "dependent chains), x 152 SMs x 2070 MHz"})
-        r["pipes"]["fp64_exp"] = {"peak_gexp": peak64, "frac": r["achieved"] / peak64}
+        r["pipes"]["fp64_fma"] = {"peak_gterm": peak64, "frac": r["achieved"] / peak64}
     if world == 1 and not args.no_cpu_baseline:
         line["cpu_baseline"] = cpu_baseline(args.cpu_iters, args.mass_div)
     return line
@@ -504,7 +499,7 @@ def run_single(args, rank, world, local_rank):
                                            iters=500, launch_mode=args.launch_mode)
             info["marg_err"] = float("nan")
             return U_, V_, info
-        work_per_iter, unit_work, kernel = 2.0 * S * n * n, "Gterm/s", "rows_lse_f64_chunks<24>"
+        work_per_iter, unit_work, kernel = 2.0 * S * n * n, "Gterm/s", "rows_lse_f64_chunks<8, 1>"
         cfg = {"workload": f"wf-flow-{S}species-3000-eps{eps:g}-tau{tau:g}-alpha1-500it-x4steps",
                "n": n, "species": S, "eps": eps, "tau": tau, "alpha": 1.0, "lambda": 1.0,
                "iters_per_flow_step": 500, "flow_steps_per_bench_step": nflow,
@@ -603,20 +598,10 @@ def run_single(args, rank, world, local_rank):
         if wl in ("bary", "color"):
             line["grid_tiles"] = uot.autotune_table().strip().splitlines()
     elif unit_work == "Gterm/s":
-        # rows_lse_f64_chunks reads the least cost of every chunk of 32 columns (4 B per
-        # 32 terms) and the chunks that can matter; at this eps it is a chain of
-        # latencies, far from any memory rate.
-        gbs = achieved * 4.0 / 32
-        line["roofline"] = {"bound": "hbm", "kernel": kernel, "achieved": gbs, "peak": HBM_PEAK_GBS,
-                            "unit": "GB/s", "frac": gbs / HBM_PEAK_GBS,
-                            "traffic": WF_ROWS_TRAFFIC_BYTES,
-                            "traffic_source": ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch "
-                                               "(cold cache)")
-                            if WF_ROWS_TRAFFIC_BYTES is not None else None,
-                            "algorithmic_bytes_per_launch": 4.0 * n * ((n + 31) // 32),
-                            "terms_per_s": achieved * 1e9,
-                            "peak_source": "MEASURED_PEAKS.json hbm_gbs (burst copy), of measured",
-                            "timing": timing}
+        # rows_lse_f64_chunks looks at every term's chunk and evaluates the few that count: a
+        # chain of latencies, which no pipe's or memory's rate describes
+        line["roofline"] = {"bound": "latency", "kernel": kernel, "achieved": achieved, "peak": None, "unit": unit_work,
+                            "frac": None, "traffic": None, "timing": timing}
     else:
         tr = ALG1_CLUSTER_TRAFFIC_BYTES if kernel == "alg1_cluster" else None
         line["roofline"] = {"bound": "alu", "kernel": kernel, "achieved": achieved, "peak": FP64_PEAK_GFLOPS,

@@ -317,8 +317,9 @@ int uot_fail_captures(int applications);
  * clock per SM measured with in-kernel clock64() over dependent-chain loops
  * with 64 resident warps per SM:
  *   out[0]: FP32 FMA lane operations, out[1]: MUFU ex2.approx.f32, out[2]: FP64
- *   FMA lane operations, out[3]: FP64 exponentials exp() (the function the FP64
- *   Gibbs passes evaluate per kernel term).  out holds 4 doubles.
+ *   FMA lane operations (what the FP64 passes over a stored kernel run per term),
+ *   out[3]: FP64 exponentials exp() (per term of the FP64 grid passes without one).
+ *   out holds 4 doubles.
  * A few milliseconds of work; synchronises `stream`.
  */
 uot_status uot_probe_pipes(double* out, void* stream);
@@ -751,6 +752,8 @@ uot_status uot_warmstart_features(const float* p, const float* q, const float* l
  *   straight from g [P][ldg] and x [P][ldx] (NHWC, ldg and ldx multiples of 8,
  *   Cout <= min(ldg, 128), Cin <= min(ldx, 128), W = 64); 1 <= splits <= N H
  *   row ranges of partial sums, part is FP32 scratch of splits x (9 Cin + 1) x 128.
+ *   The warm-start network trains with this one; uot_conv_tc_wgrad, the two
+ *   transposes and uot_bias_grad_bf16 stay for callers that hold K-major copies.
  * uot_nhwc_shift_transpose: xT[d][c][n][y][x] = x[n][y][x + (d-1) dil][c] (0 off the
  *   image), d = 0, 1, 2; x [N][H][W][C], W <= 64.
  * uot_nhwc_transpose: yT[c][p] = y[p][c], y [P][C].

@@ -1,6 +1,6 @@
 // Table-driven FP64 exponential (the method of P. T. P. Tang, ACM TOMS 15, 1989):
-// about 9 FP64 instructions against about 25 of exp(), on a pipe of 2 lanes per
-// clock and SM.  The table of 2^(k/256) is 2 KB of shared memory.
+// about 9 FP64 instructions against about 15 of exp() (by their rates: 0.15 exp() and 2.2
+// multiply-adds per clock and SM).  The table of 2^(k/256) is 2 KB of shared memory.
 #pragma once
 
 namespace uot {

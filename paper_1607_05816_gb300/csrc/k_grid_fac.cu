@@ -8,7 +8,7 @@
 //
 // for a block of outputs with centre c.  G does not depend on the line, so it
 // is stored once per eps and axis, and a term costs one FP64 multiply-add
-// where the log-sum-exp pays an FP64 exponential (about 14 FP64 instructions
+// where the log-sum-exp pays an FP64 exponential (about 15 FP64 instructions
 // on a pipe that issues 2 lanes per clock and SM); A costs one exponential per
 // input and block of 64 outputs.  Centring keeps both factors inside the FP64
 // range: with reach = (d^2 + 2 d D) / eps (d the block's half width, D the
@@ -353,26 +353,11 @@ __global__ void __launch_bounds__(128) grid_pass_f64_few(Fac64Args a, Epilogue e
   if (epi.err) block_add2<128>(num, den, epi.err + 2 * bz);
 }
 
-template <typename K>
-cudaError_t launch_pdl(K kern, dim3 grid, int threads, const Fac64Args& a, const Epilogue& epi, cudaStream_t s) {
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(threads);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, a, epi);
-}
-
 template <int TL, int KS>
 cudaError_t launch_pass(const Fac64Args& a, const Epilogue& epi, int nbatch, cudaStream_t s) {
   const dim3 grid((a.nout + kTile - 1) / kTile, (a.nlines + TL - 1) / TL, nbatch);
   if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidConfiguration;
-  return launch_pdl(grid_pass_f64<TL, KS>, grid, kTile * TL * KS, a, epi, s);
+  return launch_pdl(grid_pass_f64<TL, KS>, grid, dim3(kTile * TL * KS), 0, s, a, epi);
 }
 
 }  // namespace
@@ -405,7 +390,7 @@ cudaError_t launch_grid_pass_f64(const double* in, const double* logw, int in_is
   a.use_prev = use_prev;
   const int64_t outs = (int64_t)nlines * nout;
   if (!G && outs * nbatch <= 64 * sm_count() && nbatch <= 65535)
-    return launch_pdl(grid_pass_f64_few, dim3((unsigned)((outs + 3) / 4), nbatch), 128, a, epi, s);
+    return launch_pdl(grid_pass_f64_few, dim3((unsigned)((outs + 3) / 4), nbatch), dim3(128), 0, s, a, epi);
   // Four slices of the inputs per output: 256 x 256, 51 us a pass (one slice 49,
   // eight 66); 300 x 300, 88 (one slice 128: the short last chunk's exponentials
   // are not hidden); 64 x 64, 7.6 (9.1).

@@ -21,7 +21,7 @@
 // (programmatic dependent launch).
 // Work: n m terms per call, in three dimensions 9 FP32-pipe operations and one
 // exponential each, bound by the FP32 pipe.  20000 x 20000 points in 3-D: 118 us a
-// sweep (96 us at the pipe's rate), 127 us a pass; a solve of 40 iterations over 11
+// sweep (90 us at the pipe's nominal rate), 127 us a pass; a solve of 40 iterations over 11
 // eps 13.4 -> 10.6 ms with the shifts carried from eps to eps, one thread per
 // output in the merge and the overlapped launches.
 #include <string.h>

@@ -360,21 +360,6 @@ __global__ void __launch_bounds__(256) points64_cols_end(Rows64 a, const double*
   if (epi.err) block_add2<256>(num, den, epi.err);
 }
 
-template <typename Kern, typename... Args>
-cudaError_t launch_pdl(Kern kern, dim3 grid, dim3 block, cudaStream_t s, Args... args) {
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
 }  // namespace
 
 int64_t points64_ld(int m) { return ((int64_t)m + 1) & ~(int64_t)1; }
@@ -401,7 +386,7 @@ cudaError_t launch_points64(const Points64& p, int dir, const double* W, const d
   const dim3 line_grid((a.nin + 127) / 128);
   const bool have = rows && !first;
   count_launches(1);
-  cudaError_t e = launch_pdl(points64_line, line_grid, dim3(128), s, W, logw, a.nin, a.inv_eps, p.Ls, p.L32,
+  cudaError_t e = launch_pdl(points64_line, line_grid, dim3(128), 0, s, W, logw, a.nin, a.inv_eps, p.Ls, p.L32,
                              (const double*)p.beta, have ? p.w : (double*)nullptr, p.drift);
   if (e != cudaSuccess) return e;
   prof_mark_begin(PROF_ROWS, s);
@@ -412,11 +397,11 @@ cudaError_t launch_points64(const Points64& p, int dir, const double* W, const d
     a.ld = ld;
     count_launches(2);
     // (a stored kernel has at most 2^29 entries: the product fits)
-    e = launch_pdl(points64_cols, dim3((p.m + kColTile - 1) / kColTile * nchunks), dim3(kColTile / 2), s,
+    e = launch_pdl(points64_cols, dim3((p.m + kColTile - 1) / kColTile * nchunks), dim3(kColTile / 2), 0, s,
                    (const double*)p.K, ld, p.n, p.m, W, logw, a.inv_eps, (const double*)p.M, p.part, shift);
     if (e != cudaSuccess) return e;
     auto end = [&](auto kern) {
-      return launch_pdl(kern, dim3((p.m + 31) / 32), dim3(256), s, a, (const double*)p.part, (const double*)shift,
+      return launch_pdl(kern, dim3((p.m + 31) / 32), dim3(256), 0, s, a, (const double*)p.part, (const double*)shift,
                         nchunks, (const double*)p.beta, p.drift, epi);
     };
     e = p.d == 1 ? end(points64_cols_end<1>) : p.d == 2 ? end(points64_cols_end<2>)
@@ -433,10 +418,10 @@ cudaError_t launch_points64(const Points64& p, int dir, const double* W, const d
     }
     count_launches(1);
     const dim3 grid((a.nrows + kRowWarps - 1) / kRowWarps), block(kRowWarps * 32);
-    e = p.d == 1 ? launch_pdl(points64_rows<1>, grid, block, s, a, epi)
-        : p.d == 2 ? launch_pdl(points64_rows<2>, grid, block, s, a, epi)
-        : p.d == 3 ? launch_pdl(points64_rows<3>, grid, block, s, a, epi)
-                   : launch_pdl(points64_rows<0>, grid, block, s, a, epi);
+    e = p.d == 1 ? launch_pdl(points64_rows<1>, grid, block, 0, s, a, epi)
+        : p.d == 2 ? launch_pdl(points64_rows<2>, grid, block, 0, s, a, epi)
+        : p.d == 3 ? launch_pdl(points64_rows<3>, grid, block, 0, s, a, epi)
+                   : launch_pdl(points64_rows<0>, grid, block, 0, s, a, epi);
   }
   if (e != cudaSuccess) return e;
   prof_mark_end(PROF_ROWS, s);

@@ -1,6 +1,6 @@
 // Throughput probes of the pipes the scaling kernels are bound by (FP32 FMA,
-// MUFU ex2, FP64 FMA, and the FP64 exponential exp() of the FP64 Gibbs passes
-// as the library compiles it), reported in operations per clock per SM so that the
+// MUFU ex2, FP64 FMA, and the FP64 exponential exp() as the library compiles it,
+// which the FP64 passes evaluate where no stored kernel serves them), reported in operations per clock per SM so that the
 // result does not depend on the clock the GPU runs at.  Each thread runs
 // kChains independent dependency chains (enough to cover the pipe latency);
 // every block records its elapsed SM cycles with clock64(), and the host

@@ -848,14 +848,22 @@ def conv_tc_wgrad(dyT, xT, cin_pad, N, H, W, dil, Cout, Cin, *, splits=64, part=
     return dw
 
 
-def conv_tc_wgrad_nhwc(g, x, N, H, W, dil, Cout, Cin, *, splits=50, part=None, dw=None, db=None, err=None):
-    """uot_conv_tc_wgrad_nhwc; g [P, ldg], x [P, ldx] BF16 -> (dw [Cout, Cin, 3, 3], db [Cout]) FP32.  Three
-    CTAs per split: 50 splits fill 150 of the 152 SMs with one CTA each."""
+# Three CTAs per split: 50 splits fill 150 of the 152 SMs with one CTA each.
+WGRAD_SPLITS = 50
+
+
+def wgrad_part_floats(Cin, splits=WGRAD_SPLITS):
+    """Floats of conv_tc_wgrad_nhwc's `part`."""
+    return splits * (9 * Cin + 1) * 128
+
+
+def conv_tc_wgrad_nhwc(g, x, N, H, W, dil, Cout, Cin, *, splits=WGRAD_SPLITS, part=None, dw=None, db=None, err=None):
+    """uot_conv_tc_wgrad_nhwc; g [P, ldg], x [P, ldx] BF16 -> (dw [Cout, Cin, 3, 3], db [Cout]) FP32."""
     f, dev = torch.float32, g.device
     splits = max(1, min(splits, N * H))
     dw = torch.empty(Cout, Cin, 3, 3, dtype=f, device=dev) if dw is None else dw
     db = torch.empty(Cout, dtype=f, device=dev) if db is None else db
-    need = splits * (9 * Cin + 1) * 128
+    need = wgrad_part_floats(Cin, splits)
     part = torch.empty(need, dtype=f, device=dev) if part is None else part
     if part.numel() < need:
         raise ValueError(f"part must hold {need} floats")

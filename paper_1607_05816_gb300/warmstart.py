@@ -259,7 +259,7 @@ class WarmStartNetTC:
             cin_pad, bn, cout_kpad = self._pads(li)
             x = acts[li]
             dw, db = uot.conv_tc_wgrad_nhwc(g, x, N, H, W, dil, cout, cin,
-                                            part=self._buf(("part", cin), (50 * (9 * cin + 1) * 128,), torch.float32),
+                                            part=self._buf(("part", cin), (uot.wgrad_part_floats(cin),), torch.float32),
                                             dw=self._buf(("dw", li), (cout, cin, 3, 3), torch.float32),
                                             db=self._buf(("db", li), (cout,), torch.float32), err=self.err)
             grads[li] = (dw, db)
