@@ -161,9 +161,9 @@ __global__ void __launch_bounds__(WARPS * 32)
 // matter, where the kernel before it read the whole FP32 cost (36 MB at
 // 3000 x 3000) into shared memory and kept every term above e^-746.  WF flow of
 // 3000 samples, eps = 1e-8: 28 -> 16 us a half-step (two kernels and the growth
-// step's share).  20 iterations, 3000 random points in 2-D: eps = 1e-1 16.4 -> 13.3
-// ms (FP64 terms: all of them count), 1e-2 16.4 -> 12.2, 1e-3 16.3 -> 4.4, 1e-4
-// 5.5 -> 2.4.
+// step's share).  20 iterations, 3000 random points in 2-D: eps = 1e-1 16.5 -> 13.2
+// ms (FP64 terms: all of them count), 1e-2 16.4 -> 12.0, 1e-3 16.2 -> 4.3, 1e-4
+// 5.5 -> 2.3.
 // ---------------------------------------------------------------------------
 
 // L_j = W_j/eps + log w_j in FP64 (L64) and as a float-float pair (Lff); the

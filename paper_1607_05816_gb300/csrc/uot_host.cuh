@@ -667,7 +667,7 @@ uot_status check_geom(const uot_geom* g) {
       for (int k = 0; k < g->ndim; ++k) {
         if (g->shape_x[k] < 1 || g->shape_y[k] < 1) return UOT_EINVAL;
         if (!g->axes_x[k] || !g->axes_y[k]) return UOT_EINVAL;
-        // a staged line must fit in shared memory (4 warps x nin x 16 bytes)
+        // a staged line of the FP32 passes must fit in shared memory
         if (g->shape_x[k] > 3000 || g->shape_y[k] > 3000) {
           g_last_error = "grid axis longer than 3000 points";
           return UOT_EUNSUPPORTED;
