@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(256) chunkmin32(const double* __restrict__ C, 
 // whole CTA, so a row with hundreds of terms among rows of five (the edge of a
 // density at small eps) does not wait for one warp's loads, and every sum is taken
 // in a fixed order.
-// Rows of at most kShortChunks chunks a warp (kShort) need no bounds: all their
+// Rows of at most kShort (8 or 10) chunks a warp need no bounds: all their
 // exponents fit in registers, with the costs loaded before the preceding kernel has
 // ended (WF flow of 400 samples, two species, eps = 1e-8: 4.0 -> 3.5 ms).
 //
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(256) chunkmin32(const double* __restrict__ C, 
 // warp, the CTA's epilogue (some 150 of 16 clocks each), so many rows share a CTA
 // where there are many.
 constexpr int kRowList = 352;
-constexpr int kShortChunks = 8;  // kShort: chunks per warp, their exponents in registers
+constexpr int kShortChunks = 8, kShortWide = 10;  // kShort: chunks per warp in registers (0: by bounds)
 constexpr float kRowFarTol = 200.0f;  // an error that keeps every term between e^-200 and e^430
 constexpr unsigned kRowLeastHi = 123u << 20, kRowMostHi = 0x7ff00000u;  // high words of 2^-900 and infinity
 
@@ -246,7 +246,7 @@ size_t rows_chunks_smem(int nw, int nchunk) {
          (size_t)std::min(nchunk, kStagedChunks) * sizeof(float);
 }
 
-template <int NW, int WPR, bool kShort>
+template <int NW, int WPR, int kShort>
 __global__ void __launch_bounds__(NW * 32)
     rows_lse_f64_chunks(const double* __restrict__ C, const float* __restrict__ C32, const float* __restrict__ Cmin,
                         int nrows, int nin, int nchunk, const double* __restrict__ L64,
@@ -254,6 +254,7 @@ __global__ void __launch_bounds__(NW * 32)
                         Epilogue epi) {
   constexpr int NT = NW * 32, RPC = NW / WPR;
   static_assert(NW <= 32 && NT >= kExpUnits, "a table entry a thread, a warp's lanes cover the rows");
+  static_assert(32 * kShort <= kRowList, "a short row's columns fit its warp's list without draining it");
   extern __shared__ double pval[];  // the terms of the lists, row by row
   int* slist = reinterpret_cast<int*>(pval + NW * (kRowList + 32));  // [NW][kRowList + 32] columns
   float* sLc = reinterpret_cast<float*>(slist + NW * (kRowList + 32));  // largest inputs, relative to the line's
@@ -272,7 +273,7 @@ __global__ void __launch_bounds__(NW * 32)
   const float* cmin = Cmin + (int64_t)(i < nrows ? i : 0) * nchunk;
   // before the preceding kernel has ended: the table and the least costs of the first 128 chunks
   exp_table_load(tab);
-  constexpr int kOwn = kShort ? kShortChunks : 1;
+  constexpr int kOwn = kShort ? kShort : 1;
   float q4[4], cs[kOwn];
 #pragma unroll
   for (int u = 0; u < (kShort ? 0 : 4); ++u) {
@@ -457,15 +458,13 @@ __global__ void __launch_bounds__(NW * 32)
   const float lowest = -cut - mneg;
   // |t - t_FP64| and the error of m are below (k2 |c| + |l| + |t| + |d|) 2^-22 plus lerr
   // (and mneg): |m| <= |t| + |d|, and the two parts of an exponent have one sign
-  auto keeps = [&](float t, float mag) {
+  auto list = [&](bool in, float t, float mag, int j) {
     const float d = t - m;
     const float tol = fmaf(fabsf(t) + fabsf(d) + mag, 0x1p-22f, lerr);
-    const bool keep = !(d <= lowest - tol);
-    far = far || (keep && !(tol <= kRowFarTol));
-    return keep;
-  };
-  auto append = [&](bool keep, int j) {
+    const bool keep = in && !(d <= lowest - tol);
     const unsigned km = __ballot_sync(0xffffffffu, keep);
+    if (!km) return;  // warp-uniform, and the usual case at small eps
+    far = far || (keep && !(tol <= kRowFarTol));
     if (keep) lst[cnt + __popc(km & ((1u << lane) - 1u))] = j;
     cnt += __popc(km);
   };
@@ -473,7 +472,7 @@ __global__ void __launch_bounds__(NW * 32)
 #pragma unroll
     for (int u = 0; u < kOwn; ++u) {
       const int j = 32 * (part + WPR * u) + lane;
-      append(j < nin && keeps(ts[u], fmaf(k2f, fabsf(cs[u]), fabsf(shifted(ls[u])))), j);
+      list(j < nin, ts[u], fmaf(k2f, fabsf(cs[u]), fabsf(shifted(ls[u]))), j);
     }
   }
   if (!kShort && live && m != -INFINITY) {
@@ -495,7 +494,7 @@ __global__ void __launch_bounds__(NW * 32)
         exponents(cj, t, mag);
 #pragma unroll
         for (int u = 0; u < G; ++u) {
-          append(cj[u] < nin && keeps(t[u], mag[u]), cj[u]);
+          list(cj[u] < nin, t[u], mag[u], cj[u]);
           if (cnt > kRowList) {  // a full batch from the list's end: every lane evaluates one term
             __syncwarp();
             cnt -= 32;
@@ -948,23 +947,30 @@ cudaError_t launch_rows(int prec, const RowsGeom& g, int nrows, int nin, const d
         return launch_pdl(kern, dim3((nrows + rpc - 1) / rpc), dim3(nw * 32), smem, s, C, g.C32,
                           g.Cmin, nrows, nin, nchunk, l64, lff, lch, 1.0 / eps, 50.0f + logf((float)nin), epi);
       };
-      // Warps per row, so that few rows still fill the GPU (one warp a row left 1 x 300000
-      // at 2.3 times the time of the four-warp kernel before, 300 x 300 at 1.17).  Times of
-      // 20 iterations with 1, 2, 4 warps: 300 rows 1.19, 0.90, 0.80 ms; 400 rows (WF, eps
-      // 1e-3) 2.7, 2.2, 2.2; 1216 rows 3.5, 3.0, 2.6 at eps 1e-2 but 2.2, 2.3, 2.6 (WF, 1e-8);
-      // 3000 rows (WF, 1e-8) 3.2, 4.1, 5.0.  152 rows of 30000 columns: 4 warps 1.16 ms, 16 0.69.
+      // Warps per row, as many as keep the CTAs at one per SM, so that few rows still fill the
+      // GPU (one warp a row left 1 x 300000 at 2.3 times the time of the four-warp kernel before,
+      // 300 x 300 at 1.17).  Times of 20 iterations with 1, 2, 4 warps: 300 rows 1.19, 0.90,
+      // 0.80 ms; 450 rows (WF, eps 1e-3) 2.87, 2.19, 2.2; 784 rows (WF, 1e-8) 2.12, 2.25; 3000 rows
+      // (WF, 1e-8) 3.2, 4.1, 5.0.  152 rows of 30000 columns: 4 warps 1.16 ms, 16 0.69.
+      // Four to eight rows per SM that fit registers take CTAs of 32 warps, eight rows of four:
+      // 700 x 700 at eps 1 1.84 -> 1.70 ms, 1128 rows (WF, 1e-3) 4.43 -> 4.21, (1e-8) 2.15 both;
+      // eight SMs stay free for the kernels before and after, which such a CTA leaves no
+      // registers (1216 rows, one on every SM, WF at 1e-8: 2.36 against 2.25 ms).
       const int sms = sm_count();
       auto by_length = [&](auto shrt, auto lng, int nw, int wpr) {
         return nchunk <= kShortChunks * wpr ? run(shrt, nw, nw / wpr) : run(lng, nw, nw / wpr);
       };
       if (nrows <= sms && nchunk >= 128)
-        e = run(&rows_lse_f64_chunks<16, 16, false>, 16, 1);
+        e = run(&rows_lse_f64_chunks<16, 16, 0>, 16, 1);
       else if (nrows <= 2 * sms)
-        e = by_length(&rows_lse_f64_chunks<8, 4, true>, &rows_lse_f64_chunks<8, 4, false>, 8, 4);
-      else if (nrows <= 8 * sms)
-        e = by_length(&rows_lse_f64_chunks<8, 2, true>, &rows_lse_f64_chunks<8, 2, false>, 8, 2);
+        e = by_length(&rows_lse_f64_chunks<8, 4, kShortChunks>, &rows_lse_f64_chunks<8, 4, 0>, 8, 4);
+      else if (nrows <= 4 * sms)
+        e = by_length(&rows_lse_f64_chunks<8, 2, kShortChunks>, &rows_lse_f64_chunks<8, 2, 0>, 8, 2);
+      else if (nrows <= 8 * (sms - 8) && nchunk <= 4 * kShortWide)
+        e = nchunk <= 4 * kShortChunks ? run(&rows_lse_f64_chunks<32, 4, kShortChunks>, 32, 8)
+                                       : run(&rows_lse_f64_chunks<32, 4, kShortWide>, 32, 8);
       else
-        e = by_length(&rows_lse_f64_chunks<8, 1, true>, &rows_lse_f64_chunks<8, 1, false>, 8, 1);
+        e = by_length(&rows_lse_f64_chunks<8, 1, kShortChunks>, &rows_lse_f64_chunks<8, 1, 0>, 8, 1);
       if (e != cudaSuccess) return e;
       prof_mark_end(PROF_ROWS, s);
       return cudaGetLastError();
